@@ -122,7 +122,10 @@ typedef struct {
                                      solve when the box is periodic in y with a power-of-two
                                      ny <= 2048, bounded in x, and its free nodes form a full
                                      slab with at most one slot below it (the trench and the
-                                     plate geometries), else 1;
+                                     plate geometries); else, for such a slab and slot on up to
+                                     1024 columns of any count, periodic or between two walls, or
+                                     with x periodic, a solve by dense transforms along y; else
+                                     as 1;
                                      1: conjugate gradient preconditioned by a multigrid V-cycle */
   int64_t hit_capacity;           /* hit records kept (PIC_DIAG_HITS) */
   void *stream;                   /* cudaStream_t to run on; NULL: a library-owned stream */
@@ -200,9 +203,9 @@ enum {
   PIC_DIAG_STATE_I = 9,  /* same for ions */
   PIC_DIAG_POISSON = 10, /* [inner iterations, outer iterations, rel residual, ms] of the last solve,
                             and (with room for a fifth double) the rel residual at its first check:
-                            that of the initial guess with the multigrid inner solver, that after
-                            the first correction with the direct one (whose first pass always
-                            corrects) */
+                            that of the initial guess, except with the FFT solve, whose first pass
+                            corrects unchecked: there that after the first correction.  With the
+                            FFT and the dense-transform solve an inner iteration is one pass */
   PIC_DIAG_STATUS = 11,  /* uint32: status word; reading clears it */
   PIC_DIAG_TIMING = 12,  /* [steps, ms particle kernel, ms sort, ms Poisson (the solve's
                             residual passes also form E), ms rho,
@@ -211,8 +214,9 @@ enum {
                             pic_step calls since the last read; reading resets it */
   PIC_DIAG_PHI_VACUUM = 13, /* [nxn*nyn]: potential of the empty box (Dirichlet values only),
                                solved once to 1e-10 */
-  PIC_DIAG_SOLVER = 14,     /* int32: inner Poisson solver in use, 0 direct, 1 multigrid PCG
-                               (pic_config.poisson_method) */
+  PIC_DIAG_SOLVER = 14,     /* int32: inner Poisson solver in use, 0 the direct FFT solve, 1 one
+                               of the others (dense transforms where poisson_method 0 allows
+                               them, multigrid PCG elsewhere and with poisson_method 1) */
   PIC_DIAG_SORT = 15,       /* int32[2]: steps between tile sorts in use (0 while it is being
                                tuned), and 1 if it was chosen by the tuning of sort_every = 0 */
   PIC_DIAG_TILE = 16        /* int32[5]: tile variant in use, its tile cells along x and y,

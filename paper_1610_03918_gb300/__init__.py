@@ -49,7 +49,7 @@ FREE_FN = ctypes.CFUNCTYPE(None, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void
 
 
 # pic_config.poisson_method
-POISSON_AUTO = 0        # direct FFT / tridiagonal / capacitance solve where the geometry allows
+POISSON_AUTO = 0        # direct solve (FFT or dense transforms, tridiagonal, capacitance) where the box allows
 POISSON_MULTIGRID = 1   # multigrid-preconditioned conjugate gradient everywhere
 
 
@@ -545,8 +545,9 @@ class Sim:
         return tuple(int(v) for v in self.diag(PIC_DIAG_TILE, np.zeros(5, np.int32))[0])
 
     def solver(self):
-        """Inner Poisson solver in use: POISSON_AUTO (0) = the direct one,
-        POISSON_MULTIGRID (1) = multigrid-preconditioned CG."""
+        """Inner Poisson solver in use: POISSON_AUTO (0) = the direct FFT one,
+        POISSON_MULTIGRID (1) = another: dense transforms where poisson_method
+        is POISSON_AUTO and the box allows them, else multigrid-preconditioned CG."""
         return int(self.diag(PIC_DIAG_SOLVER, np.zeros(1, np.int32))[0][0])
 
     def status(self):

@@ -227,6 +227,31 @@ struct FastPoisson {
   int kernels = 0;                 // launches per inner solve
 };
 
+// Transform solve of the boxes the direct solve above does not take
+// (boxpoisson.cu): a block of rows x columns diagonalised along y by a dense
+// orthonormal basis, one tridiagonal system along x per mode.
+struct BoxBlock {
+  int m = 0, n = 0;                // rows, columns (= modes)
+  int row0 = 0, col0 = 0;          // grid row and column of the first
+  int mp = 0, ldv = 0;             // padded row counts of the [n][mp] and [n][ldv] tables
+  const float *v = nullptr;        // [n][ldv] basis V[j][k]
+  const float *vt = nullptr;       // [n][n] its transpose
+  const float *w = nullptr;        // [n][mp] Thomas factors of mode k's system
+  const float *z = nullptr;        // [n][mp] response to a unit value on the row next to the
+                                   // interface (of a ring: to its held row 0), or null
+  const float *ring = nullptr;     // [n] x periodic: reciprocal pivot of the held row
+  float *c = nullptr;              // [n][mp] solved spectra
+};
+struct BoxPoisson {
+  int enabled = 0;
+  int slot = 0, xs = 0;            // interface and slot present; the interface's row
+  BoxBlock b[2];                   // slab, slot
+  const float *sinv = nullptr;     // [wc][wc] inverse of the interface's Schur complement
+  float *fh = nullptr, *sh = nullptr;   // spectra of the interface values
+  int bm = 8;                      // rows per CTA of the inverse transform
+  size_t solve_smem = 0, add_smem = 0;
+};
+
 // Programmatic dependent launch.  The solver's kernels wait for the grid
 // before them (its results are then visible) and at once let the next kernel
 // of the stream be scheduled, so that kernel's blocks are resident and waiting
@@ -313,6 +338,7 @@ struct pic_ctx {
   picgb::Reducer red;
   int singular;
   picgb::FastPoisson fp;       // direct inner solve (enabled when the geometry allows it)
+  picgb::BoxPoisson box;       // transform inner solve (enabled where fp is not and the box allows it)
   double last_ms;
   int last_outer;
   cudaEvent_t ev0, ev1;
@@ -414,8 +440,14 @@ cudaError_t poisson_setup(pic_ctx *c);
 // residual r into the correction e.
 cudaError_t fast_poisson_setup(pic_ctx *c);
 void fast_poisson_launch(pic_ctx *c, const float *r, float2 *pot, PoissonState *ps);
+// Transform inner solve (boxpoisson.cu), likewise: two kernels per pass.
+cudaError_t box_poisson_setup(pic_ctx *c);
+void box_poisson_launch(pic_ctx *c, const float *r, float2 *pot, PoissonState *ps);
+// one of the two is in use: each refinement pass is one of its solves, which
+// adds the correction to the potential itself
+inline bool one_pass_solver(const pic_ctx *c) { return c->fp.enabled || c->box.enabled; }
 cudaError_t launch_rho(pic_ctx *c, int advance_step, int init_solve = 0);
-// In a captured step with the direct solve and the previous potential as the
+// In a captured step with one of those solves and the previous potential as the
 // guess, the solve's first residual pass forms rho itself (no density kernel).
 bool rho_in_solve(const pic_ctx *c);
 pic_status poisson_solve(pic_ctx *c, bool zero_guess);

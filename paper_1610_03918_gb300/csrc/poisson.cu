@@ -321,7 +321,7 @@ struct FineArgs {
   double *fe;
   uint32_t *status;
   int graph;                 // kernels run inside the step graph: drive its conditionals
-  int direct;                // the inner solve is the direct one (no inner loop)
+  int direct;                // the inner solve is the direct or the transform one (no inner loop)
   cudaGraphConditionalHandle h_outer, h_if_outer, h_inner, h_if_inner;
 };
 
@@ -501,10 +501,14 @@ __device__ __forceinline__ float resid_node(float2 rho, const float2 (&ph)[5]) {
 // it checks and its energy, so the pass that accepts the potential leaves
 // the step's field, and decides whether the solve goes on.  A first pass
 // known not to be the last (the direct solve's, which always corrects once)
-// skips all that and leaves only its ||b||^2 block sums for the next pass.
-template <bool CHECK, bool SING, bool FROM_ACC = false>
+// skips all that and leaves only its ||b||^2 block sums for the next pass; the
+// transform solve's first pass (kOpen) forms the guess's norms, but no field
+// and no decision, since a correction follows it in any case.
+enum { kFirst = 0, kFull = 1, kOpen = 2 };
+template <int MODE, bool SING, bool FROM_ACC = false>
 __global__ void k_resid(FineArgs a) {
-  static_assert(!FROM_ACC || (!CHECK && !SING), "rho is formed only by a first pass without a check");
+  static_assert(!FROM_ACC || (MODE != kFull && !SING), "rho is formed only by a first pass");
+  constexpr bool CHECK = MODE != kFirst, FIELD = MODE == kFull;
   pdl_enter();
   const Geom g = a.g;
   const int nn = g.nxn * g.nyn;
@@ -556,7 +560,7 @@ __global__ void k_resid(FineArgs a) {
         if (bb_here) sq_add(q3[1], rho.x + (rho.y + lf[k]));
       }
       a.r32[n] = r32;
-      if (CHECK) {
+      if (FIELD) {
         const float2 E = node_field(fl[k], ph[k]);
         a.E[n] = E;
         sq_add(q3[2], E.x);
@@ -578,17 +582,23 @@ __global__ void k_resid(FineArgs a) {
     }
     return;
   }
-  float c[9] = {q3[0].mid, q3[0].big, q3[0].tiny, q3[1].mid, q3[1].big, q3[1].tiny,
-                q3[2].mid, q3[2].big, q3[2].tiny};
-  if (!publish_sums<9>(c, a.partf, a.ticket)) return;
-  sum_published<9>(a.partf, gridDim.x, c);
+  constexpr int NC = FIELD ? 9 : 6;
+  float c[NC];
+#pragma unroll
+  for (int k = 0; k < NC; k += 3) {
+    c[k] = q3[k / 3].mid;
+    c[k + 1] = q3[k / 3].big;
+    c[k + 2] = q3[k / 3].tiny;
+  }
+  if (!publish_sums<NC>(c, a.partf, a.ticket)) return;
+  sum_published<NC>(a.partf, gridDim.x, c);
   PoissonState *ps = a.ps;
   const bool bb_parts = a.bb_from_part && ps->outer_iters == 1;
   float cb[3] = {0.f, 0.f, 0.f};
   if (bb_parts) sum_published<3>(a.bbpart, gridDim.x, cb);
   if (threadIdx.x == 0) {
     const double rr = sq_join(c);
-    a.fe[0] = 0.5 * sq_join(c + 6);
+    if (FIELD) a.fe[0] = 0.5 * sq_join(c + NC - 3);
     ps->rr64 = rr;
     if (first) ps->bb = sq_join(c + 3);
     if (bb_parts) ps->bb = sq_join(cb);
@@ -599,6 +609,10 @@ __global__ void k_resid(FineArgs a) {
     else
       ps->rel = sqrt_ratio(rr, bb > 0 ? bb : 1.0);
     if (first || bb_parts) ps->rel_first = ps->rel;
+    if (MODE == kOpen) {   // a correction follows in any case
+      *a.ticket = 0u;
+      return;
+    }
     const bool ok = ps->rel <= a.rtol || rr == 0.0;
     const bool give_up = !ok && ps->outer_iters >= kMaxOuter;
     if (give_up) atomicOr(a.status, PIC_ST_NOCONV);
@@ -1474,9 +1488,15 @@ __global__ void __launch_bounds__(kCoarseThreads) k_coarse(MGArgs a) {
 
 // --------------------------------------------------------------------------
 // the residual kernel for the box: with or without the mean of rho removed
-template <bool CHECK>
+template <int MODE>
 void (*resid_kernel(const pic_ctx *c))(FineArgs) {
-  return c->singular ? k_resid<CHECK, true> : k_resid<CHECK, false>;
+  return c->singular ? k_resid<MODE, true> : k_resid<MODE, false>;
+}
+
+// one solve of A e = r by the direct or the transform solver, added to the potential
+void launch_one_pass(pic_ctx *c) {
+  if (c->fp.enabled) fast_poisson_launch(c, c->d_r32, c->d_phi, c->d_ps);
+  else box_poisson_launch(c, c->d_r32, c->d_phi, c->d_ps);
 }
 
 FineArgs fine_args(pic_ctx *c) {
@@ -1520,7 +1540,7 @@ FineArgs fine_args(pic_ctx *c) {
   a.fe = c->d_fe;
   a.status = c->d_status;
   a.graph = 0;
-  a.direct = c->fp.enabled;
+  a.direct = one_pass_solver(c) ? 1 : 0;
   a.h_outer = a.h_if_outer = a.h_inner = a.h_if_inner = 0;
   return a;
 }
@@ -1870,12 +1890,13 @@ cudaError_t poisson_setup(pic_ctx *c) {
   cudaEventCreate(&c->ev0);
   cudaEventCreate(&c->ev1);
   e = fast_poisson_setup(c);
+  if (e == cudaSuccess) e = box_poisson_setup(c);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
 
 bool rho_in_solve(const pic_ctx *c) {
-  return c->fp.enabled && c->cfg.warm_start == 1 && !c->singular;
+  return one_pass_solver(c) && c->cfg.warm_start == 1 && !c->singular;
 }
 
 cudaError_t launch_rho(pic_ctx *c, int advance_step, int init_solve) {
@@ -1975,13 +1996,13 @@ pic_status poisson_solve(pic_ctx *c, bool zero_guess) {
   c->launches += 1;
   const int batch = 4;
   for (;;) {
-    launch(resid_kernel<true>(c), nb, kThreads, 0, c->stream, a);
+    launch(resid_kernel<kFull>(c), nb, kThreads, 0, c->stream, a);
     c->launches += 1;
     cudaMemcpyAsync(c->h_ps, c->d_ps, sizeof(PoissonState), cudaMemcpyDeviceToHost, c->stream);
     if (cudaStreamSynchronize(c->stream) != cudaSuccess) return PIC_ECUDA;
     if (!c->h_ps->go) break;
-    if (c->fp.enabled) {   // the direct solve adds its correction to phi itself
-      fast_poisson_launch(c, c->d_r32, c->d_phi, c->d_ps);
+    if (one_pass_solver(c)) {   // adds its correction to phi itself
+      launch_one_pass(c);
       continue;
     }
     launch_vcycle(c, m);
@@ -2058,7 +2079,7 @@ cudaError_t add_cond(cudaGraph_t g, const std::vector<cudaGraphNode_t> &deps,
 //   [phi reset] -> init -> WHILE(outer) { resid -> IF(go) { V-cycle ->
 //     WHILE(inner) { cg -> IF(!done) { V-cycle } } -> correct } }
 // where a V-cycle also forms w = A z and the inner products of the next step.
-// With the direct inner solve, whose one pass nearly always suffices, the
+// With the direct or the transform solve, whose one pass nearly always suffices, the
 // first pass runs unconditionally (a potential that already meets the
 // tolerance takes one correction it does not need) and only further passes
 // are conditional (the direct solve adds its correction to phi itself):
@@ -2068,7 +2089,7 @@ cudaError_t poisson_capture(pic_ctx *c, cudaGraph_t top, std::vector<cudaGraphNo
   FineArgs a = fine_args(c);
   const MGArgs m = mg_args(c);
   const int nb = c->red.nblocks;
-  const bool direct = c->fp.enabled;
+  const bool direct = one_pass_solver(c);
   cudaGraphConditionalHandle h[4];
   const int nh = direct ? 1 : 4;
   for (int k = 0; k < nh; ++k) {
@@ -2093,18 +2114,20 @@ cudaError_t poisson_capture(pic_ctx *c, cudaGraph_t top, std::vector<cudaGraphNo
   // before opened the solve)
   if (c->cfg.warm_start != 1) launch(k_outer_init, 1, 1, 0, s, c->d_ps);
   if (direct) {
-    // the first pass always corrects: it leaves ||b||^2 to the second
+    // the first pass always corrects: the direct solve's leaves ||b||^2 to the
+    // second, the transform solve's forms the norms of the guess
+    const bool fp = c->fp.enabled != 0;
     if (rho_in_solve(c)) {   // and forms rho, opening the step's solve
       FineArgs r = a;
       r.advance_step = 1;
       r.init_solve = 1;
-      launch(k_resid<false, false, true>, nb, kThreads, 0, s, r);
+      launch(fp ? k_resid<kFirst, false, true> : k_resid<kOpen, false, true>, nb, kThreads, 0, s, r);
     } else {
-      launch(resid_kernel<false>(c), nb, kThreads, 0, s, a);
+      launch(fp ? resid_kernel<kFirst>(c) : resid_kernel<kOpen>(c), nb, kThreads, 0, s, a);
     }
-    fast_poisson_launch(c, c->d_r32, c->d_phi, c->d_ps);
-    a.bb_from_part = 1;
-    launch(resid_kernel<true>(c), nb, kThreads, 0, s, a);
+    launch_one_pass(c);
+    a.bb_from_part = fp ? 1 : 0;
+    launch(resid_kernel<kFull>(c), nb, kThreads, 0, s, a);
   }
   CK(cap_end(s, deps));
   cudaGraphNode_t n_outer, n_if_outer, n_inner, n_if_inner;
@@ -2113,14 +2136,14 @@ cudaError_t poisson_capture(pic_ctx *c, cudaGraph_t top, std::vector<cudaGraphNo
   std::vector<cudaGraphNode_t> d;
   if (direct) {
     CK(cap_begin(s, b_outer, {}));
-    fast_poisson_launch(c, c->d_r32, c->d_phi, c->d_ps);
-    launch(resid_kernel<true>(c), nb, kThreads, 0, s, a);
+    launch_one_pass(c);
+    launch(resid_kernel<kFull>(c), nb, kThreads, 0, s, a);
     CK(cap_end(s, d));
     deps.assign(1, n_outer);
     return cudaGetLastError();
   }
   CK(cap_begin(s, b_outer, {}));
-  launch(resid_kernel<true>(c), nb, kThreads, 0, s, a);
+  launch(resid_kernel<kFull>(c), nb, kThreads, 0, s, a);
   CK(cap_end(s, d));
   CK(add_cond(b_outer, d, h[1], cudaGraphCondTypeIf, &n_if_outer, &b_if_outer));
   CK(cap_begin(s, b_if_outer, {}));
@@ -2151,8 +2174,8 @@ int64_t poisson_kernel_count(pic_ctx *c, int64_t S, int64_t O, int64_t I) {
   // final resid, and unless the density kernel opens the solve: guess and init
   int64_t per_solve = 1 + (c->cfg.warm_start != 1 ? 2 : 0);
   if (c->cfg.warm_start == 3) per_solve += 2 + unet_forward_kernels();   // absmax, input, network
-  if (c->fp.enabled)   // per pass: resid, direct solve (which corrects phi)
-    return S * per_solve + O * (c->fp.kernels + 1);
+  if (one_pass_solver(c))   // per pass: resid, solve (which corrects phi)
+    return S * per_solve + O * ((c->fp.enabled ? c->fp.kernels : 2) + 1);
   // a V-cycle with w = A z and the inner products: fused into its last kernel unless lc = 0
   const int64_t vc = 2 * c->lc + 1 + (c->lc == 0 ? 1 : 0);
   // per pass: resid, V-cycle, correct; per iteration: cg; per non-final iteration: V-cycle
