@@ -551,6 +551,7 @@ pic_status pic_batch_init(const pic_config *cfgs, int32_t n, void *stream, pic_b
       pic_batch_free(b);
       return st;
     }
+    c->sharing = n;
     b->m.push_back(c);
   }
   *out = b;
@@ -745,11 +746,14 @@ pic_status pic_init(const pic_config *cfg, pic_ctx **out) {
   c->d_tile_cursor = (uint32_t *)A(2 * size_t(ntiles) * 4);
   c->d_tile_start = (uint32_t *)A(2 * size_t(ntiles) * 4);
   c->max_chunks = 0;
+  // chunks of kChunk, or of a share of the resident CTAs on small grids, and a remainder per tile
   for (int s = 0; s < 2; ++s) c->max_chunks += ntiles + c->cap[s] / kChunk + 1;
+  c->max_chunks += int64_t(c->num_sms) * kMaxCtasPerSm + ntiles / 8 + 64;
   c->d_chunks = (Chunk *)A(size_t(c->max_chunks) * sizeof(Chunk));
   c->d_nchunks = (int32_t *)A(4);
   c->d_nslots = (int64_t *)A(4 * 8);
   c->d_ke_part = (double *)A(size_t(c->max_chunks) * 8);
+  c->d_work = (unsigned int *)A(2 * sizeof(unsigned int));
   c->d_step = (int32_t *)A(4);
   c->d_walls = (unsigned long long *)A(2 * PIC_NWALLS * 8);
   c->d_bottom = (unsigned long long *)A(2 * size_t(g.ny) * 8);
@@ -843,6 +847,7 @@ pic_status pic_init(const pic_config *cfg, pic_ctx **out) {
   cudaMemsetAsync(c->d_tile_count, 0, 2 * size_t(ntiles) * 4, c->stream);
   cudaMemsetAsync(c->d_tile_cursor, 0, 2 * size_t(ntiles) * 4, c->stream);
   cudaMemsetAsync(c->d_nchunks, 0, 4, c->stream);
+  cudaMemsetAsync(c->d_work, 0, 2 * sizeof(unsigned int), c->stream);
   cudaMemsetAsync(c->d_nslots, 0, 32, c->stream);
   cudaMemsetAsync(c->d_step, 0, 4, c->stream);
   cudaMemsetAsync(c->d_walls, 0, 2 * PIC_NWALLS * 8, c->stream);

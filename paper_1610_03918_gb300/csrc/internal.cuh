@@ -36,6 +36,8 @@ constexpr TileVariant kTileVariants[kNumTileVariants] = {
 };
 constexpr int kMinTileLog2 = 4;  // the smallest tile (16 x 16) sizes the tile arrays
 constexpr int kChunk = 4092;     // particles per work item (multiple of 4, <= 4095)
+constexpr int kMinChunk = 512;   // one pass of the particle kernel's smaller CTA
+constexpr int kMaxCtasPerSm = 16;
 constexpr int kWalkLimit = 16;   // face crossings followed per move
 
 // Double-float values.  The potential, the charge density and the Dirichlet
@@ -366,10 +368,12 @@ struct pic_ctx {
   int32_t *d_nchunks;
   int64_t max_chunks;
   int tile_variant;            // index into kTileVariants
+  int sharing;                 // contexts that step on the GPU together (members of an ensemble)
   int suppress_sort;           // autotuning: no scheduled sorts while a variant is timed
   int max_tiles;               // tiles of the smallest tile shape (array sizes)
   int64_t *d_nslots;           // [4]: slots in use per species; [2..3] staged by the sort
   double *d_ke_part;           // [max_chunks]
+  unsigned int *d_work;        // [2] the particle kernel's chunk dispenser
   int32_t *d_step;
 
   // tallies and status

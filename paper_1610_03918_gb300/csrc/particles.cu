@@ -9,6 +9,8 @@
 // four particles with 16-byte vector loads and stores.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "internal.cuh"
 #include "philox.cuh"
 
@@ -19,6 +21,9 @@ __device__ __forceinline__ int wrapmod(int a, int n) {
   a %= n;
   return a < 0 ? a + n : a;
 }
+
+// a wrapped into [0, n) for a in [-n, 2n): no integer division
+__device__ __forceinline__ int wrap_once(int a, int n) { return a < 0 ? a + n : (a >= n ? a - n : a); }
 
 __device__ __forceinline__ int cell_i(int c) { return c >> 16; }
 __device__ __forceinline__ int cell_j(int c) { return c & 0xffff; }
@@ -43,6 +48,7 @@ struct SortArgs {
   int64_t *nslots_out;
   Geom g;
   int ntiles;
+  int ctas;                // CTAs of the particle kernel resident at once
 };
 
 // The counting passes take 4 consecutive slots per lane (16-byte loads, 128
@@ -123,10 +129,22 @@ __device__ uint32_t block_exscan(uint32_t v, uint32_t *total) {
 // list is written with consecutive threads on consecutive chunks: each thread
 // finds the tile of its chunk by a binary search over the tiles' first chunk
 // indices, kept in shared memory.
+//
+// A tile's particles are split into equal chunks of at most `most` particles:
+// an even part of a resident CTA's share of all particles, at most kChunk and
+// at least one pass of a CTA (kMinChunk).  With chunks of kChunk the 80 x 30
+// run's 420k particles made 103 chunks, which left a third of the SMs idle and
+// the others with four warps each (particle phase 31.9 us, now 14.9 us), and
+// 13M particles in 16 x 16 tiles 2.6 chunks a CTA, which run as long as 3.
+// Equal parts, because a remainder costs a whole window: 4096 particles a tile
+// (16 per cell) made a chunk of 4092 and one of 4 (512 x 512: 80.3 -> 71.7 us).
 __global__ void __launch_bounds__(1024) k_sort_scan(SortArgs a) {
   __shared__ uint32_t s_first[1025];   // first chunk of each tile of the round, then the round's total
   __shared__ uint32_t s_off[1024], s_padded[1024];
   uint32_t chunk_base = 0;
+  const int64_t share = (a.nslots[0] + a.nslots[1] + a.ctas - 1) / a.ctas;
+  const int64_t rounds = max(int64_t(1), (share + kChunk - 1) / kChunk), part = (share + rounds - 1) / rounds;
+  const uint32_t most = uint32_t(min(int64_t(kChunk), max(int64_t(kMinChunk), (part + kMinChunk - 1) / kMinChunk * kMinChunk)));
   for (int s = 0; s < 2; ++s) {
     uint32_t slot_base = 0;
     uint32_t *cnt = a.count + int64_t(s) * a.ntiles;
@@ -139,7 +157,7 @@ __global__ void __launch_bounds__(1024) k_sort_scan(SortArgs a) {
       if (t < a.ntiles) {
         n = cnt[t];
         padded = (n + 3u) & ~3u;
-        nch = (padded + kChunk - 1) / kChunk;
+        nch = (padded + most - 1) / most;
       }
       uint32_t tot_slots, tot_ch;
       const uint32_t off = block_exscan(padded, &tot_slots) + slot_base;
@@ -162,9 +180,10 @@ __global__ void __launch_bounds__(1024) k_sort_scan(SortArgs a) {
           const int mid = (lo + hi) >> 1;
           if (s_first[mid] <= c) lo = mid; else hi = mid;
         }
-        const uint32_t q = c - s_first[lo];
-        const uint32_t b0 = s_off[lo] + q * kChunk;
-        const uint32_t b1 = s_off[lo] + min(s_padded[lo], (q + 1) * kChunk);
+        const uint32_t q = c - s_first[lo], pad = s_padded[lo];
+        const uint32_t parts = (pad + most - 1) / most, per = ((pad + parts - 1) / parts + 3u) & ~3u;
+        const uint32_t b0 = s_off[lo] + min(pad, q * per);
+        const uint32_t b1 = s_off[lo] + min(pad, (q + 1) * per);
         reinterpret_cast<int4 *>(a.chunks)[chunk_base + c] = make_int4(s, t0 + lo, int(b0), int(b1));
       }
       __syncthreads();
@@ -253,6 +272,7 @@ struct PArgs {
   uint32_t *status;
   const int32_t *step;
   double *ke_part;
+  unsigned int *work;        // [2]: chunks handed out beyond the first of each CTA, CTAs done
   double *fe;                // [0] energy of the current E, [1] of the E used by the last step
   // ion recycling: absorbed ions re-enter in cell rows [src_x0, src_x0 + src_rows)
   int recycle;
@@ -477,11 +497,16 @@ __device__ __forceinline__ void move_one(const PArgs &a, const float2 *sE, uint3
   const int cx = int(cxf), cy = int(cyf);
   int oi = 0, oj = 0;     // cell offset of the move
   if (cx | cy) {
+    int ni, nj;           // the end cell
     const bool near = (unsigned)(cx + 1) <= 2u && (unsigned)(cy + 1) <= 2u;
     if (near && (__ldg(&a.cellmask[i * g.ny + j]) & kCellInterior)) {
       // all eight neighbours are plasma: no face within one cell can absorb
       oi = cx;
       oj = cy;
+      ni = i + oi;
+      nj = j + oj;
+      if (g.px) ni = wrap_once(ni, g.nx);
+      if (g.py) nj = wrap_once(nj, g.ny);
     } else if (const int gone = walk_move(a, s, i, j, fx, fy, dx, dy, cx, cy, vx1, vy1, id, slot, oi, oj)) {
       if (gone == 1 && s == 1 && a.recycle) {
         // tallied above; a thermal ion takes its place and joins the deposit
@@ -493,14 +518,16 @@ __device__ __forceinline__ void move_one(const PArgs &a, const float2 *sE, uint3
       }
       c = -1;   // absorbed and tallied, or moved beyond the walk limit
       return;
+    } else {
+      ni = i + oi;
+      nj = j + oj;
+      if (g.px) ni = wrapmod(ni, g.nx);
+      if (g.py) nj = wrapmod(nj, g.ny);
     }
     nfx = __fsub_rn(nfx, cxf);
     nfy = __fsub_rn(nfy, cyf);
     nfx = fminf(nfx, 0x1.fffffep-1f);
     nfy = fminf(nfy, 0x1.fffffep-1f);
-    int ni = i + oi, nj = j + oj;
-    if (g.px) ni = wrapmod(ni, g.nx);
-    if (g.py) nj = wrapmod(nj, g.ny);
     c = pack_cell(ni, nj);
   }
   fx = nfx;
@@ -525,8 +552,15 @@ __device__ __forceinline__ void prefetch_l2(const void *p, unsigned bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 
+// 84.5M particles, 16 x 16 tiles: 641 us with statically strided chunks and
+// integer divisions in every cell change and window node, 605 us without
+// either at 64 registers (8 CTAs per SM), 589 us held to 56 (9 CTAs; 48
+// registers and 10 CTAs: 677 us): 5.74 TB/s of algorithmic traffic, 0.85 of a
+// copy's.  Sparing the particles of all-interior windows the cell mask's look
+// (+3%), the next chunk's first state prefetched across the chunk boundary
+// (+1.6%), loads past L1 (+11%) and plain stores (+0.4%) did not pay.
 template <int MODE, int V>
-__global__ void __launch_bounds__(Win<V>::THREADS, 1024 / Win<V>::THREADS) k_particles(PArgs a) {
+__global__ void __launch_bounds__(Win<V>::THREADS, Win<V>::THREADS == 128 ? 9 : 4) k_particles(PArgs a) {
   constexpr int NWX = Win<V>::NWX, NWY = Win<V>::NWY, THREADS = Win<V>::THREADS;
   __shared__ float2 sE[NWX * NWY];
   __shared__ uint32_t sAcc[NWX * NWY];
@@ -535,7 +569,16 @@ __global__ void __launch_bounds__(Win<V>::THREADS, 1024 / Win<V>::THREADS) k_par
   const int nch = *a.nchunks;
   const int nnodes = g.nxn * g.nyn;
   if (MODE == 0 && blockIdx.x == 0 && threadIdx.x == 0) a.fe[1] = a.fe[0];
-  for (int ci = blockIdx.x; ci < nch; ci += gridDim.x) {
+  // window nodes wrap at most once around a periodic box at least a tile and a halo wide
+  const bool once_x = g.nxn >= Win<V>::TX + Win<V>::H, once_y = g.nyn >= Win<V>::TY + Win<V>::H;
+  auto wrap_node = [&](int &gi, int &gj) {
+    if (g.px) gi = once_x ? wrap_once(gi, g.nxn) : wrapmod(gi, g.nxn);
+    if (g.py) gj = once_y ? wrap_once(gj, g.nyn) : wrapmod(gj, g.nyn);
+  };
+  // a CTA's first chunk is its index, the next ones are handed out as CTAs
+  // come free, so that the last wave ends together
+  __shared__ int s_next;
+  for (int ci = blockIdx.x; ci < nch; ci = s_next) {
     const Chunk ch = a.chunks[ci];
     const int s = ch.species;
     const int ti = ch.tile / g.nty;
@@ -546,8 +589,7 @@ __global__ void __launch_bounds__(Win<V>::THREADS, 1024 / Win<V>::THREADS) k_par
       if (MODE != 1) {
         const int wi = k / NWY, wj = k - (k / NWY) * NWY;
         int gi = wi0 + wi, gj = wj0 + wj;
-        if (g.px) gi = wrapmod(gi, g.nxn);
-        if (g.py) gj = wrapmod(gj, g.nyn);
+        wrap_node(gi, gj);
         float2 e = make_float2(0.f, 0.f);
         if (gi >= 0 && gi < g.nxn && gj >= 0 && gj < g.nyn) e = a.E[gi * g.nyn + gj];
         sE[k] = e;
@@ -555,6 +597,7 @@ __global__ void __launch_bounds__(Win<V>::THREADS, 1024 / Win<V>::THREADS) k_par
       sAcc[k] = 0u;
     }
     __syncthreads();
+    if (threadIdx.x == 0) s_next = int(gridDim.x + atomicAdd(&a.work[0], 1u));   // read after the chunk's last barrier
     unsigned long long *acc = a.acc + (int64_t)s * nnodes;
     const ParticleBuf P = a.pbufs[2 * s + a.cur[s]];
     float ke = 0.f;
@@ -603,8 +646,7 @@ __global__ void __launch_bounds__(Win<V>::THREADS, 1024 / Win<V>::THREADS) k_par
         if (v) {
           const int wi = k / NWY, wj = k - (k / NWY) * NWY;
           int gi = wi0 + wi, gj = wj0 + wj;
-          if (g.px) gi = wrapmod(gi, g.nxn);
-          if (g.py) gj = wrapmod(gj, g.nyn);
+          wrap_node(gi, gj);
           // The node's sum over the chunk lies in [-kChunk, kChunk * 2^20]: each of
           // at most kChunk particles adds a share in [-1, 2^20].  That range is
           // narrower than 2^32, so the 32-bit sum decodes uniquely; values above
@@ -628,6 +670,10 @@ __global__ void __launch_bounds__(Win<V>::THREADS, 1024 / Win<V>::THREADS) k_par
       }
     }
     __syncthreads();
+  }
+  if (threadIdx.x == 0 && atomicAdd(&a.work[1], 1u) == gridDim.x - 1) {   // no CTA asks any more
+    a.work[0] = 0u;
+    a.work[1] = 0u;
   }
 }
 
@@ -767,12 +813,17 @@ __global__ void k_moments(ParticleBuf P, const int64_t *nslots_p, double *part) 
   }
 }
 
-template <int MODE, int V>
-cudaError_t launch_particles_v(pic_ctx *c, const PArgs &a) {
+// CTAs of the step kernel that are resident at once
+template <int V>
+int resident_ctas(const pic_ctx *c) {
   int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_particles<0, V>, Win<V>::THREADS, 0);
-  if (per_sm < 1) per_sm = 1;
-  k_particles<MODE, V><<<c->num_sms * per_sm, Win<V>::THREADS, 0, c->stream>>>(a);
+  return c->num_sms * std::min(std::max(per_sm, 1), kMaxCtasPerSm);
+}
+
+template <int MODE, int V>
+cudaError_t launch_particles_v(pic_ctx *c, const PArgs &a) {
+  k_particles<MODE, V><<<resident_ctas<V>(c), Win<V>::THREADS, 0, c->stream>>>(a);
   return cudaGetLastError();
 }
 
@@ -801,6 +852,13 @@ cudaError_t launch_sort(pic_ctx *c) {
   a.nslots_out = c->d_nslots + 2;
   a.g = c->g;
   a.ntiles = c->g.ntx * c->g.nty;
+  switch (c->tile_variant) {
+    case 1: a.ctas = resident_ctas<1>(c); break;
+    case 2: a.ctas = resident_ctas<2>(c); break;
+    case 3: a.ctas = resident_ctas<3>(c); break;
+    default: a.ctas = resident_ctas<0>(c); break;
+  }
+  a.ctas = std::max(1, a.ctas / std::max(1, c->sharing));   // an ensemble's members share the GPU
   const dim3 grid(c->num_sms * 8, 2);   // 8 CTAs of 256 threads per SM and species
   if (a.ntiles <= kHistSmemTiles)
     k_sort_hist<true><<<grid, 256, size_t(a.ntiles) * 4, c->stream>>>(a);
@@ -836,6 +894,7 @@ cudaError_t launch_particles(pic_ctx *c, int mode, float kick_factor, const int 
   a.status = c->d_status;
   a.step = c->d_step;
   a.ke_part = c->d_ke_part;
+  a.work = c->d_work;
   a.fe = c->d_fe;
   a.recycle = c->cfg.recycle ? 1 : 0;
   a.src_x0 = c->src_x0;
