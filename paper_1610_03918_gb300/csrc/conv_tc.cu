@@ -31,6 +31,7 @@
 #include <cuda_runtime.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "internal.cuh"
@@ -129,6 +130,40 @@ __device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t da, uint64_t 
       "l"(da), "l"(db), "r"(idesc), "r"(accumulate)
       : "memory");
 }
+// the same from the low words of the descriptors; their high words (stride,
+// version, swizzle) are one constant
+__device__ __forceinline__ void mma_bf16_lo(uint32_t tmem_d, uint32_t da, uint32_t db, uint32_t hi, uint32_t idesc,
+                                            uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\t"
+      "setp.ne.b32 p, %5, 0;\n\t"
+      "mov.b64 a, {%1, %3};\n\t"
+      "mov.b64 b, {%2, %3};\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, p;\n\t}" ::"r"(tmem_d),
+      "r"(da), "r"(db), "r"(hi), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+// One lane of a converged warp.  The MMA warps run their loops with all lanes
+// and issue from one: control flow and descriptors then stay warp-uniform, in
+// uniform registers, where a lone thread's code spent 25 instructions -- about
+// 100 cycles -- on moving each MMA's descriptors there (N = 64: 48 cycles of
+// tensor core).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred q;\n\t"
+      "elect.sync _|q, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(p));
+  return p != 0;
+}
+// mbar_wait for a whole warp: the answer is warp-uniform
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity)) != 0;
+}
+// this thread's warp index, known to the compiler as warp-uniform
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0); }
+
 // arrives on the mbarrier once every MMA this thread issued before has completed
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
@@ -360,6 +395,319 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_before();
   __syncthreads();
   if (warp == 0) tmem_dealloc(tmem, L::NCOLS);
+}
+
+// ---------------------------------------------------------------- wide images
+// The 3x3 convolution on images at least 128 pixels wide, persistent and by
+// input rows.  A CTA keeps the weights of its N output channels in shared
+// memory and takes a run of output rows of one 128-pixel column block after
+// another; every input row of the run (130 pixels: the row's and a neighbour
+// on either side) is loaded once, KB channels a unit, and multiplied at once
+// into the up to three output rows it belongs to: the three vertical taps'
+// weights lie side by side, [dy = 2 | 1 | 0], as one B operand of 3 N columns,
+// and the accumulators of consecutive output rows are consecutive column
+// blocks of a TMEM ring of kRing rows, so one MMA covers them.  A horizontal
+// tap starts one pixel row further into the unit.
+//   warps 0-7  epilogue, rows in turn between warps 0-3 and 4-7 (bias, ReLU,
+//              BF16, 32-byte stores)
+//   warp 8     TMA        warp 9     MMA
+// An output row still sums over (dy, chunk, dx), or with TAPS over (dy, dx,
+// chunk), the K order of k_conv3x3_tc for the same layer, so the results are
+// the same bit for bit.
+// What bounds it: an MMA of 128 x N x 16 takes max(N / 2, 44) cycles for N <= 64
+// (it reads A at 128 B a cycle), 56 for 96 and 96 for 192 columns: three taps at
+// once cost 56 instead of 3 x 45 at N = 32, 96 instead of 3 x 48 at N = 64.  The
+// one-tile CTAs before this were bound by their L2 loads (weights and three
+// rows a tile) and by the MMA thread's own instructions.  Cold caches, before
+// and now: 32 -> 32 at 1032 x 512 41 -> 17 us (a copy's floor 10), 64 -> 32 46 ->
+// 22; batch 4, 64 -> 64 at 516 x 256 79 -> 33, 128 -> 64 104 -> 52 (1.51 PFLOP/s),
+// at 258 x 128 128 -> 128 54 -> 29 and 256 -> 128 85 -> 70.
+struct RowArgs {
+  bf16 *out;
+  int out_cs, out_off;
+  const float *bias;
+  int relu;
+  int H, W, in_off, cin;
+  int col_blocks;          // 128-pixel column blocks per row
+  int tiles;               // B x col_blocks x H output rows of 128 pixels
+  int wide;                // 32-byte stores are aligned
+  int *err;
+};
+
+constexpr int kRowThreads = 320;
+constexpr int kRing = 8;                     // accumulators (output rows) in TMEM
+constexpr uint32_t kRowSmem = 233472;        // shared memory of an SM for CTAs
+
+template <int N, int KB, int KC>
+struct RowCfg {
+  static constexpr uint32_t UNIT_TX = kHaloPix * KB * 2;
+  static constexpr uint32_t UNIT = (UNIT_TX + 1023) / 1024 * 1024;
+  static constexpr uint32_t W_TILE = N * KB * 2;
+  static constexpr uint32_t W_BYTES = 9 * KC * W_TILE;
+  static constexpr int CPS = N == 32 && KC == 1 ? 2 : 1;   // CTAs per SM (TMEM: kRing N columns each)
+  static constexpr int ROOM = (int(kRowSmem / CPS) - int(W_BYTES) - 3072) / int(UNIT);
+  static constexpr int S = ROOM < 8 ? ROOM : 8;             // units in the ring
+  static_assert(S >= KC && S >= 2, "a whole input row beside the weights");
+  static constexpr uint32_t BAR_OFF = W_BYTES + S * UNIT;
+  static constexpr uint32_t BYTES = BAR_OFF + (2 * S + 1 + 2 * kRing) * 8 + 16 + 1024;
+  static constexpr uint32_t NCOLS = kRing * N;
+};
+
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+// two floats, BF16-rounded, lo in the low half; with relu, negative values and NaN become 0
+__device__ __forceinline__ uint32_t bf16_pair(float lo, float hi, bool relu) {
+  __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+  if (relu) v = __hmax2(v, __floats2bfloat162_rn(0.f, 0.f));
+  return *reinterpret_cast<uint32_t *>(&v);
+}
+// 16 BF16 values as one 32-byte store, or two of 16 bytes
+__device__ __forceinline__ void store16(bf16 *dst, const uint32_t (&o)[8], bool wide) {
+  if (wide) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(o[0]), "r"(o[1]), "r"(o[2]),
+                 "r"(o[3]), "r"(o[4]), "r"(o[5]), "r"(o[6]), "r"(o[7])
+                 : "memory");
+  } else {
+    reinterpret_cast<uint4 *>(dst)[0] = make_uint4(o[0], o[1], o[2], o[3]);
+    reinterpret_cast<uint4 *>(dst)[1] = make_uint4(o[4], o[5], o[6], o[7]);
+  }
+}
+
+// the CTA's runs of output rows: tiles are numbered (image, column block, row)
+struct Runs {
+  int t, t1, H, cbs;
+  int b, cb, h0, rows;
+  __device__ __forceinline__ Runs(const RowArgs &a)
+      : t(int((long long)a.tiles * blockIdx.x / gridDim.x)),
+        t1(int((long long)a.tiles * (blockIdx.x + 1) / gridDim.x)), H(a.H), cbs(a.col_blocks) {}
+  __device__ __forceinline__ bool next() {
+    if (t >= t1) return false;
+    const int col = t / H;
+    h0 = t - col * H;
+    rows = min(t1 - t, H - h0);
+    b = col / cbs;
+    cb = col - b * cbs;
+    t += rows;
+    return true;
+  }
+};
+
+template <int N, int KB, int KC, bool TAPS>
+__global__ void __launch_bounds__(kRowThreads, RowCfg<N, KB, KC>::CPS)
+    k_conv_rows(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, RowArgs a) {
+  using C = RowCfg<N, KB, KC>;
+  constexpr uint32_t S = C::S;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  const uint32_t sW = saddr(smem), sU = sW + C::W_BYTES, bar0 = sW + C::BAR_OFF;
+  // full[s], empty[s] of the units; the weights; accumulators full, accumulators empty
+  const uint32_t wbar = bar0 + 16 * S, tfull = wbar + 8, tempty = tfull + 8 * kRing;
+  uint32_t *slot = reinterpret_cast<uint32_t *>(smem + C::BAR_OFF + (2 * S + 1 + 2 * kRing) * 8);
+  __shared__ int s_fail;
+  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
+  __shared__ float4 s_bias[N / 4];
+  const int n0 = int(blockIdx.y) * N;
+  if (tid < N) reinterpret_cast<float *>(s_bias)[tid] = a.bias ? a.bias[n0 + tid] : 0.f;
+  if (tid == 0) {
+    for (uint32_t s = 0; s < 2 * S; ++s) mbar_init(bar0 + 8 * s, 1);
+    mbar_init(wbar, 1);
+    for (int q = 0; q < kRing; ++q) {
+      mbar_init(tfull + 8 * q, 1);
+      mbar_init(tempty + 8 * q, 4);
+    }
+    s_fail = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) tmem_alloc(saddr(slot), C::NCOLS);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *slot;
+  volatile int *fail = &s_fail;
+
+  if (warp == 8) {
+    if (lane == 0) {
+      mbar_expect_tx(wbar, C::W_BYTES);
+      for (int dx = 0; dx < 3; ++dx)
+        for (int c = 0; c < KC; ++c)
+          for (int dy = 0; dy < 3; ++dy)
+            tma_load_2d(sW + ((dx * KC + c) * 3 + 2 - dy) * C::W_TILE, &tmB, (3 * dy + dx) * a.cin + c * KB, n0, wbar);
+      uint32_t s = 0, ph = 1;   // next unit's slot, and the phase its release completes (the first round waits for none)
+      bool ok = true;
+      Runs r(a);
+      while (ok && r.next())
+        for (int q = -1; q <= r.rows && ok && !*fail; ++q)
+          for (int c = 0; c < KC && ok; ++c) {
+            ok = mbar_wait(bar0 + 8 * (S + s), ph);
+            if (!ok) break;
+            mbar_expect_tx(bar0 + 8 * s, C::UNIT_TX);
+            tma_load_4d(sU + s * C::UNIT, &tmA, a.in_off + c * KB, r.cb * kM - 1, r.h0 + q, r.b, bar0 + 8 * s);
+            if (++s == S) {
+              s = 0;
+              ph ^= 1;
+            }
+          }
+      if (!ok) {
+        atomicExch(&s_fail, 1);
+        atomicCAS(a.err, 0, 1);
+      }
+    }
+  } else if (warp == 9) {
+    const bool leader = elect_one();
+    constexpr uint32_t idesc1 = instr_desc<N>(), idn = (N >> 3) << 17;   // one row's columns; what each row adds
+    // descriptors: only the address field (16-byte units) varies
+    const uint64_t dw64 = smem_desc<KB>(sW);
+    const uint32_t dw = uint32_t(dw64), du = uint32_t(smem_desc<KB>(sU)), dhi = uint32_t(dw64 >> 32);
+    constexpr uint32_t UN = C::UNIT >> 4, WT = C::W_TILE >> 4;
+    bool ok = mbar_wait_warp(wbar, 0);
+    uint32_t s0 = 0, ph = 0;   // slot of the input row's first unit and its phase
+    uint32_t i0 = 0;           // output rows of the runs before
+    Runs r(a);
+    while (ok && r.next()) {
+      for (int q = -1; q <= r.rows && ok; ++q) {
+        // output rows lo .. hi of the run take input row q; row q + 1 starts with it
+        const int lo = max(q - 1, 0), hi = min(q + 1, r.rows - 1);
+        const bool starts = q + 1 < r.rows;
+        if (starts) {
+          const uint32_t i = i0 + q + 1;
+          ok = mbar_wait_warp(tempty + 8 * (i % kRing), ((i / kRing) & 1) ^ 1) && !__any_sync(0xffffffffu, *fail);
+        }
+        // their accumulators: up to the end of the TMEM ring, and from its start
+        const uint32_t r0 = (i0 + lo) % kRing, cnt = hi - lo + 1, ca = min(cnt, kRing - r0), cb = cnt - ca;
+        const uint32_t d0 = tmem + r0 * N, ia = idesc1 + (ca - 1) * idn, ib = idesc1 + (cb - 1) * idn;
+        const uint32_t b0 = 1 - q + lo;   // first weight block: dy = q + 1 - lo, stored as 2 - dy
+        auto unit = [&](int c) { return s0 + c < S ? s0 + c : s0 + c - S; };
+        auto need = [&](int c) {
+          ok = ok && mbar_wait_warp(bar0 + 8 * unit(c), s0 + c < S ? ph : ph ^ 1);
+          tc_fence_after();
+        };
+        auto mma = [&](int c, int dx) {
+          const uint32_t da = du + unit(c) * UN + dx * (Swz<KB>::row_bytes >> 4);
+          const uint32_t db = dw + ((dx * KC + c) * 3 + b0) * WT;
+          const bool head = starts && dx == 0 && c == 0;
+          if (head && leader) {
+            // the starting row's first product replaces what its accumulator held
+            const uint32_t old = cnt - 1, oa = min(old, ca), ob = old - oa;
+            if (oa) mma_bf16_lo(d0, da, db, dhi, idesc1 + (oa - 1) * idn, 1u);
+            if (ob) mma_bf16_lo(tmem, da, db + oa * WT, dhi, idesc1 + (ob - 1) * idn, 1u);
+            mma_bf16_lo(tmem + (i0 + hi) % kRing * N, da, db + old * WT, dhi, idesc1, 0u);
+          }
+          const bool first = !head;
+          if (cb == 0) {
+            if (leader) {
+              if (first) mma_bf16_lo(d0, da, db, dhi, ia, 1u);
+#pragma unroll
+              for (int k = 1; k < KB / 16; ++k) mma_bf16_lo(d0, da + 2 * k, db + 2 * k, dhi, ia, 1u);
+            }
+          } else if (leader) {
+#pragma unroll
+            for (int k = 0; k < KB / 16; ++k)
+              if (k > 0 || first) {
+                mma_bf16_lo(d0, da + 2 * k, db + 2 * k, dhi, ia, 1u);
+                mma_bf16_lo(tmem, da + 2 * k, db + ca * WT + 2 * k, dhi, ib, 1u);
+              }
+          }
+        };
+        auto release = [&](int c) {
+          if (leader) mma_commit(bar0 + 8 * (S + unit(c)));
+        };
+        if (TAPS) {
+#pragma unroll
+          for (int dx = 0; dx < 3; ++dx)
+#pragma unroll
+            for (int c = 0; c < KC; ++c) {
+              if (dx == 0) need(c);
+              if (!ok) break;
+              mma(c, dx);
+              if (dx == 2) release(c);
+            }
+        } else {
+#pragma unroll
+          for (int c = 0; c < KC; ++c) {
+            need(c);
+            if (!ok) break;
+#pragma unroll
+            for (int dx = 0; dx < 3; ++dx) mma(c, dx);
+            release(c);
+          }
+        }
+        if (q >= 1 && leader) mma_commit(tfull + 8 * ((i0 + q - 1) % kRing));   // output row q - 1 is complete
+        s0 += KC;
+        if (s0 >= S) {
+          s0 -= S;
+          ph ^= 1;
+        }
+      }
+      i0 += r.rows;
+    }
+    if (!ok && leader) {
+      atomicExch(&s_fail, 1);
+      atomicCAS(a.err, 0, 2);
+    }
+  } else {
+    // thread (warp w, lane l) owns pixel 32 (w mod 4) + l, the accumulators' TMEM lane
+    const int quad = warp & 3, half = warp >> 2;
+    const bool relu = a.relu != 0, wide = a.wide != 0;
+    uint32_t i = 0;
+    bool ok = true;
+    Runs r(a);
+    while (ok && r.next()) {
+      const int w = r.cb * kM + 32 * quad + lane;
+      bf16 *dst = a.out + ((size_t(r.b) * a.H + r.h0) * a.W + w) * a.out_cs + a.out_off + n0;
+      for (int t = 0; t < r.rows; ++t, ++i, dst += size_t(a.W) * a.out_cs) {
+        if (int(i & 1) != half) continue;
+        const uint32_t acc = i % kRing;
+        ok = __all_sync(0xffffffffu, mbar_wait(tfull + 8 * acc, (i / kRing) & 1));
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t tl = tmem + (uint32_t(32 * quad) << 16) + acc * N;
+#pragma unroll
+        for (int c = 0; c < N; c += 32) {
+          uint32_t v[32];
+          tmem_ld32(tl + c, v);
+          if (c + 32 == N) {   // read out: the MMA may use the accumulator again
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(tempty + 8 * acc);
+          }
+#pragma unroll
+          for (int q = 0; q < 32; q += 16) {
+            uint32_t o[8];
+#pragma unroll
+            for (int k = 0; k < 8; k += 2) {
+              const float4 b = s_bias[(c + q + 2 * k) / 4];
+              const float *x = reinterpret_cast<const float *>(v + q + 2 * k);
+              o[k] = bf16_pair(x[0] + b.x, x[1] + b.y, relu);
+              o[k + 1] = bf16_pair(x[2] + b.z, x[3] + b.w, relu);
+            }
+            if (w < a.W) store16(dst + c + q, o, wide);
+          }
+          __syncwarp();
+        }
+      }
+    }
+    if (!ok && lane == 0) {
+      atomicExch(&s_fail, 1);
+      atomicCAS(a.err, 0, 3);
+    }
+  }
+  __syncwarp();
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0) tmem_dealloc(tmem, C::NCOLS);
 }
 
 // ---------------------------------------------------------------- first layer
@@ -818,6 +1166,58 @@ cudaError_t launch_nks(const ConvTC &c, cudaStream_t s, int nblk) {
   return cudaGetLastError();
 }
 
+// ---- the persistent row kernel (k_conv_rows)
+template <int N, int KB, int KC, bool TAPS>
+cudaError_t prepare_rows() {
+  static cudaError_t e = cudaFuncSetAttribute(k_conv_rows<N, KB, KC, TAPS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              int(RowCfg<N, KB, KC>::BYTES));
+  return e;
+}
+
+template <int N, int KB, int KC, bool TAPS>
+cudaError_t launch_rows(const ConvTC &c, cudaStream_t s, int sms) {
+  using R = RowCfg<N, KB, KC>;
+  auto fn = encode_fn();
+  if (!fn) return cudaErrorNotSupported;
+  const cudaError_t attr = prepare_rows<N, KB, KC, TAPS>();
+  if (attr != cudaSuccess) return attr;
+  CUtensorMap ta, tb;
+  const cuuint32_t one[4] = {1, 1, 1, 1};
+  const cuuint64_t adim[4] = {cuuint64_t(c.in_cs), cuuint64_t(c.W), cuuint64_t(c.H), cuuint64_t(c.B)};
+  const cuuint64_t astr[3] = {cuuint64_t(c.in_cs) * 2, cuuint64_t(c.in_cs) * 2 * c.W,
+                              cuuint64_t(c.in_cs) * 2 * c.W * c.H};
+  const cuuint32_t abox[4] = {cuuint32_t(KB), cuuint32_t(kHaloPix), 1, 1};
+  if (fn(&ta, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<bf16 *>(c.in), adim, astr, abox, one,
+         CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle_of(KB), CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+    return cudaErrorInvalidValue;
+  const cuuint64_t bdim[2] = {cuuint64_t(9) * c.cin, cuuint64_t(c.cout)};
+  const cuuint64_t bstr[1] = {cuuint64_t(9) * c.cin * 2};
+  const cuuint32_t bbox[2] = {cuuint32_t(KB), cuuint32_t(N)};
+  if (fn(&tb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<bf16 *>(c.w), bdim, bstr, bbox, one,
+         CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle_of(KB), CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+    return cudaErrorInvalidValue;
+  RowArgs a;
+  a.out = c.out;
+  a.out_cs = c.out_cs;
+  a.out_off = c.out_off;
+  a.bias = c.bias;
+  a.relu = c.relu;
+  a.H = c.H;
+  a.W = c.W;
+  a.in_off = c.in_off;
+  a.cin = c.cin;
+  a.col_blocks = (c.W + kM - 1) / kM;
+  a.tiles = c.B * a.col_blocks * c.H;
+  a.wide = c.out_cs % 16 == 0 && c.out_off % 16 == 0 && (reinterpret_cast<uintptr_t>(c.out) & 31) == 0;
+  a.err = c.err;
+  const int nblk = c.cout / N;
+  const int ctas = std::max(1, std::min(a.tiles, sms * R::CPS / nblk));
+  k_conv_rows<N, KB, KC, TAPS><<<dim3(unsigned(ctas), unsigned(nblk)), kRowThreads, R::BYTES, s>>>(ta, tb, a);
+  return cudaGetLastError();
+}
+
 template <int N, int KB, bool UP>
 cudaError_t launch_nk(const ConvTC &c, cudaStream_t s, int nblk, long long ctas, int sms) {
   // the halo loads for the 3x3 convolutions of up to 64 columns on images at
@@ -1052,7 +1452,12 @@ cudaError_t conv3x3_tc_prepare() {
   if (e == cudaSuccess) e = tc::prepare_n<256>();
   for (cudaError_t f : {tc::prepare_wgrad<32, 16>(), tc::prepare_wgrad<32, 32>(), tc::prepare_wgrad<32, 64>(),
                         tc::prepare_wgrad<64, 16>(), tc::prepare_wgrad<64, 32>(), tc::prepare_wgrad<64, 64>(),
-                        tc::prepare_wgrad<32, 64, true>(), tc::prepare_wgrad<64, 64, true>()})
+                        tc::prepare_wgrad<32, 64, true>(), tc::prepare_wgrad<64, 64, true>(),
+                        tc::prepare_rows<32, 32, 1, false>(), tc::prepare_rows<32, 64, 1, false>(),
+                        tc::prepare_rows<64, 32, 1, false>(), tc::prepare_rows<64, 64, 1, false>(),
+                        tc::prepare_rows<64, 64, 2, false>(), tc::prepare_rows<64, 64, 1, true>(),
+                        tc::prepare_rows<64, 64, 2, true>(), tc::prepare_rows<32, 64, 4, false>(),
+                        tc::prepare_rows<32, 64, 4, true>()})
     if (e == cudaSuccess) e = f;
   return e;
 }
@@ -1081,6 +1486,20 @@ cudaError_t conv3x3_tc(const ConvTC &c, cudaStream_t s) {
   }
   const long long ctas = tiles * nblk;
   const bool up = c.up_cout != 0;
+  // the persistent row kernel (whole 128-pixel rows; input channels whose
+  // weights fit beside a row), with the K order of the kernel it replaces: that
+  // one takes (dy, chunk, dx) up to 64 columns a CTA and (dy, dx, chunk) above
+  if (!up && c.W >= tc::kM && (long long)c.B * ((c.W + tc::kM - 1) / tc::kM) * c.H < (1LL << 31)) {
+    if (n == 32 && c.cin == 32) return tc::launch_rows<32, 32, 1, false>(c, s, sms);
+    if (n == 32 && c.cin == 64) return tc::launch_rows<32, 64, 1, false>(c, s, sms);
+    if (n == 64 && c.cin == 32) return tc::launch_rows<64, 32, 1, false>(c, s, sms);
+    if (n == 64 && c.cin == 64) return tc::launch_rows<64, 64, 1, false>(c, s, sms);
+    if (n == 64 && c.cin == 128) return tc::launch_rows<64, 64, 2, false>(c, s, sms);
+    if (n == 64 && c.cin == 256) return tc::launch_rows<32, 64, 4, false>(c, s, sms);
+    if (n >= 128 && c.cin == 64) return tc::launch_rows<64, 64, 1, true>(c, s, sms);
+    if (n >= 128 && c.cin == 128) return tc::launch_rows<64, 64, 2, true>(c, s, sms);
+    if (n >= 128 && c.cin == 256) return tc::launch_rows<32, 64, 4, true>(c, s, sms);
+  }
   switch (n) {
     case 32: return up ? tc::launch_n<32, true>(c, s, nblk, ctas, sms) : tc::launch_n<32, false>(c, s, nblk, ctas, sms);
     case 64: return up ? tc::launch_n<64, true>(c, s, nblk, ctas, sms) : tc::launch_n<64, false>(c, s, nblk, ctas, sms);
