@@ -463,49 +463,63 @@ struct pic_batch {
   int sort_every = 1;
   int steps_since_sort = 0;
   int timing = 0;
-  cudaGraph_t graph[2] = {nullptr, nullptr};
-  cudaGraphExec_t gexec[2] = {nullptr, nullptr};
-  cudaEvent_t ev[2] = {nullptr, nullptr};
+  // Groups of members, each with its own graph (a member a branch) and stream:
+  // a group's next step does not wait for the other groups' solves.
+  struct Group {
+    std::vector<pic_ctx *> m;
+    cudaStream_t stream = nullptr;
+    cudaEvent_t done = nullptr;
+    cudaGraph_t graph[2] = {nullptr, nullptr};
+    cudaGraphExec_t gexec[2] = {nullptr, nullptr};
+  };
+  std::vector<Group> groups;
+  cudaEvent_t ev[2] = {nullptr, nullptr};   // the groups' start on the batch's stream, their end
   double t_ms = 0.0;
   int64_t t_steps = 0;
 };
 
+// As many groups as the device has independent work queues by default.  In one
+// graph per ensemble step every member waited for the slowest one's solve, some
+// 50 us a step with little else running (eight members of the width sweep).
+constexpr int kMaxGroups = 8;
+
 namespace picgb {
 namespace {
 
-// The ensemble graph: an event node, then every member's step as an
-// independent branch, then an event node after all of them.
-cudaError_t batch_graph(pic_batch *b, int with_sort) {
-  if (b->gexec[with_sort]) return cudaSuccess;
+// A group's graph: every member's step as an independent branch.
+cudaError_t group_graph(pic_batch::Group &q, int with_sort) {
+  if (q.gexec[with_sort]) return cudaSuccess;
   cudaGraph_t g;
   cudaError_t e = cudaGraphCreate(&g, 0);
   if (e != cudaSuccess) return e;
-  std::vector<cudaGraphNode_t> root, leaves;
-  e = cudaStreamBeginCaptureToGraph(b->stream, g, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
-  if (e == cudaSuccess) {
-    cudaEventRecordWithFlags(b->ev[0], b->stream, cudaEventRecordExternal);
-    e = capture_leaves(b->stream, root);
-  }
-  for (size_t k = 0; e == cudaSuccess && k < b->m.size(); ++k) {
-    std::vector<cudaGraphNode_t> d = root;
-    e = capture_step(b->m[k], g, d, with_sort, false);
-    leaves.insert(leaves.end(), d.begin(), d.end());
-  }
-  if (e == cudaSuccess) {
-    e = cudaStreamBeginCaptureToGraph(b->stream, g, leaves.data(), nullptr, leaves.size(),
-                                      cudaStreamCaptureModeThreadLocal);
-    if (e == cudaSuccess) {
-      cudaEventRecordWithFlags(b->ev[1], b->stream, cudaEventRecordExternal);
-      std::vector<cudaGraphNode_t> tail;
-      e = capture_leaves(b->stream, tail);
-    }
+  for (size_t k = 0; e == cudaSuccess && k < q.m.size(); ++k) {
+    std::vector<cudaGraphNode_t> d;
+    e = capture_step(q.m[k], g, d, with_sort, false);
   }
   note(e, "ensemble graph capture");
-  if (e == cudaSuccess) e = note(cudaGraphInstantiate(&b->gexec[with_sort], g, 0), "ensemble graph instantiate");
-  if (e == cudaSuccess) b->graph[with_sort] = g;
+  if (e == cudaSuccess) e = note(cudaGraphInstantiate(&q.gexec[with_sort], g, 0), "ensemble graph instantiate");
+  if (e == cudaSuccess) q.graph[with_sort] = g;
   else cudaGraphDestroy(g);
   cudaGetLastError();
   return e;
+}
+
+// the groups' streams take up after what the batch's stream holds, and the
+// batch's stream after theirs
+pic_status groups_fork(pic_batch *b) {
+  cudaError_t e = cudaEventRecord(b->ev[0], b->stream);
+  for (auto &q : b->groups)
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(q.stream, b->ev[0], 0);
+  return note(e, "ensemble streams") == cudaSuccess ? PIC_OK : PIC_ECUDA;
+}
+pic_status groups_join(pic_batch *b) {
+  cudaError_t e = cudaSuccess;
+  for (auto &q : b->groups) {
+    if (e == cudaSuccess) e = cudaEventRecord(q.done, q.stream);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, q.done, 0);
+  }
+  if (e == cudaSuccess) e = cudaEventRecord(b->ev[1], b->stream);
+  return note(e, "ensemble streams") == cudaSuccess ? PIC_OK : PIC_ECUDA;
 }
 
 }  // namespace
@@ -554,6 +568,23 @@ pic_status pic_batch_init(const pic_config *cfgs, int32_t n, void *stream, pic_b
     c->sharing = n;
     b->m.push_back(c);
   }
+  // members to groups by size, back and forth, so that the groups' steps take about as long
+  std::vector<pic_ctx *> order = b->m;
+  std::stable_sort(order.begin(), order.end(), [](const pic_ctx *x, const pic_ctx *y) {
+    return x->cfg.capacity[0] + x->cfg.capacity[1] > y->cfg.capacity[0] + y->cfg.capacity[1];
+  });
+  const int ng = std::min<int>(n, kMaxGroups);
+  b->groups.resize(ng);
+  for (int k = 0; k < n; ++k) {
+    const int r = k % (2 * ng);
+    b->groups[r < ng ? r : 2 * ng - 1 - r].m.push_back(order[k]);
+  }
+  for (auto &q : b->groups)
+    if (cudaStreamCreateWithFlags(&q.stream, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaEventCreateWithFlags(&q.done, cudaEventDisableTiming) != cudaSuccess) {
+      pic_batch_free(b);
+      return PIC_ECUDA;
+    }
   *out = b;
   return PIC_OK;
 }
@@ -577,15 +608,25 @@ pic_status pic_batch_step(pic_batch *b, int32_t nsteps) {
     b->steps_since_sort = 0;
     for (pic_ctx *c : b->m) c->steps_since_sort = 0;
   }
-  for (int32_t k = 0; k < nsteps; ++k) {
+  pic_status st = PIC_OK;
+  for (int32_t k = 0; k < nsteps && st == PIC_OK; ++k) {
     int sorting = b->steps_since_sort >= b->sort_every ? 1 : 0;
     for (pic_ctx *c : b->m) {   // a member restored from a checkpoint
       if (c->needs_sort) sorting = 1;
       c->needs_sort = 0;
     }
-    if (check(batch_graph(b, sorting)) != PIC_OK) return PIC_ECUDA;
-    if (note(cudaGraphLaunch(b->gexec[sorting], b->stream), "ensemble graph launch") != cudaSuccess)
-      return PIC_ECUDA;
+    for (auto &q : b->groups)
+      if (check(group_graph(q, sorting)) != PIC_OK) st = PIC_ECUDA;
+    if (st == PIC_OK && (k == 0 || b->timing)) st = groups_fork(b);
+    for (auto &q : b->groups)
+      if (st == PIC_OK && note(cudaGraphLaunch(q.gexec[sorting], q.stream), "ensemble graph launch") != cudaSuccess)
+        st = PIC_ECUDA;
+    // (also after a failure: what was launched ends before later work of the batch's stream)
+    if (k + 1 == nsteps || b->timing || st != PIC_OK) {
+      const pic_status sj = groups_join(b);
+      if (st == PIC_OK) st = sj;
+    }
+    if (st != PIC_OK) break;
     for (pic_ctx *c : b->m) {
       if (sorting) {
         c->cur[0] ^= 1;
@@ -604,7 +645,7 @@ pic_status pic_batch_step(pic_batch *b, int32_t nsteps) {
       b->t_steps += 1;
     }
   }
-  return PIC_OK;
+  return st;
 }
 
 pic_status pic_batch_timing(pic_batch *b, double *out) {
@@ -621,10 +662,16 @@ pic_status pic_batch_timing(pic_batch *b, double *out) {
 pic_status pic_batch_free(pic_batch *b) {
   if (!b) return PIC_OK;
   cudaSetDevice(b->dev);
+  for (auto &q : b->groups)
+    if (q.stream) cudaStreamSynchronize(q.stream);
   if (b->stream) cudaStreamSynchronize(b->stream);
-  for (int k = 0; k < 2; ++k) {
-    if (b->gexec[k]) cudaGraphExecDestroy(b->gexec[k]);
-    if (b->graph[k]) cudaGraphDestroy(b->graph[k]);
+  for (auto &q : b->groups) {
+    for (int k = 0; k < 2; ++k) {
+      if (q.gexec[k]) cudaGraphExecDestroy(q.gexec[k]);
+      if (q.graph[k]) cudaGraphDestroy(q.graph[k]);
+    }
+    if (q.done) cudaEventDestroy(q.done);
+    if (q.stream) cudaStreamDestroy(q.stream);
   }
   for (pic_ctx *c : b->m) pic_free(c);
   for (int k = 0; k < 2; ++k)

@@ -31,224 +31,30 @@
 #include <cmath>
 #include <vector>
 
+#include "boxpoisson.cuh"
 #include "internal.cuh"
 
 namespace picgb {
 namespace {
 
-constexpr int kSolveThreads = 512;
 constexpr int kAddThreads = 128;       // one column per thread
-constexpr int kKB = 4;                 // modes per CTA of the solve
 constexpr int kChunkK = 32;            // modes staged per round of the inverse transform
 constexpr int kMaxCols = 1024;         // columns of the basis (V is n x n)
 constexpr int kMaxRows = 4096;
 constexpr int kMaxSlot = 512;          // interface columns (their Schur complement is inverted on the host)
 
-__host__ __device__ constexpr int pad4(int n) { return (n + 3) & ~3; }
-__host__ __device__ constexpr int pad8(int n) { return (n + 7) & ~7; }
+int pad4(int n) { return (n + 3) & ~3; }
+int pad8(int n) { return (n + 7) & ~7; }
 
-struct BoxArgs {
-  BoxBlock b[2];           // slab, slot
-  int nblk[2];             // CTAs of the solve per block
-  int pitch;               // nodes per grid row
-  int slot, xs, singular;
-  const float *sinv;       // [wc][wc] inverse of the interface's Schur complement
-  float *fh, *sh;          // spectra of the interface values in the slab's and the slot's basis
-  unsigned int *ticket;
-  const float *r;
-  float2 *pot;
-  PoissonState *ps;
-};
-
-// tridiag(-1, d, -1) x = y in place for one warp: y_i <- w_i (y_i + y_{i-1}),
-// then x_i = y_i + w_i x_{i+1} (Thomas, w_i = 1 / (d - w_{i-1})).  Each lane
-// takes a run of rows; both recurrences are linear in the value carried into
-// the run, so a first pass gives every run's result for a zero carry and the
-// product of its factors, a scan over the lanes the carries, and a second pass
-// the values.  An odd run length keeps the lanes on different banks.
-__device__ __forceinline__ void tri_warp(float *y, const float *w, int m) {
-  const int lane = threadIdx.x & 31, L = ((m + 31) / 32) | 1;
-  const int lo = min(m, lane * L), hi = min(m, lo + L);
-  float v = 0.f, p = 1.f;
-  for (int i = lo; i < hi; ++i) {
-    v = w[i] * (y[i] + v);
-    p *= w[i];
-  }
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const float v0 = __shfl_up_sync(0xffffffffu, v, o), p0 = __shfl_up_sync(0xffffffffu, p, o);
-    if (lane >= o) {
-      v = fmaf(p, v0, v);
-      p *= p0;
-    }
-  }
-  float c = __shfl_up_sync(0xffffffffu, v, 1);
-  if (lane == 0) c = 0.f;
-  for (int i = lo; i < hi; ++i) {
-    c = w[i] * (y[i] + c);
-    y[i] = c;
-  }
-  __syncwarp();
-  v = 0.f;
-  p = 1.f;
-  for (int i = hi - 1; i >= lo; --i) {
-    v = fmaf(w[i], v, y[i]);
-    p *= w[i];
-  }
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const float v0 = __shfl_down_sync(0xffffffffu, v, o), p0 = __shfl_down_sync(0xffffffffu, p, o);
-    if (lane + o < 32) {
-      v = fmaf(p, v0, v);
-      p *= p0;
-    }
-  }
-  c = __shfl_down_sync(0xffffffffu, v, 1);
-  if (lane == 31) c = 0.f;
-  for (int i = hi - 1; i >= lo; --i) {
-    c = fmaf(w[i], c, y[i]);
-    y[i] = c;
-  }
-  __syncwarp();
-}
-
-// The interface, in the last CTA to finish: g = r_G + v_R(row m) + v_S(first
-// slot row), u_G = S^-1 g added to the potential, and the spectra of u_G that
-// the inverse transform applies.
-__device__ void box_interface(const BoxArgs &f, float *sm) {
-  const BoxBlock &R = f.b[0], &S = f.b[1];
-  const int wc = S.n, nk = R.n, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  float *vm = sm, *vs = vm + nk, *g = vs + wc, *u = g + wc;
-  for (int k = threadIdx.x; k < nk; k += blockDim.x) vm[k] = __ldcg(R.c + size_t(k) * R.mp + R.m - 1);
-  for (int k = threadIdx.x; k < wc; k += blockDim.x) vs[k] = __ldcg(S.c + size_t(k) * S.mp);
-  __syncthreads();
-  const int c0 = S.col0 - R.col0;   // the slot's first column in the slab's numbering
-  for (int c = warp; c < wc; c += nw) {
-    const float *vr = R.v + size_t(c0 + c) * R.ldv, *vc = S.v + size_t(c) * S.ldv;
-    float a = 0.f;
-    for (int k = lane; k < nk; k += 32) a = fmaf(vm[k], __ldg(vr + k), a);
-    for (int k = lane; k < wc; k += 32) a = fmaf(vs[k], __ldg(vc + k), a);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-    if (lane == 0) g[c] = f.r[size_t(f.xs) * f.pitch + S.col0 + c] + a;
-  }
-  __syncthreads();
-  for (int c = warp; c < wc; c += nw) {
-    float a = 0.f;
-    for (int q = lane; q < wc; q += 32) a = fmaf(__ldg(f.sinv + size_t(c) * wc + q), g[q], a);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-    if (lane == 0) {
-      u[c] = a;
-      const size_t n = size_t(f.xs) * f.pitch + S.col0 + c;
-      f.pot[n] = pair_add_f(f.pot[n], a);
-    }
-  }
-  __syncthreads();
-  for (int k = threadIdx.x; k < nk; k += blockDim.x) {
-    float a = 0.f;
-#pragma unroll 8
-    for (int c = 0; c < wc; ++c) a = fmaf(u[c], __ldg(R.v + size_t(c0 + c) * R.ldv + k), a);
-    f.fh[k] = a;
-  }
-  for (int k = threadIdx.x; k < wc; k += blockDim.x) {
-    float a = 0.f;
-#pragma unroll 8
-    for (int c = 0; c < wc; ++c) a = fmaf(u[c], __ldg(S.v + size_t(c) * S.ldv + k), a);
-    f.sh[k] = a;
-  }
-}
-
-// kKB modes of one block per CTA: c[k][i] = sum_j r[i][j] V[j][k] over all
-// rows i (a warp takes four rows at a time, lanes along j; the basis columns
-// and the Thomas factors are static and staged before the wait for the
-// preceding kernel), then each mode's tridiagonal system in one warp.
-__global__ void __launch_bounds__(kSolveThreads) k_box_solve(BoxArgs f) {
+// one group of modes per CTA (the tables staged before the wait for the
+// preceding kernel); the last CTA to finish solves the interface
+__global__ void __launch_bounds__(kBoxThreads, 1) k_box_solve(BoxArgs f) {
   extern __shared__ __align__(16) float sm[];
   __shared__ bool last;
-  const int which = int(blockIdx.x) < f.nblk[0] ? 0 : 1;
-  const BoxBlock &B = f.b[which];
-  const int k0 = (int(blockIdx.x) - (which ? f.nblk[0] : 0)) * kKB;
-  const int n = B.n, m = B.m, mp = B.mp;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  float4 *vs = reinterpret_cast<float4 *>(sm);   // [n] the CTA's basis columns
-  float *ws = sm + 4 * n;                        // [kKB][mp] Thomas factors
-  float *cs = ws + kKB * mp;                     // [kKB][mp] spectra
-  for (int j = threadIdx.x; j < n; j += blockDim.x)
-    vs[j] = __ldg(reinterpret_cast<const float4 *>(B.v + size_t(j) * B.ldv + k0));
-  for (int t = threadIdx.x; t < kKB * mp; t += blockDim.x) {
-    const int kk = t / mp;
-    ws[t] = k0 + kk < n ? __ldg(B.w + size_t(k0) * mp + t) : 0.f;
-  }
+  box_stage(f, blockIdx.x, sm);
   pdl_enter();
   __syncthreads();
-  for (int i0 = 4 * warp; i0 < m; i0 += 4 * nw) {
-    float a[16];
-#pragma unroll
-    for (int q = 0; q < 16; ++q) a[q] = 0.f;
-    const float *r0 = f.r + size_t(B.row0 + i0) * f.pitch + B.col0;
-#pragma unroll 4
-    for (int j = lane; j < n; j += 32) {
-      const float4 v = vs[j];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const float rv = i0 + q < m ? r0[size_t(q) * f.pitch + j] : 0.f;
-        a[4 * q + 0] = fmaf(rv, v.x, a[4 * q + 0]);
-        a[4 * q + 1] = fmaf(rv, v.y, a[4 * q + 1]);
-        a[4 * q + 2] = fmaf(rv, v.z, a[4 * q + 2]);
-        a[4 * q + 3] = fmaf(rv, v.w, a[4 * q + 3]);
-      }
-    }
-    // sums over the lanes: each exchange halves the values a lane still holds,
-    // lane l ends with value l >> 1 (both lanes of a pair hold half of it)
-#pragma unroll
-    for (int h = 8, o = 16; h >= 1; h >>= 1, o >>= 1) {
-      const bool upper = (lane & o) != 0;
-#pragma unroll
-      for (int q = 0; q < h; ++q) {
-        const float keep = upper ? a[q + h] : a[q], give = upper ? a[q] : a[q + h];
-        a[q] = keep + __shfl_xor_sync(0xffffffffu, give, o);
-      }
-    }
-    a[0] += __shfl_xor_sync(0xffffffffu, a[0], 1);
-    const int q = lane >> 1, i = i0 + (q >> 2);
-    if (!(lane & 1) && i < m) cs[(q & 3) * mp + i] = a[0];
-  }
-  __syncthreads();
-  if (warp < kKB && k0 + warp < n) {
-    const int k = k0 + warp;
-    float *y = cs + warp * mp;
-    const float *w = ws + warp * mp;
-    if (!B.ring) {
-      tri_warp(y, w, m);
-    } else {
-      // a ring of m rows: rows 1 .. m - 1 with row 0 held, then row 0 from
-      // its own equation and its response z on the others; the singular
-      // system (a doubly periodic box's constant mode) keeps row 0 at 0 and
-      // loses its mean
-      tri_warp(y + 1, w + 1, m - 1);
-      const float x0 = (y[0] + y[1] + y[m - 1]) * __ldg(B.ring + k);
-      __syncwarp();
-      const float *z = B.z + size_t(k) * mp;
-      float s = 0.f;
-      for (int i = 1 + lane; i < m; i += 32) {
-        const float x = fmaf(x0, __ldg(z + i), y[i]);
-        y[i] = x;
-        s += x;
-      }
-      __syncwarp();
-      if (lane == 0) y[0] = x0;
-      if (f.singular && k == 0) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        s /= float(m);
-        __syncwarp();
-        for (int i = lane; i < m; i += 32) y[i] -= s;
-      }
-      __syncwarp();
-    }
-    for (int i = lane; i < m; i += 32) B.c[size_t(k) * mp + i] = y[i];
-  }
+  box_modes(f, blockIdx.x, sm);
   if (!f.slot) return;
   __syncthreads();   // the CTA's stores, then its arrival
   if (threadIdx.x == 0) {
@@ -343,7 +149,6 @@ __global__ void __launch_bounds__(kAddThreads) k_box_add(BoxArgs f, int split) {
     if (i0 + q < m) f.pot[size_t(B.row0 + i0 + q) * f.pitch + B.col0 + j] = pair_add_f(pot[q], e[q]);
 }
 
-size_t solve_smem(const BoxBlock &b) { return (4 * size_t(b.n) + 2 * kKB * size_t(b.mp)) * 4; }
 size_t add_smem(const BoxBlock &b, int bm) { return (2 * size_t(kChunkK) * kAddThreads + size_t(b.n) * bm) * 4; }
 int add_ctas(const BoxBlock &b, int bm) {
   return ((b.n + kAddThreads - 1) / kAddThreads) * ((b.m + bm - 1) / bm);
@@ -460,6 +265,8 @@ bool invert_spd(std::vector<double> &A, int n) {   // in place, Gauss-Jordan (di
   return true;
 }
 
+}  // namespace
+
 BoxArgs box_args(pic_ctx *c, const float *r, float2 *pot, PoissonState *ps) {
   const BoxPoisson &p = c->box;
   BoxArgs a;
@@ -481,8 +288,6 @@ BoxArgs box_args(pic_ctx *c, const float *r, float2 *pot, PoissonState *ps) {
   return a;
 }
 
-}  // namespace
-
 // Enabled (automatic method only) for free nodes that form a full slab --
 // rows 1 .. m of a bounded x, or every row of a periodic one, all columns of a
 // periodic y or all between the walls of a bounded one -- and, below a bounded
@@ -492,7 +297,9 @@ cudaError_t box_poisson_setup(pic_ctx *c) {
   BoxPoisson &p = c->box;
   p = BoxPoisson();
   const Geom &g = c->g;
-  if (c->cfg.poisson_method != 0 || c->fp.enabled) return cudaSuccess;
+  if (c->cfg.poisson_method != 0) return cudaSuccess;
+  // beside the FFT solve only for the passes its closing kernel may add
+  if (c->fp.enabled && c->g.nxn * c->g.nyn > kTailNodes) return cudaSuccess;
   const int nyn = g.nyn, nxn = g.nxn, col0 = g.py ? 0 : 1, n = g.py ? nyn : nyn - 2;
   if (n < 2 || n > kMaxCols) return cudaSuccess;
   auto free_at = [&](int i, int j) { return (c->h_nodeflags[size_t(i) * nyn + j] & kFree) != 0; };
@@ -580,10 +387,10 @@ cudaError_t box_poisson_setup(pic_ctx *c) {
   // rows per CTA of the inverse transform: 8 halves the basis traffic, 4 gives
   // twice the CTAs where 8 would leave SMs idle
   p.bm = add_ctas(R, 8) >= c->num_sms ? 8 : 4;
-  p.solve_smem = std::max(solve_smem(R), (size_t(n) + 3 * kMaxSlot) * 4);
+  p.solve_smem = std::max(box_solve_smem(R), (size_t(n) + 3 * kMaxSlot) * 4);
   p.add_smem = add_smem(R, p.bm);
   if (p.slot) {
-    p.solve_smem = std::max(p.solve_smem, solve_smem(S));
+    p.solve_smem = std::max(p.solve_smem, box_solve_smem(S));
     p.add_smem = std::max(p.add_smem, add_smem(S, p.bm));
   }
   constexpr size_t kSmem = 220 * 1024;   // the largest size any context may use
@@ -592,18 +399,19 @@ cudaError_t box_poisson_setup(pic_ctx *c) {
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_box_add<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSmem));
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_box_add<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSmem));
   if (e != cudaSuccess) return e;
-  p.enabled = 1;
+  p.enabled = c->fp.enabled ? 0 : 1;
+  if ((e = box_tail_setup(c)) != cudaSuccess) return e;
   return cudaGetLastError();
 }
 
 void box_poisson_launch(pic_ctx *c, const float *r, float2 *pot, PoissonState *ps) {
   const BoxPoisson &p = c->box;
   const BoxArgs a = box_args(c, r, pot, ps);
-  launch(k_box_solve, a.nblk[0] + a.nblk[1], kSolveThreads, p.solve_smem, c->stream, a);
+  launch(k_box_solve, a.nblk[0] + a.nblk[1], kBoxThreads, p.solve_smem, c->stream, a);
+  c->launches += 2;
   const int s0 = add_ctas(p.b[0], p.bm), s1 = p.slot ? add_ctas(p.b[1], p.bm) : 0;
   if (p.bm == 8) launch(k_box_add<8>, s0 + s1, kAddThreads, p.add_smem, c->stream, a, s0);
   else launch(k_box_add<4>, s0 + s1, kAddThreads, p.add_smem, c->stream, a, s0);
-  c->launches += 2;
 }
 
 }  // namespace picgb

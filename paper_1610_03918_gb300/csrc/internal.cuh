@@ -251,6 +251,9 @@ struct BoxPoisson {
   const float *sinv = nullptr;     // [wc][wc] inverse of the interface's Schur complement
   float *fh = nullptr, *sh = nullptr;   // spectra of the interface values
   int bm = 8;                      // rows per CTA of the inverse transform
+  int tail = 0;                    // the captured step's solve is checked, and repeated, in one cluster
+  int cluster = 0;                 // CTAs of that cluster
+  size_t tail_smem = 0;
   size_t solve_smem = 0, add_smem = 0;
 };
 
@@ -268,6 +271,26 @@ constexpr bool kPdl = true;
 #else
 constexpr bool kPdl = false;
 #endif
+
+// one cluster of `ctas` CTAs
+template <typename... P, typename... A>
+void launch_cluster(void (*k)(P...), int ctas, int block, size_t smem, cudaStream_t s, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(unsigned(ctas));
+  cfg.blockDim = dim3(unsigned(block));
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = unsigned(ctas);
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = kPdl ? 2 : 1;
+  cudaLaunchKernelEx(&cfg, k, args...);
+}
 
 template <typename... P, typename... A>
 void launch(void (*k)(P...), int grid, int block, size_t smem, cudaStream_t s, A... args) {
@@ -447,6 +470,8 @@ void fast_poisson_launch(pic_ctx *c, const float *r, float2 *pot, PoissonState *
 // Transform inner solve (boxpoisson.cu), likewise: two kernels per pass.
 cudaError_t box_poisson_setup(pic_ctx *c);
 void box_poisson_launch(pic_ctx *c, const float *r, float2 *pot, PoissonState *ps);
+// the closing kernel's set-up (poisson.cu)
+cudaError_t box_tail_setup(pic_ctx *c);
 // one of the two is in use: each refinement pass is one of its solves, which
 // adds the correction to the potential itself
 inline bool one_pass_solver(const pic_ctx *c) { return c->fp.enabled || c->box.enabled; }

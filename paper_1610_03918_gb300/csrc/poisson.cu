@@ -39,6 +39,7 @@
 #include <map>
 #include <type_traits>
 
+#include "boxpoisson.cuh"
 #include "internal.cuh"
 
 namespace picgb {
@@ -642,6 +643,130 @@ __global__ void k_resid(FineArgs a) {
     ps->beta = 0.0;
     ps->rz = 0.0;
     *a.ticket = 0u;
+  }
+}
+
+// The end of a step's transform solve in one thread-block cluster: the checking
+// pass (E, norms, decision) and, while the decision asks for them, further
+// passes -- transforms, interface, check -- with the cluster's barrier between
+// their parts.  Every CTA takes the same decision from the same sums.  A
+// conditional graph node that decides whether to repeat costs 6 to 9 us a step
+// even when it does not; the price is that a cluster has 16 SMs.  Step on 80 x
+// 30: 49.9 -> 38.4 us, 128 x 96 50.0 -> 41.1, 256 x 256 181.7 -> 175.1.  With the
+// first pass's inverse transform in the cluster as well, a kernel less, 46.8,
+// 57.3 and 315 us: 16 SMs are too few for it.
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+template <bool SING>
+__global__ void __launch_bounds__(kBoxThreads, 1) k_box_tail(FineArgs a, BoxArgs f, int first_check) {
+  extern __shared__ __align__(16) float sm[];
+  __shared__ int s_go;
+  const int rank = blockIdx.x, ncta = gridDim.x;
+  pdl_enter();
+  const Geom g = a.g;
+  const int nn = g.nxn * g.nyn, per = (nn + ncta - 1) / ncta, n0 = rank * per, n1 = min(nn, n0 + per);
+  PoissonState *ps = a.ps;
+  int outer = __ldcg(&ps->outer_iters), total = __ldcg(&ps->total_iters);
+  const double bb = __ldcg(&ps->bb);
+  float2 bm = make_float2(0.f, 0.f);
+  if (SING) bm = pair_split(ps->bmean);
+  for (;;) {
+    SqSum q[2] = {};
+    for (int base = n0 + int(threadIdx.x); base < n1; base += kVB * kBoxThreads) {
+      float2 rh[kVB], ph[kVB][5];
+      uint8_t fl[kVB];
+#pragma unroll
+      for (int k = 0; k < kVB; ++k) {
+        const int n = base + k * kBoxThreads;
+        if (n >= n1) continue;
+        int xm, xp, ym, yp;
+        nbr_index(g, n, xm, xp, ym, yp);
+        fl[k] = a.flags[n];
+        rh[k] = a.rho[n];
+        ph[k][0] = __ldcg(a.phi + n);
+        ph[k][1] = __ldcg(a.phi + xm);
+        ph[k][2] = __ldcg(a.phi + xp);
+        ph[k][3] = __ldcg(a.phi + ym);
+        ph[k][4] = __ldcg(a.phi + yp);
+      }
+#pragma unroll
+      for (int k = 0; k < kVB; ++k) {
+        const int n = base + k * kBoxThreads;
+        if (n >= n1) continue;
+        float r32 = 0.f;
+        if (fl[k] & kFree) {
+          r32 = resid_node(SING ? pair_sub(rh[k], bm) : rh[k], ph[k]);
+          sq_add(q[0], r32);
+        }
+        a.r32[n] = r32;
+        const float2 E = node_field(fl[k], ph[k]);
+        a.E[n] = E;
+        sq_add(q[1], E.x);
+        sq_add(q[1], E.y);
+      }
+    }
+    float c[6] = {q[0].mid, q[0].big, q[0].tiny, q[1].mid, q[1].big, q[1].tiny};
+    block_tree<6>(c);
+    if (threadIdx.x == 0) {
+#pragma unroll
+      for (int k = 0; k < 6; ++k) a.partf[rank * 6 + k] = c[k];
+    }
+    cluster_sync();
+    if (threadIdx.x < 32) {
+#pragma unroll
+      for (int k = 0; k < 6; ++k) {
+        c[k] = int(threadIdx.x) < ncta ? __ldcg(a.partf + threadIdx.x * 6 + k) : 0.f;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) c[k] += __shfl_down_sync(0xffffffffu, c[k], o);
+      }
+    }
+    if (threadIdx.x == 0) {
+      const double rr = sq_join(c);
+      const float bbf = float(bb);
+      const double rel = (c[1] == 0.f && c[2] == 0.f && bbf > 1e-30f && bbf < 1e30f)
+                             ? double(sqrtf(c[0] / bbf))
+                             : sqrt_ratio(rr, bb > 0 ? bb : 1.0);
+      const bool ok = rel <= a.rtol || rr == 0.0, give_up = !ok && outer >= kMaxOuter, go = !ok && !give_up;
+      s_go = go ? 1 : 0;
+      if (rank == 0) {
+        if (give_up) atomicOr(a.status, PIC_ST_NOCONV);
+        a.fe[0] = 0.5 * sq_join(c + 3);
+        ps->rr64 = rr;
+        ps->rr = rr;
+        ps->rr0 = rr;
+        ps->rel = rel;
+        if (first_check && outer == 1) ps->rel_first = rel;   // the FFT solve reports the first corrected residual
+        ps->outer_done = ok ? 1 : 0;
+        ps->go = 0;
+        ps->inner_done = go ? 0 : 1;
+        ps->inner_iters = 0;
+        ps->outer_iters = outer;
+        ps->total_iters = total;
+        if (!go) {
+          ps->n_solves += 1;
+          ps->sum_outer += outer;
+          ps->sum_total += total;
+        }
+      }
+    }
+    __syncthreads();
+    if (!s_go) return;
+    for (int q0 = rank; q0 < f.nblk[0] + f.nblk[1]; q0 += ncta) {
+      __syncthreads();
+      box_stage(f, q0, sm);
+      __syncthreads();
+      box_modes(f, q0, sm);
+    }
+    cluster_sync();
+    if (f.slot) {
+      if (rank == 0) box_interface(f, sm);
+      cluster_sync();
+    }
+    box_add_rows(f, sm, rank, ncta);
+    ++outer;
+    ++total;
+    cluster_sync();
   }
 }
 
@@ -1493,6 +1618,13 @@ void (*resid_kernel(const pic_ctx *c))(FineArgs) {
   return c->singular ? k_resid<MODE, true> : k_resid<MODE, false>;
 }
 
+// (the closing kernel of c->box.tail)
+void (*tail_kernel(const pic_ctx *c))(FineArgs, BoxArgs, int) {
+  return c->singular ? k_box_tail<true> : k_box_tail<false>;
+}
+
+bool closing_cluster(const pic_ctx *c) { return c->box.tail != 0; }
+
 // one solve of A e = r by the direct or the transform solver, added to the potential
 void launch_one_pass(pic_ctx *c) {
   if (c->fp.enabled) fast_poisson_launch(c, c->d_r32, c->d_phi, c->d_ps);
@@ -1895,6 +2027,42 @@ cudaError_t poisson_setup(pic_ctx *c) {
   return cudaGetLastError();
 }
 
+// the closing cluster: 16 CTAs where the device takes clusters of that size
+constexpr int kTailCtas = 16;
+
+cudaError_t box_tail_setup(pic_ctx *c) {
+  BoxPoisson &p = c->box;
+  const int nn = c->g.nxn * c->g.nyn;
+  p.tail = nn <= kTailNodes ? 1 : 0;
+  if (!p.tail) return cudaSuccess;
+  p.tail_smem = std::max(p.solve_smem, size_t(p.b[0].n) * 8 * sizeof(float));
+  if (p.slot) p.tail_smem = std::max(p.tail_smem, size_t(p.b[1].n) * 8 * sizeof(float));
+  p.cluster = 0;
+  for (auto k : {k_box_tail<false>, k_box_tail<true>}) {
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kCoarseSmemMax));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+  }
+  // the largest cluster the device takes
+  for (int n = kTailCtas; n >= 2 && !p.cluster; n /= 2) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(unsigned(n));
+    cfg.blockDim = dim3(kBoxThreads);
+    cfg.dynamicSmemBytes = p.tail_smem;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = unsigned(n);
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    int fit = 0;
+    if (cudaOccupancyMaxActiveClusters(&fit, tail_kernel(c), &cfg) == cudaSuccess && fit > 0) p.cluster = n;
+  }
+  cudaGetLastError();
+  if (!p.cluster) p.tail = 0;
+  return cudaSuccess;
+}
+
 bool rho_in_solve(const pic_ctx *c) {
   return one_pass_solver(c) && c->cfg.warm_start == 1 && !c->singular;
 }
@@ -2084,6 +2252,9 @@ cudaError_t add_cond(cudaGraph_t g, const std::vector<cudaGraphNode_t> &deps,
 // tolerance takes one correction it does not need) and only further passes
 // are conditional (the direct solve adds its correction to phi itself):
 //   [phi reset] -> init -> resid -> solve -> resid -> WHILE(go) { solve -> resid }
+// or, on grids small enough, the transform solve ends in a cluster that checks and
+// repeats by itself:
+//   [phi reset] -> init -> resid -> solve -> k_box_tail
 cudaError_t poisson_capture(pic_ctx *c, cudaGraph_t top, std::vector<cudaGraphNode_t> &deps) {
   cudaStream_t s = c->stream;
   FineArgs a = fine_args(c);
@@ -2091,14 +2262,15 @@ cudaError_t poisson_capture(pic_ctx *c, cudaGraph_t top, std::vector<cudaGraphNo
   const int nb = c->red.nblocks;
   const bool direct = one_pass_solver(c);
   cudaGraphConditionalHandle h[4];
-  const int nh = direct ? 1 : 4;
+  const bool tail = closing_cluster(c);
+  const int nh = direct ? (tail ? 0 : 1) : 4;
   for (int k = 0; k < nh; ++k) {
     cudaError_t e = cudaGraphConditionalHandleCreate(&h[k], top, (k == 0 && !direct) ? 1u : 0u,
                                                      cudaGraphCondAssignDefault);
     if (e != cudaSuccess) return note(e, "cudaGraphConditionalHandleCreate");
   }
   a.graph = 1;
-  a.h_outer = h[0];
+  a.h_outer = tail ? 0 : h[0];
   a.h_if_outer = direct ? 0 : h[1];
   a.h_inner = direct ? 0 : h[2];
   a.h_if_inner = direct ? 0 : h[3];
@@ -2116,7 +2288,8 @@ cudaError_t poisson_capture(pic_ctx *c, cudaGraph_t top, std::vector<cudaGraphNo
   if (direct) {
     // the first pass always corrects: the direct solve's leaves ||b||^2 to the
     // second, the transform solve's forms the norms of the guess
-    const bool fp = c->fp.enabled != 0;
+    // (as does the direct solve's before a closing kernel, which needs ||b||)
+    const bool fp = c->fp.enabled && !tail;
     if (rho_in_solve(c)) {   // and forms rho, opening the step's solve
       FineArgs r = a;
       r.advance_step = 1;
@@ -2124,6 +2297,12 @@ cudaError_t poisson_capture(pic_ctx *c, cudaGraph_t top, std::vector<cudaGraphNo
       launch(fp ? k_resid<kFirst, false, true> : k_resid<kOpen, false, true>, nb, kThreads, 0, s, r);
     } else {
       launch(fp ? resid_kernel<kFirst>(c) : resid_kernel<kOpen>(c), nb, kThreads, 0, s, a);
+    }
+    if (tail) {
+      launch_one_pass(c);
+      launch_cluster(tail_kernel(c), c->box.cluster, kBoxThreads, c->box.tail_smem, s, a,
+                     box_args(c, c->d_r32, c->d_phi, c->d_ps), c->fp.enabled);
+      return cap_end(s, deps);
     }
     launch_one_pass(c);
     a.bb_from_part = fp ? 1 : 0;
@@ -2174,6 +2353,8 @@ int64_t poisson_kernel_count(pic_ctx *c, int64_t S, int64_t O, int64_t I) {
   // final resid, and unless the density kernel opens the solve: guess and init
   int64_t per_solve = 1 + (c->cfg.warm_start != 1 ? 2 : 0);
   if (c->cfg.warm_start == 3) per_solve += 2 + unet_forward_kernels();   // absmax, input, network
+  if (closing_cluster(c))   // opening pass, solve, closing kernel (further passes are its own)
+    return S * (per_solve + 1 + (c->fp.enabled ? c->fp.kernels : 2));
   if (one_pass_solver(c))   // per pass: resid, solve (which corrects phi)
     return S * per_solve + O * ((c->fp.enabled ? c->fp.kernels : 2) + 1);
   // a V-cycle with w = A z and the inner products: fused into its last kernel unless lc = 0
