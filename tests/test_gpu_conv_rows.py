@@ -48,3 +48,47 @@ def test_row_kernel_matches_oracle(case):
     assert np.all(np.abs(got - ref) <= 2.0 ** -8 * np.abs(ref) + 1e-3 * np.abs(ref).max())
     rest = np.delete(out, np.s_[out_off:out_off + cout], axis=3)
     assert np.all(rest == 7.0)   # channels outside the output slice are untouched
+
+
+@pytest.mark.parametrize("W, cin, cout", [(40, 64, 64), (9, 32, 256), (200, 16, 32)])
+def test_store_width_changes_no_result(W, cin, cout):
+    # the tile kernel stores 16 channels in one piece where they are 32-byte
+    # aligned (offset 0) and in two where not (offset 8): the same bits
+    import paper_1610_03918_gb300 as pg
+    rng = np.random.default_rng(W + cin)
+    x = bf16_round(rng.standard_normal((2, 13, W, cin)))
+    Wt = bf16_round(rng.standard_normal((cout, 3, 3, cin)) * 0.1)
+    bias = rng.standard_normal(cout) * 0.1
+    wide, st = run_conv(pg, 0, x, 0, cin, Wt, bias, True, cout, 0)
+    assert st == pg.PIC_OK
+    for cs, off in ((cout + 8, 8), (cout + 8, 0), (cout + 16, 8)):
+        out, st = run_conv(pg, 0, x, 0, cin, Wt, bias, True, cs, off)
+        assert st == pg.PIC_OK
+        assert np.array_equal(out[..., off:off + cout], wide)
+        assert np.all(np.delete(out, np.s_[off:off + cout], axis=3) == 7.0)
+
+
+@pytest.mark.parametrize("H, W, cin, cout", [(5, 24, 64, 32), (3, 130, 128, 64), (4, 64, 256, 128)])
+def test_upconv_store_width_changes_no_result(H, W, cin, cout):
+    import ctypes
+    import torch
+    import paper_1610_03918_gb300 as pg
+    f = pg.load_library().pic_upconv_bf16
+    f.argtypes = [ctypes.c_int32] * 4 + [ctypes.c_void_p, ctypes.c_int32] + [ctypes.c_void_p] * 3 \
+        + [ctypes.c_int32] * 3 + [ctypes.c_void_p]
+    g = torch.Generator(device="cuda").manual_seed(H + W)
+    x = torch.randn((2, H, W, cin), generator=g, device="cuda").bfloat16()
+    w = torch.randn((2, 2, cin, cout), generator=g, device="cuda")
+    b = torch.randn((cout,), generator=g, device="cuda")
+    outs = []
+    for cs, off in ((cout, 0), (2 * cout, cout), (cout + 8, 8)):
+        out = torch.full((2, 2 * H, 2 * W, cs), 7.0, device="cuda").bfloat16()
+        assert f(0, 2, H, W, x.data_ptr(), cin, w.data_ptr(), b.data_ptr(), out.data_ptr(), cs, off, cout,
+                 torch.cuda.current_stream().cuda_stream) == pg.PIC_OK
+        outs.append(out[..., off:off + cout].clone())
+        out[..., off:off + cout] = 7.0
+        assert bool((out == 7.0).all())
+    ref = torch.einsum("bhwi,acio->bhawco", x.double(), w.bfloat16().double()).reshape(2, 2 * H, 2 * W, cout) + b
+    # FP32 sums of cin products and one rounding to BF16
+    assert float((outs[0].double() - ref).norm() / ref.norm()) <= 4e-3
+    assert all(torch.equal(o, outs[0]) for o in outs[1:])
