@@ -405,7 +405,7 @@ struct pic_ctx {
   pic_hit *d_hits;
   unsigned long long *d_nhits;
   uint32_t *d_status;
-  uint32_t *h_status;             // pinned
+  uint32_t *h_status;             // pinned mirror
 
   // staging for pic_load / diag
   double *d_stage;

@@ -20,11 +20,13 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
 #include <new>
 #include <string>
+#include <thread>
 #include <vector>
 
 #include "internal.cuh"
@@ -1315,8 +1317,51 @@ pic_status pic_unet_load(pic_unet *u, const char *path) {
 }  // extern "C"
 
 namespace {
-// error word of pic_conv3x3_bf16's tcgen05 kernel (a bounded wait gave up)
-__device__ int g_conv_err;
+// Error words of the layer entry points' tcgen05 kernels (a bounded wait gave
+// up).  A kernel writes its word only then, so the words stay zero and need no
+// clearing before a launch; they are managed memory, which the host reads in
+// place once the stream has ended: against a device word that is cleared
+// before and copied back after the kernel, a call of a 10 us kernel takes 19.2
+// instead of 28.6 us.  Each call in progress has a word of its own.
+constexpr int kErrWords = 64;
+__managed__ int g_layer_err[kErrWords];
+std::atomic<uint64_t> g_err_taken{0};
+
+class ErrWord {
+ public:
+  ErrWord() {
+    uint64_t t = g_err_taken.load(std::memory_order_relaxed);
+    for (;;) {
+      if (t == ~uint64_t(0)) {   // 64 calls in progress: until one of them returns
+        std::this_thread::yield();
+        t = g_err_taken.load(std::memory_order_relaxed);
+        continue;
+      }
+      k_ = __builtin_ctzll(~t);
+      if (g_err_taken.compare_exchange_weak(t, t | (uint64_t(1) << k_), std::memory_order_acquire)) return;
+    }
+  }
+  ~ErrWord() { g_err_taken.fetch_and(~(uint64_t(1) << k_), std::memory_order_release); }
+  ErrWord(const ErrWord &) = delete;
+  ErrWord &operator=(const ErrWord &) = delete;
+  int *device() const {
+    int *p = nullptr;
+    return cudaGetSymbolAddress((void **)&p, g_layer_err) == cudaSuccess ? p + k_ : nullptr;
+  }
+  // after the stream's synchronisation: the call's status (1 producer, 2 MMA,
+  // 3 epilogue wait gave up, for pic_last_error); the word is zero again
+  pic_status read(const char *what) const {
+    volatile int *w = g_layer_err + k_;
+    const int e = *w;
+    if (!e) return PIC_OK;
+    *w = 0;
+    picgb::note(cudaErrorTimeout, (std::string("tcgen05 ") + what + " wait " + std::to_string(e)).c_str());
+    return PIC_ETIMEOUT;
+  }
+
+ private:
+  int k_ = 0;
+};
 }  // namespace
 
 extern "C" {
@@ -1331,10 +1376,10 @@ pic_status pic_conv3x3_bf16(int32_t impl, int32_t B, int32_t H, int32_t W, const
   const bf16 *bin = static_cast<const bf16 *>(in), *bw = static_cast<const bf16 *>(w);
   bf16 *bout = static_cast<bf16 *>(out);
   if (impl == 0) {
-    int *err = nullptr;
-    if (cudaGetSymbolAddress((void **)&err, g_conv_err) != cudaSuccess) return PIC_ECUDA;
+    const ErrWord word;
+    int *err = word.device();
+    if (!err) return PIC_ECUDA;
     if (!picgb::conv3x3_tc_supported(cin, cout, in_cs, in_off, out_cs, out_off, W)) return PIC_EINVAL;
-    if (cudaMemsetAsync(err, 0, 4, s) != cudaSuccess) return PIC_ECUDA;
     picgb::ConvTC c;
     c.in = bin;
     c.in_cs = in_cs;
@@ -1352,14 +1397,7 @@ pic_status pic_conv3x3_bf16(int32_t impl, int32_t B, int32_t H, int32_t W, const
     c.relu = relu ? 1 : 0;
     c.err = err;
     if (picgb::conv3x3_tc(c, s) != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) return PIC_ECUDA;
-    int e = 0;
-    if (cudaMemcpy(&e, err, 4, cudaMemcpyDeviceToHost) != cudaSuccess) return PIC_ECUDA;
-    if (e) {
-      // the wait that gave up (1 producer, 2 MMA, 3 epilogue), for pic_last_error
-      picgb::note(cudaErrorTimeout, ("tcgen05 convolution wait " + std::to_string(e)).c_str());
-      return PIC_ETIMEOUT;
-    }
-    return PIC_OK;
+    return word.read("convolution");
   }
   // the mma.sync implicit GEMM: cout 32 (cin 16 or a multiple of 32) or a multiple of 64
   ConvArgs a;
@@ -1405,9 +1443,9 @@ pic_status pic_conv3x3_wgrad_bf16(int32_t impl, int32_t B, int32_t H, int32_t W,
     return PIC_OK;
   }
   if (!picgb::conv_wgrad_tc_supported(cin, cout, in_cs, in_off, dw)) return PIC_EINVAL;
-  int *err = nullptr;
-  if (cudaGetSymbolAddress((void **)&err, g_conv_err) != cudaSuccess) return PIC_ECUDA;
-  if (cudaMemsetAsync(err, 0, 4, s) != cudaSuccess) return PIC_ECUDA;
+  const ErrWord word;
+  int *err = word.device();
+  if (!err) return PIC_ECUDA;
   picgb::WgradTC g;
   g.dpre = bd;
   g.in = bi;
@@ -1421,13 +1459,7 @@ pic_status pic_conv3x3_wgrad_bf16(int32_t impl, int32_t B, int32_t H, int32_t W,
   g.W = W;
   g.err = err;
   if (picgb::conv_wgrad_tc(g, s) != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) return PIC_ECUDA;
-  int e = 0;
-  if (cudaMemcpy(&e, err, 4, cudaMemcpyDeviceToHost) != cudaSuccess) return PIC_ECUDA;
-  if (e) {
-    picgb::note(cudaErrorTimeout, ("tcgen05 weight gradient wait " + std::to_string(e)).c_str());
-    return PIC_ETIMEOUT;
-  }
-  return PIC_OK;
+  return word.read("weight gradient");
 }
 
 namespace {
@@ -1515,8 +1547,9 @@ pic_status pic_upconv_bf16(int32_t impl, int32_t B, int32_t H, int32_t W, const 
   const int total = 4 * cout, step = total > 256 ? 256 : total;
   if (total % step || cout % 16 || !picgb::conv3x3_tc_supported(cin, step, cin, 0, out_cs, out_off, W))
     return PIC_EINVAL;
-  int *err = nullptr;
-  if (cudaGetSymbolAddress((void **)&err, g_conv_err) != cudaSuccess) return PIC_ECUDA;
+  const ErrWord word;
+  int *err = word.device();
+  if (!err) return PIC_ECUDA;
   bf16 *wt = nullptr;
   if (cudaMalloc(&wt, size_t(total) * cin * 2) != cudaSuccess) return PIC_ENOMEM;
   k_upw_to_bf16<<<gridn(4LL * cout * cin), 256, 0, s>>>(w, wt, cin, cout);
@@ -1536,23 +1569,15 @@ pic_status pic_upconv_bf16(int32_t impl, int32_t B, int32_t H, int32_t W, const 
   c.relu = 0;
   c.err = err;
   c.up_cout = cout;
-  pic_status st = (cudaGetLastError() == cudaSuccess && cudaMemsetAsync(err, 0, 4, s) == cudaSuccess) ? PIC_OK
-                                                                                                   : PIC_ECUDA;
+  pic_status st = cudaGetLastError() == cudaSuccess ? PIC_OK : PIC_ECUDA;
   for (int n0 = 0; st == PIC_OK && n0 < total; n0 += step) {
     c.cout = step;
     c.n_base = n0;
     if (picgb::conv3x3_tc(c, s) != cudaSuccess) st = PIC_ECUDA;
   }
-  if (st == PIC_OK && cudaStreamSynchronize(s) != cudaSuccess) st = PIC_ECUDA;
-  int e = 0;
-  if (st == PIC_OK && cudaMemcpy(&e, err, 4, cudaMemcpyDeviceToHost) != cudaSuccess) st = PIC_ECUDA;
-  cudaStreamSynchronize(s);
+  if (cudaStreamSynchronize(s) != cudaSuccess && st == PIC_OK) st = PIC_ECUDA;
   cudaFree(wt);
-  if (st == PIC_OK && e) {
-    picgb::note(cudaErrorTimeout, ("tcgen05 convolution wait " + std::to_string(e)).c_str());
-    st = PIC_ETIMEOUT;
-  }
-  return st;
+  return st == PIC_OK ? word.read("convolution") : st;
 }
 
 pic_status pic_upconv_wgrad_bf16(int32_t impl, int32_t B, int32_t H, int32_t W, const void *in, int32_t cin,
@@ -1581,9 +1606,9 @@ pic_status pic_upconv_wgrad_bf16(int32_t impl, int32_t B, int32_t H, int32_t W, 
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return PIC_ECUDA;
-  int *err = nullptr;
-  if (cudaGetSymbolAddress((void **)&err, g_conv_err) != cudaSuccess) return PIC_ECUDA;
-  if (cudaMemsetAsync(err, 0, 4, s) != cudaSuccess) return PIC_ECUDA;
+  const ErrWord word;
+  int *err = word.device();
+  if (!err) return PIC_ECUDA;
   picgb::UpWgradTC g;
   g.in = bi;
   g.g = bg;
@@ -1601,13 +1626,7 @@ pic_status pic_upconv_wgrad_bf16(int32_t impl, int32_t B, int32_t H, int32_t W, 
   k_colsum<<<int(std::min<long long>((np + ppb - 1) / ppb, 8LL * sms)), 256, 0, s>>>(bg, gout_cs, gout_off, cout,
                                                                                    np, db);
   if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) return PIC_ECUDA;
-  int e = 0;
-  if (cudaMemcpy(&e, err, 4, cudaMemcpyDeviceToHost) != cudaSuccess) return PIC_ECUDA;
-  if (e) {
-    picgb::note(cudaErrorTimeout, ("tcgen05 weight gradient wait " + std::to_string(e)).c_str());
-    return PIC_ETIMEOUT;
-  }
-  return PIC_OK;
+  return word.read("weight gradient");
 }
 
 pic_status pic_upconv_back_bf16(int32_t impl, int32_t B, int32_t H, int32_t W, const void *gout,
@@ -1626,8 +1645,9 @@ pic_status pic_upconv_back_bf16(int32_t impl, int32_t B, int32_t H, int32_t W, c
     return PIC_OK;
   }
   if (!picgb::conv3x3_tc_supported(cout, cin, gout_cs, gout_off, cin, 0, W)) return PIC_EINVAL;
-  int *err = nullptr;
-  if (cudaGetSymbolAddress((void **)&err, g_conv_err) != cudaSuccess) return PIC_ECUDA;
+  const ErrWord word;
+  int *err = word.device();
+  if (!err) return PIC_ECUDA;
   const long long nw = 4LL * cin * cout;
   bf16 *wb = nullptr;
   if (cudaMalloc(&wb, size_t(nw) * 2) != cudaSuccess) return PIC_ENOMEM;
@@ -1649,17 +1669,11 @@ pic_status pic_upconv_back_bf16(int32_t impl, int32_t B, int32_t H, int32_t W, c
   c.err = err;
   k_to_bf16<<<gridn(nw), 256, 0, s>>>(w, wb, nw);
   pic_status st = PIC_OK;
-  if (cudaGetLastError() != cudaSuccess || cudaMemsetAsync(err, 0, 4, s) != cudaSuccess ||
-      picgb::conv_upback_tc(c, s) != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess)
+  if (cudaGetLastError() != cudaSuccess || picgb::conv_upback_tc(c, s) != cudaSuccess ||
+      cudaStreamSynchronize(s) != cudaSuccess)
     st = PIC_ECUDA;
-  int e = 0;
-  if (st == PIC_OK && cudaMemcpy(&e, err, 4, cudaMemcpyDeviceToHost) != cudaSuccess) st = PIC_ECUDA;
   cudaFree(wb);
-  if (st == PIC_OK && e) {
-    picgb::note(cudaErrorTimeout, ("tcgen05 convolution wait " + std::to_string(e)).c_str());
-    st = PIC_ETIMEOUT;
-  }
-  return st;
+  return st == PIC_OK ? word.read("convolution") : st;
 }
 
 pic_status pic_unet_set_conv_impl(pic_unet *u, int32_t impl) {
