@@ -303,7 +303,7 @@ pic_status step_kernels(pic_ctx *c, bool sorting, cudaEvent_t *ev) {
   cudaEventRecord(ev[0], c->stream);
   if (sorting) {
     if ((st = check(launch_sort(c))) != PIC_OK) return st;
-    c->launches += 4;
+    c->launches += 3;
   }
   cudaEventRecord(ev[1], c->stream);
   if ((st = check(launch_particles(c, 0, 1.f, nullptr))) != PIC_OK) return st;
@@ -818,7 +818,7 @@ pic_status pic_init(const pic_config *cfg, pic_ctx **out) {
   c->d_nchunks = (int32_t *)A(4);
   c->d_nslots = (int64_t *)A(4 * 8);
   c->d_ke_part = (double *)A(size_t(c->max_chunks) * 8);
-  c->d_work = (unsigned int *)A(2 * sizeof(unsigned int));
+  c->d_work = (unsigned int *)A(3 * sizeof(unsigned int));
   c->d_step = (int32_t *)A(4);
   c->d_walls = (unsigned long long *)A(2 * PIC_NWALLS * 8);
   c->d_bottom = (unsigned long long *)A(2 * size_t(g.ny) * 8);
@@ -912,7 +912,7 @@ pic_status pic_init(const pic_config *cfg, pic_ctx **out) {
   cudaMemsetAsync(c->d_tile_count, 0, 2 * size_t(ntiles) * 4, c->stream);
   cudaMemsetAsync(c->d_tile_cursor, 0, 2 * size_t(ntiles) * 4, c->stream);
   cudaMemsetAsync(c->d_nchunks, 0, 4, c->stream);
-  cudaMemsetAsync(c->d_work, 0, 2 * sizeof(unsigned int), c->stream);
+  cudaMemsetAsync(c->d_work, 0, 3 * sizeof(unsigned int), c->stream);
   cudaMemsetAsync(c->d_nslots, 0, 32, c->stream);
   cudaMemsetAsync(c->d_step, 0, 4, c->stream);
   cudaMemsetAsync(c->d_walls, 0, 2 * PIC_NWALLS * 8, c->stream);
@@ -1125,7 +1125,7 @@ pic_status pic_step(pic_ctx *c, int32_t nsteps) {
             return PIC_ECUDA;
       }
       // particle kernel, [sort], [density]; the solve's kernels are counted from its totals
-      c->launches += (sorting ? 4 : 0) + (rho_in_solve(c) ? 1 : 2) +
+      c->launches += (sorting ? 3 : 0) + (rho_in_solve(c) ? 1 : 2) +
                      (c->cfg.phi_rf_amp != 0.0 && (c->n_rf_dir || c->n_rf_lift) ? 1 : 0);
       if (note(cudaGraphLaunch(c->gexec[ws][ev], c->stream), "step graph launch") != cudaSuccess)
         return PIC_ECUDA;
@@ -1213,14 +1213,14 @@ pic_status pic_step_particles(pic_ctx *c) {
       c->cur[0] ^= 1;
       c->cur[1] ^= 1;
     }
-    c->launches += (sorting ? 4 : 0) + 1;
+    c->launches += (sorting ? 3 : 0) + 1;
   } else {
     if (sorting && (st = check(launch_sort(c))) != PIC_OK) return st;
     if ((st = check(launch_particles(c, 0, 1.f, nullptr))) != PIC_OK) return st;
     if (cudaMemcpyAsync(c->d_acc + 2 * nn, c->d_bottom, 2 * size_t(c->g.ny) * 8, cudaMemcpyDeviceToDevice,
                         c->stream) != cudaSuccess)
       return PIC_ECUDA;
-    c->launches += (sorting ? 4 : 0) + 1;
+    c->launches += (sorting ? 3 : 0) + 1;
   }
   if (sorting) {
     c->steps_since_sort = 0;

@@ -396,7 +396,7 @@ struct pic_ctx {
   int max_tiles;               // tiles of the smallest tile shape (array sizes)
   int64_t *d_nslots;           // [4]: slots in use per species; [2..3] staged by the sort
   double *d_ke_part;           // [max_chunks]
-  unsigned int *d_work;        // [2] the particle kernel's chunk dispenser
+  unsigned int *d_work;        // [3] the particle kernel's chunk dispenser, the scatter's CTAs done
   int32_t *d_step;
 
   // tallies and status
