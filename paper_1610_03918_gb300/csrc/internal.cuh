@@ -36,6 +36,7 @@ constexpr TileVariant kTileVariants[kNumTileVariants] = {
 };
 constexpr int kMinTileLog2 = 4;  // the smallest tile (16 x 16) sizes the tile arrays
 constexpr int kChunk = 4092;     // particles per work item (multiple of 4, <= 4095)
+constexpr int kRunSteps = 8;     // most steps of one graph launch
 constexpr int kMinChunk = 512;   // one pass of the particle kernel's smaller CTA
 constexpr int kMaxCtasPerSm = 16;
 constexpr int kWalkLimit = 16;   // face crossings followed per move
@@ -416,6 +417,10 @@ struct pic_ctx {
   // captured step graphs [with the tile sort][with phase event nodes]
   cudaGraph_t graph[2][2];
   cudaGraphExec_t gexec[2][2];
+  // graphs of several steps [first step sorts][steps], and which were asked for once
+  cudaGraph_t graph_run[2][picgb::kRunSteps + 1];
+  cudaGraphExec_t gexec_run[2][picgb::kRunSteps + 1];
+  uint8_t run_asked[2][picgb::kRunSteps + 1];
   // decomposed run: particle phase without / with the sort, field phase
   cudaGraph_t graph_dp[3];
   cudaGraphExec_t gexec_dp[3];
@@ -481,6 +486,10 @@ cudaError_t launch_rho(pic_ctx *c, int advance_step, int init_solve = 0);
 bool rho_in_solve(const pic_ctx *c);
 pic_status poisson_solve(pic_ctx *c, bool zero_guess);
 cudaError_t poisson_capture(pic_ctx *c, cudaGraph_t top, std::vector<cudaGraphNode_t> &deps);
+// Grids whose solve ends in a cluster that checks and repeats by itself, and
+// that solve, into the capture in progress (no conditional nodes).
+bool closing_cluster(const pic_ctx *c);
+cudaError_t launch_closed_solve(pic_ctx *c);
 int64_t poisson_kernel_count(pic_ctx *c, int64_t S, int64_t O, int64_t I);
 pic_status ensure_vacuum_potential(pic_ctx *c);
 pic_status learned_input(pic_ctx *c, int hpad, float *x, double *scale);

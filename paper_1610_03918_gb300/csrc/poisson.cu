@@ -1623,7 +1623,6 @@ void (*tail_kernel(const pic_ctx *c))(FineArgs, BoxArgs, int) {
   return c->singular ? k_box_tail<true> : k_box_tail<false>;
 }
 
-bool closing_cluster(const pic_ctx *c) { return c->box.tail != 0; }
 
 // one solve of A e = r by the direct or the transform solver, added to the potential
 void launch_one_pass(pic_ctx *c) {
@@ -2242,6 +2241,59 @@ cudaError_t add_cond(cudaGraph_t g, const std::vector<cudaGraphNode_t> &deps,
 
 }  // namespace
 
+// The initial guess of a captured solve.
+static cudaError_t launch_guess(pic_ctx *c, const FineArgs &a) {
+  cudaStream_t s = c->stream;
+  const int nb = c->red.nblocks;
+  if (c->cfg.warm_start == 0) launch(k_phi_reset, nb, kThreads, 0, s, a);
+  if (c->cfg.warm_start == 2) launch(k_extrapolate, nb, kThreads, 0, s, a);
+  if (c->cfg.warm_start == 3) {
+    const cudaError_t e = launch_learned_guess(c);
+    if (e != cudaSuccess) return e;
+  }
+  if (c->cfg.warm_start == 4)
+    launch(k_guess_lift, nb, kThreads, 0, s, c->d_phi, c->d_phiL, c->d_nodeflags, c->g.nxn * c->g.nyn);
+  // (with the previous step's potential as the guess the density kernel just
+  // before opened the solve)
+  if (c->cfg.warm_start != 1) launch(k_outer_init, 1, 1, 0, s, c->d_ps);
+  return cudaSuccess;
+}
+
+// The first residual of a one-pass solve, which always corrects: the direct
+// solve's leaves ||b||^2 to the second (bb_later), the transform solve's forms
+// the norms of the guess, as does the direct solve's before a closing kernel,
+// which needs ||b||.
+static void launch_first_pass(pic_ctx *c, const FineArgs &a, bool bb_later) {
+  const int nb = c->red.nblocks;
+  if (rho_in_solve(c)) {   // and forms rho, opening the step's solve
+    FineArgs r = a;
+    r.advance_step = 1;
+    r.init_solve = 1;
+    launch(bb_later ? k_resid<kFirst, false, true> : k_resid<kOpen, false, true>, nb, kThreads, 0, c->stream, r);
+  } else {
+    launch(bb_later ? resid_kernel<kFirst>(c) : resid_kernel<kOpen>(c), nb, kThreads, 0, c->stream, a);
+  }
+}
+
+
+bool closing_cluster(const pic_ctx *c) { return c->box.tail != 0; }
+
+// The solve of a grid whose closing cluster checks and repeats by itself, into
+// the capture in progress:
+//   [phi reset] -> init -> resid -> solve -> k_box_tail
+cudaError_t launch_closed_solve(pic_ctx *c) {
+  FineArgs a = fine_args(c);
+  a.graph = 1;
+  a.h_outer = a.h_if_outer = a.h_inner = a.h_if_inner = 0;
+  const cudaError_t e = launch_guess(c, a);
+  if (e != cudaSuccess) return e;
+  launch_first_pass(c, a, false);
+  launch_one_pass(c);
+  launch_cluster(tail_kernel(c), c->box.cluster, kBoxThreads, c->box.tail_smem, c->stream, a,
+                 box_args(c, c->d_r32, c->d_phi, c->d_ps), c->fp.enabled);
+  return cudaGetLastError();
+}
+
 // Appends the solve to graph `top` after the nodes in `deps`; on return
 // `deps` holds the solve's last node.  With the multigrid inner solve:
 //   [phi reset] -> init -> WHILE(outer) { resid -> IF(go) { V-cycle ->
@@ -2252,60 +2304,40 @@ cudaError_t add_cond(cudaGraph_t g, const std::vector<cudaGraphNode_t> &deps,
 // tolerance takes one correction it does not need) and only further passes
 // are conditional (the direct solve adds its correction to phi itself):
 //   [phi reset] -> init -> resid -> solve -> resid -> WHILE(go) { solve -> resid }
-// or, on grids small enough, the transform solve ends in a cluster that checks and
-// repeats by itself:
-//   [phi reset] -> init -> resid -> solve -> k_box_tail
+// Grids small enough end in a cluster that checks and repeats by itself
+// (launch_closed_solve): no conditional node.
 cudaError_t poisson_capture(pic_ctx *c, cudaGraph_t top, std::vector<cudaGraphNode_t> &deps) {
   cudaStream_t s = c->stream;
+  if (closing_cluster(c)) {
+    cudaError_t e = cap_begin(s, top, deps);
+    if (e == cudaSuccess) e = launch_closed_solve(c);
+    const cudaError_t e2 = cap_end(s, deps);
+    return note(e == cudaSuccess ? e2 : e, "capture: solve");
+  }
   FineArgs a = fine_args(c);
   const MGArgs m = mg_args(c);
   const int nb = c->red.nblocks;
   const bool direct = one_pass_solver(c);
   cudaGraphConditionalHandle h[4];
-  const bool tail = closing_cluster(c);
-  const int nh = direct ? (tail ? 0 : 1) : 4;
+  const int nh = direct ? 1 : 4;
   for (int k = 0; k < nh; ++k) {
     cudaError_t e = cudaGraphConditionalHandleCreate(&h[k], top, (k == 0 && !direct) ? 1u : 0u,
                                                      cudaGraphCondAssignDefault);
     if (e != cudaSuccess) return note(e, "cudaGraphConditionalHandleCreate");
   }
   a.graph = 1;
-  a.h_outer = tail ? 0 : h[0];
+  a.h_outer = h[0];
   a.h_if_outer = direct ? 0 : h[1];
   a.h_inner = direct ? 0 : h[2];
   a.h_if_inner = direct ? 0 : h[3];
   cudaError_t e;
 #define CK(x) do { if ((e = (x)) != cudaSuccess) { note(e, #x); return e; } } while (0)
   CK(cap_begin(s, top, deps));
-  if (c->cfg.warm_start == 0) launch(k_phi_reset, nb, kThreads, 0, s, a);
-  if (c->cfg.warm_start == 2) launch(k_extrapolate, nb, kThreads, 0, s, a);
-  if (c->cfg.warm_start == 3) CK(launch_learned_guess(c));
-  if (c->cfg.warm_start == 4)
-    launch(k_guess_lift, nb, kThreads, 0, s, c->d_phi, c->d_phiL, c->d_nodeflags, c->g.nxn * c->g.nyn);
-  // (with the previous step's potential as the guess the density kernel just
-  // before opened the solve)
-  if (c->cfg.warm_start != 1) launch(k_outer_init, 1, 1, 0, s, c->d_ps);
+  CK(launch_guess(c, a));
   if (direct) {
-    // the first pass always corrects: the direct solve's leaves ||b||^2 to the
-    // second, the transform solve's forms the norms of the guess
-    // (as does the direct solve's before a closing kernel, which needs ||b||)
-    const bool fp = c->fp.enabled && !tail;
-    if (rho_in_solve(c)) {   // and forms rho, opening the step's solve
-      FineArgs r = a;
-      r.advance_step = 1;
-      r.init_solve = 1;
-      launch(fp ? k_resid<kFirst, false, true> : k_resid<kOpen, false, true>, nb, kThreads, 0, s, r);
-    } else {
-      launch(fp ? resid_kernel<kFirst>(c) : resid_kernel<kOpen>(c), nb, kThreads, 0, s, a);
-    }
-    if (tail) {
-      launch_one_pass(c);
-      launch_cluster(tail_kernel(c), c->box.cluster, kBoxThreads, c->box.tail_smem, s, a,
-                     box_args(c, c->d_r32, c->d_phi, c->d_ps), c->fp.enabled);
-      return cap_end(s, deps);
-    }
+    launch_first_pass(c, a, c->fp.enabled);
     launch_one_pass(c);
-    a.bb_from_part = fp ? 1 : 0;
+    a.bb_from_part = c->fp.enabled ? 1 : 0;
     launch(resid_kernel<kFull>(c), nb, kThreads, 0, s, a);
   }
   CK(cap_end(s, deps));
