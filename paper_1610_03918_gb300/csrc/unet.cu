@@ -332,16 +332,29 @@ __global__ void __launch_bounds__(256) k_relu_back(const bf16 *g, int g_cs, int 
   }
 }
 
-// W'[ci][tap][co] = W[co][8 - tap][ci]
-__global__ void k_wflip(const bf16 *w, bf16 *wt, int cout, int cin) {
-  GSTRIDE(i, (long long)cout * 9 * cin) {
-    const int ci = int(i % cin);
-    const int tap = int((i / cin) % 9);
-    const int co = int(i / (9LL * cin));
-    wt[(size_t(ci) * 9 + (8 - tap)) * cout + co] = w[i];
+// W'[ci][tap][co] = W[co][8 - tap][ci] of every layer, a row of the grid each:
+// tiles of 32 x 32 (co, ci) of a tap, turned in shared memory.  A launch per layer
+// that wrote 2 bytes a sector took 57 us a pass, this one 6.4.
+constexpr int kFlips = 13;
+struct FlipArgs {
+  const bf16 *w[kFlips];
+  bf16 *wt[kFlips];
+  int cout[kFlips], cin[kFlips];   // multiples of 32
+};
+__global__ void __launch_bounds__(256) k_wflip(FlipArgs a) {
+  __shared__ bf16 tile[32][34];
+  const int q = blockIdx.y, cout = a.cout[q], cin = a.cin[q], nci = cin / 32;
+  const int tiles = 9 * (cout / 32) * nci, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
+    const int tap = t % 9, b = t / 9, co0 = b / nci * 32, ci0 = b % nci * 32;
+    __syncthreads();
+#pragma unroll
+    for (int k = ty; k < 32; k += 8) tile[k][tx] = a.w[q][(size_t(co0 + k) * 9 + tap) * cin + ci0 + tx];
+    __syncthreads();
+#pragma unroll
+    for (int k = ty; k < 32; k += 8) a.wt[q][(size_t(ci0 + k) * 9 + 8 - tap) * cout + co0 + tx] = tile[tx][k];
   }
 }
-
 
 // transposed 2x2 stride-2 convolution: out (2h x 2w) from in (h x w); W [2][2][ci][co] FP32
 __global__ void k_up_fwd(const bf16 *in, int cin, const float *w, const float *bias, bf16 *out,
@@ -426,8 +439,10 @@ __global__ void __launch_bounds__(256) k_up_back_w(const bf16 *in, int cin, cons
 }
 
 
-// MSE: dy = 2 (y - t) / n, loss partial sums in FP64
-__global__ void k_mse(const float *y, const float *t, float *dy, long long n, double *loss) {
+// MSE: dy = 2 (y - t) / n, loss partial sums in FP64, one atomic per CTA (one
+// per warp, on the one address, made 25 us of 2.1M pixels; now 16.5, the FP64 adds)
+__global__ void __launch_bounds__(256) k_mse(const float *y, const float *t, float *dy, long long n, double *loss) {
+  __shared__ double part[8];
   double s = 0.0;
   GSTRIDE(p, n) {
     const float d = y[p] - t[p];
@@ -435,22 +450,30 @@ __global__ void k_mse(const float *y, const float *t, float *dy, long long n, do
     s += double(d) * double(d);
   }
   for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-  if ((threadIdx.x & 31) == 0) atomicAdd(loss, s / double(n));
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) s += part[w];
+    atomicAdd(loss, s / double(n));
+  }
 }
 
-// head backward: gh[p][c] = dy[p] w[c]; dw[c] += sum_p dy h; db += sum dy
 // backward through the 1x1 head y[p] = b + sum_c w[c] h[p][c]: gh[p][c] = dy[p] w[c],
 // dw[c] += sum_p dy[p] h[p][c], db += sum_p dy[p].  Each thread moves 8 channels
-// (16 bytes) of a pixel and keeps one channel group for the whole loop.
+// (16 bytes) of a pixel and keeps one channel group for the whole loop.  With
+// RELU, gh goes on through the ReLU that made h, 0 where h is not positive, and
+// dbh[c] += sum_p gh[p][c]: what k_relu_back would make of it, without a pass of
+// its own (4 x 1032 x 512: 47.6 + 66.2 us in two, 56.1 in one).
+template <bool RELU>
 __global__ void __launch_bounds__(256) k_head_back(const float *dy, const bf16 *hin, const float *w, bf16 *gh,
-                                                   float *dw, float *db, long long npix) {
+                                                   float *dw, float *db, float *dbh, long long npix) {
   constexpr int G = kC0 / 8, PPB = 256 / G;
   const int grp = threadIdx.x % G;
-  float wk[8], s[8], bs = 0.f;
+  float wk[8], s[8], sh[8], bs = 0.f;
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
     wk[k] = w[8 * grp + k];
-    s[k] = 0.f;
+    s[k] = sh[k] = 0.f;
   }
   for (long long p = blockIdx.x * (long long)PPB + threadIdx.x / G; p < npix; p += (long long)gridDim.x * PPB) {
     const float d = dy[p];
@@ -461,12 +484,25 @@ __global__ void __launch_bounds__(256) k_head_back(const float *dy, const bf16 *
     bf16 *oo = reinterpret_cast<bf16 *>(&ov);
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-      oo[k] = __float2bfloat16(d * wk[k]);
-      s[k] = fmaf(d, __bfloat162float(hh[k]), s[k]);
+      const float h = __bfloat162float(hh[k]);
+      oo[k] = !RELU || h > 0.f ? __float2bfloat16(d * wk[k]) : __float2bfloat16(0.f);
+      s[k] = fmaf(d, h, s[k]);
+      if (RELU) sh[k] += __bfloat162float(oo[k]);
     }
     *reinterpret_cast<uint4 *>(gh + p * kC0 + 8 * grp) = ov;
   }
   __shared__ float red[9][256];
+  if (RELU) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) red[k][threadIdx.x] = sh[k];
+    __syncthreads();
+    if (threadIdx.x < kC0) {
+      float t = 0.f;
+      for (int j = threadIdx.x >> 3; j < 256; j += G) t += red[threadIdx.x & 7][j];
+      atomicAdd(&dbh[threadIdx.x], t);
+    }
+    __syncthreads();
+  }
 #pragma unroll
   for (int k = 0; k < 8; ++k) red[k][threadIdx.x] = s[k];
   red[8][threadIdx.x] = grp == 0 ? bs : 0.f;
@@ -790,10 +826,25 @@ void conv_fwd(pic_unet *u, int ci, const bf16 *in, int in_cs, int in_off, bf16 *
   }
 }
 
+// the flipped weights of all layers but the first (which has no data gradient)
+void flip_weights(pic_unet *u) {
+  FlipArgs a;
+  int n = 0;
+  for (int ci = 0; ci < int(sizeof(u->conv) / sizeof(u->conv[0])); ++ci) {
+    const pic_unet::Conv &c = u->conv[ci];
+    if (ci == E0A) continue;
+    a.w[n] = c.w;
+    a.wt[n] = c.wt;
+    a.cout[n] = c.cout;
+    a.cin[n] = c.cin_c;
+    n += 1;
+  }
+  k_wflip<<<dim3(unsigned(2 * u->num_sms), unsigned(n)), 256, 0, u->stream>>>(a);
+}
+
 // data gradient: gin (cin channels) = conv(dpre, flipped weights)
 void conv_back_data(pic_unet *u, int ci, const bf16 *dpre, bf16 *gin, int gin_cs, int gin_off, int l) {
   const pic_unet::Conv &c = u->conv[ci];
-  k_wflip<<<gridn((long long)c.cout * 9 * c.cin_c), 256, 0, u->stream>>>(c.w, c.wt, c.cout, c.cin_c);
   if (conv_tc(u, dpre, c.cout, 0, c.cout, c.wt, nullptr, gin, gin_cs, gin_off, c.cin_c, l, false)) return;
   ConvArgs a;
   a.in = dpre;
@@ -868,6 +919,14 @@ void conv_back_weights(pic_unet *u, int ci, const bf16 *dpre, const bf16 *in, in
                                                                           c.cout, c.cin_m, c.cin_c);
 }
 
+// the weight gradient and the gradient gin at the input (unless null) of a
+// convolution whose pre-activation gradient is in dpre[l]
+void conv_grads(pic_unet *u, int ci, const bf16 *in, int in_cs, int in_off, bf16 *gin, int gin_cs, int gin_off,
+                int l) {
+  conv_back_weights(u, ci, u->dpre[l], in, in_cs, in_off, l);
+  if (gin) conv_back_data(u, ci, u->dpre[l], gin, gin_cs, gin_off, l);
+}
+
 // backward through relu(conv(in)) given the gradient g at its output;
 // writes the gradient at its input into gin (unless gin is null)
 // gp: the gradient of the average pool that follows y's block (added to g), or null
@@ -885,8 +944,7 @@ void conv_block_back(pic_unet *u, int ci, const bf16 *g, int g_cs, int g_off, co
   else
     k_relu_back<false><<<grid, 256, 0, u->stream>>>(g, g_cs, g_off, y, y_cs, y_off, nullptr, 1, 1, dpre,
                                                     c.cout, np, u->G + c.b_off);
-  conv_back_weights(u, ci, dpre, in, in_cs, in_off, l);
-  if (gin) conv_back_data(u, ci, dpre, gin, gin_cs, gin_off, l);
+  conv_grads(u, ci, in, in_cs, in_off, gin, gin_cs, gin_off, l);
 }
 
 void weights_to_bf16(pic_unet *u) {
@@ -1035,14 +1093,18 @@ void forward(pic_unet *u, const float *x, bool keep_input) {
 void backward(pic_unet *u) {
   const int C3 = kC[3];
   cudaMemsetAsync(u->G, 0, size_t(u->nparam) * 4, u->stream);
-  k_head_back<<<int(std::min<long long>((pix(u, 0) + 63) / 64, 8LL * u->num_sms)), 256, 0, u->stream>>>(
-      u->dy, u->dout[0], u->P + u->head_w, u->gdout[0], u->G + u->head_w, u->G + u->head_b, pix(u, 0));
+  flip_weights(u);
+  // the head, and through the ReLU of the layer before it
+  k_head_back<true><<<int(std::min<long long>((pix(u, 0) + 63) / 64, 8LL * u->num_sms)), 256, 0, u->stream>>>(
+      u->dy, u->dout[0], u->P + u->head_w, u->dpre[0], u->G + u->head_w, u->G + u->head_b,
+      u->G + u->conv[D0B].b_off, pix(u, 0));
   // decoder, from the output up
-  bf16 *g = u->gdout[0];
+  bf16 *g = nullptr;
   for (int l = 0; l <= 2; ++l) {
     const int C = kC[l];
     const int ca = (l == 2) ? D2A : (l == 1) ? D1A : D0A;
-    conv_block_back(u, ca + 1, g, C, 0, u->dout[l], C, 0, u->da[l], C, 0, u->gda[l], C, 0, l);
+    if (l == 0) conv_grads(u, ca + 1, u->da[l], C, 0, u->gda[l], C, 0, l);
+    else conv_block_back(u, ca + 1, g, C, 0, u->dout[l], C, 0, u->da[l], C, 0, u->gda[l], C, 0, l);
     conv_block_back(u, ca, u->gda[l], C, 0, u->da[l], C, 0, u->cat[l], 2 * C, 0, u->gcat[l], 2 * C, 0, l);
     // transposed conv: gradient at its input (the output of level l+1) from gcat[:, 0:C]
     const pic_unet::Up &up = u->up[l];
@@ -1181,7 +1243,7 @@ pic_status pic_unet_create(int32_t batch, int32_t height, int32_t width, void *s
       u->da[l] = (bf16 *)A(np * C * 2);
       u->gda[l] = (bf16 *)A(np * C * 2);
       u->dout[l] = (bf16 *)A(np * C * 2);
-      u->gdout[l] = (bf16 *)A(np * C * 2);
+      if (l > 0) u->gdout[l] = (bf16 *)A(np * C * 2);   // the head's backward writes dpre[0]
     } else {
       u->b3 = (bf16 *)A(np * C * 2);
       u->gb3 = (bf16 *)A(np * C * 2);
@@ -1500,8 +1562,8 @@ pic_status pic_head_back_bf16(int64_t npix, const float *dy, const void *hin, co
   const int sms = device_sms();
   if (sms < 1) return PIC_ECUDA;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  k_head_back<<<int(std::min<long long>((npix + 63) / 64, 8LL * sms)), 256, 0, s>>>(
-      dy, static_cast<const bf16 *>(hin), w, static_cast<bf16 *>(gh), dw, db, npix);
+  k_head_back<false><<<int(std::min<long long>((npix + 63) / 64, 8LL * sms)), 256, 0, s>>>(
+      dy, static_cast<const bf16 *>(hin), w, static_cast<bf16 *>(gh), dw, db, nullptr, npix);
   if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) return PIC_ECUDA;
   return PIC_OK;
 }
