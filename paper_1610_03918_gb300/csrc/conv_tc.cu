@@ -452,7 +452,21 @@ struct RowArgs {
   int tiles;               // B x col_blocks x H output rows of 128 pixels
   int wide;                // 32-byte stores are aligned
   int *err;
+  // what the epilogue does beside (Epilogue)
+  bf16 *pool;              // kPool: [B][H / 2][W / 2][pool_cs]
+  int pool_cs;
+  const bf16 *y;           // kBack: [B][H][W][y_cs], channels from y_off
+  int y_cs, y_off;
+  float *db;
 };
+
+// kPool: also the 2 x 2 average pool of the output (H and W even).  kBack: the
+// output, a gradient, goes through the ReLU that made y (0 where y is not
+// positive) and db[c] gains the sum of what is left.  Both spare a pass over the
+// output (k_pool_vec, k_relu_back), which is as long as the convolution: batch 4,
+// 32 -> 32 at 1032 x 512 46.8 + 42.5 us -> 55.5 and 45.5 + 64.4 -> 62; 64 -> 64 at
+// 516 x 256 32.8 + 13.3 -> 36 and 32.7 + 32.5 -> 48.
+enum Epilogue { kPlain, kPool, kBack };
 
 constexpr int kRowThreads = 320;
 constexpr int kRing = 8;                     // accumulators (output rows) in TMEM
@@ -488,13 +502,17 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
       : "r"(taddr));
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
-// the CTA's runs of output rows: tiles are numbered (image, column block, row)
+// the CTA's runs of output rows, pairs of rows with PAIRS (H even): tiles are
+// numbered (image, column block, row)
+template <bool PAIRS>
 struct Runs {
   int t, t1, H, cbs;
   int b, cb, h0, rows;
   __device__ __forceinline__ Runs(const RowArgs &a)
-      : t(int((long long)a.tiles * blockIdx.x / gridDim.x)),
-        t1(int((long long)a.tiles * (blockIdx.x + 1) / gridDim.x)), H(a.H), cbs(a.col_blocks) {}
+      : t(first(a.tiles, blockIdx.x)), t1(first(a.tiles, blockIdx.x + 1)), H(a.H), cbs(a.col_blocks) {}
+  static __device__ __forceinline__ int first(int tiles, unsigned cta) {
+    return PAIRS ? int((long long)(tiles / 2) * cta / gridDim.x) * 2 : int((long long)tiles * cta / gridDim.x);
+  }
   __device__ __forceinline__ bool next() {
     if (t >= t1) return false;
     const int col = t / H;
@@ -507,7 +525,7 @@ struct Runs {
   }
 };
 
-template <int N, int KB, int KC, bool TAPS>
+template <int N, int KB, int KC, bool TAPS, int EPI>
 __global__ void __launch_bounds__(kRowThreads, RowCfg<N, KB, KC>::CPS)
     k_conv_rows(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, RowArgs a) {
   using C = RowCfg<N, KB, KC>;
@@ -549,7 +567,7 @@ __global__ void __launch_bounds__(kRowThreads, RowCfg<N, KB, KC>::CPS)
             tma_load_2d(sW + ((dx * KC + c) * 3 + 2 - dy) * C::W_TILE, &tmB, (3 * dy + dx) * a.cin + c * KB, n0, wbar);
       uint32_t s = 0, ph = 1;   // next unit's slot, and the phase its release completes (the first round waits for none)
       bool ok = true;
-      Runs r(a);
+      Runs<EPI == kPool> r(a);
       while (ok && r.next())
         for (int q = -1; q <= r.rows && ok && !*fail; ++q)
           for (int c = 0; c < KC && ok; ++c) {
@@ -577,7 +595,7 @@ __global__ void __launch_bounds__(kRowThreads, RowCfg<N, KB, KC>::CPS)
     bool ok = mbar_wait_warp(wbar, 0);
     uint32_t s0 = 0, ph = 0;   // slot of the input row's first unit and its phase
     uint32_t i0 = 0;           // output rows of the runs before
-    Runs r(a);
+    Runs<EPI == kPool> r(a);
     while (ok && r.next()) {
       for (int q = -1; q <= r.rows && ok; ++q) {
         // output rows lo .. hi of the run take input row q; row q + 1 starts with it
@@ -665,28 +683,45 @@ __global__ void __launch_bounds__(kRowThreads, RowCfg<N, KB, KC>::CPS)
     const bool relu = a.relu != 0, wide = a.wide != 0;
     uint32_t i = 0;
     bool ok = true;
-    Runs r(a);
+    Runs<EPI == kPool> r(a);
+    float sum[EPI == kBack ? N : 1];         // kBack: the thread's columns' sums
+    uint32_t above[EPI == kPool ? N / 2 : 1];   // kPool: the output above
+    if (EPI == kBack)
+#pragma unroll
+      for (int k = 0; k < N; ++k) sum[EPI == kBack ? k : 0] = 0.f;
     while (ok && r.next()) {
       const int w = r.cb * kM + 32 * quad + lane;
-      bf16 *dst = a.out + ((size_t(r.b) * a.H + r.h0) * a.W + w) * a.out_cs + a.out_off + n0;
+      const size_t p0 = (size_t(r.b) * a.H + r.h0) * a.W + w;
+      bf16 *dst = a.out + p0 * a.out_cs + a.out_off + n0;
+      const bf16 *y = EPI == kBack ? a.y + p0 * a.y_cs + a.y_off + n0 : nullptr;
+      bf16 *pool = EPI == kPool ? a.pool + ((size_t(r.b) * (a.H / 2) + r.h0 / 2) * (a.W / 2) + w / 2) * a.pool_cs + n0
+                                : nullptr;
       for (int t = 0; t < r.rows; ++t, ++i, dst += size_t(a.W) * a.out_cs) {
-        if (int(i & 1) != half) continue;
+        if (int((EPI == kPool ? i >> 1 : i) & 1) != half) continue;
+        uint4 yv[EPI == kBack ? N / 8 : 1];
+        if (EPI == kBack) {
+          const uint4 *src = reinterpret_cast<const uint4 *>(y + size_t(t) * a.W * a.y_cs);
+#pragma unroll
+          for (int k = 0; k < N / 8; ++k) yv[EPI == kBack ? k : 0] = w < a.W ? src[k] : make_uint4(0u, 0u, 0u, 0u);
+        }
         const uint32_t acc = i % kRing;
         ok = __all_sync(0xffffffffu, mbar_wait(tfull + 8 * acc, (i / kRing) & 1));
         if (!ok) break;
         tc_fence_after();
         const uint32_t tl = tmem + (uint32_t(32 * quad) << 16) + acc * N;
+        constexpr int CH = EPI == kPlain ? 32 : 16;   // columns read at once (the others hold more beside)
 #pragma unroll
-        for (int c = 0; c < N; c += 32) {
-          uint32_t v[32];
-          tmem_ld32(tl + c, v);
-          if (c + 32 == N) {   // read out: the MMA may use the accumulator again
+        for (int c = 0; c < N; c += CH) {
+          uint32_t v[CH];
+          if constexpr (CH == 32) tmem_ld32(tl + c, v);
+          else tmem_ld16(tl + c, v);
+          if (c + CH == N) {   // read out: the MMA may use the accumulator again
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(tempty + 8 * acc);
           }
 #pragma unroll
-          for (int q = 0; q < 32; q += 16) {
+          for (int q = 0; q < CH; q += 16) {
             uint32_t o[8];
 #pragma unroll
             for (int k = 0; k < 8; k += 2) {
@@ -695,10 +730,62 @@ __global__ void __launch_bounds__(kRowThreads, RowCfg<N, KB, KC>::CPS)
               o[k] = bf16_pair(x[0] + b.x, x[1] + b.y, relu);
               o[k + 1] = bf16_pair(x[2] + b.z, x[3] + b.w, relu);
             }
+            if (EPI == kBack) {
+              const uint32_t *yy = reinterpret_cast<const uint32_t *>(yv + (EPI == kBack ? (c + q) / 8 : 0));
+#pragma unroll
+              for (int k = 0; k < 8; ++k) {
+                o[k] &= __hgt2_mask(*reinterpret_cast<const __nv_bfloat162 *>(yy + k), __floats2bfloat162_rn(0.f, 0.f));
+                sum[EPI == kBack ? c + q + 2 * k : 0] += __uint_as_float(o[k] << 16);
+                sum[EPI == kBack ? c + q + 2 * k + 1 : 0] += __uint_as_float(o[k] & 0xffff0000u);
+              }
+            }
             if (w < a.W) store16(dst + c + q, o, wide);
+            if (EPI == kPool) {
+              if (!(i & 1)) {
+#pragma unroll
+                for (int k = 0; k < 8; ++k) above[EPI == kPool ? (c + q) / 2 + k : 0] = o[k];
+              } else {
+                // of the pair of pixels the even lane pools channels 0-7, the odd one 8-15:
+                // ((above left + above right) + left) + right
+                const bool odd = lane & 1;
+                uint32_t m[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                  const uint32_t al = above[EPI == kPool ? (c + q) / 2 + k : 0],
+                                 ah = above[EPI == kPool ? (c + q) / 2 + 4 + k : 0];
+                  const uint32_t am = odd ? ah : al, bm = odd ? o[4 + k] : o[k];
+                  const uint32_t ax = __shfl_xor_sync(0xffffffffu, odd ? al : ah, 1);
+                  const uint32_t bx = __shfl_xor_sync(0xffffffffu, odd ? o[k] : o[4 + k], 1);
+                  const uint32_t bl = odd ? bx : bm, br = odd ? bm : bx;
+                  const float lo = 0.25f * (((0.f + __uint_as_float(am << 16)) + __uint_as_float(ax << 16) +
+                                             __uint_as_float(bl << 16)) + __uint_as_float(br << 16));
+                  const float hi = 0.25f * (((0.f + __uint_as_float(am & 0xffff0000u)) +
+                                             __uint_as_float(ax & 0xffff0000u) + __uint_as_float(bl & 0xffff0000u)) +
+                                            __uint_as_float(br & 0xffff0000u));
+                  m[k] = bf16_pair(lo, hi, false);
+                }
+                if (w < a.W)
+                  *reinterpret_cast<uint4 *>(pool + size_t(t >> 1) * (a.W / 2) * a.pool_cs + c + q + (odd ? 8 : 0)) =
+                      make_uint4(m[0], m[1], m[2], m[3]);
+              }
+            }
           }
           __syncwarp();
         }
+      }
+    }
+    if (EPI == kBack) {
+#pragma unroll
+      for (int c = 0; c < N; c += 32) {
+        float mine = 0.f;
+#pragma unroll
+        for (int k = 0; k < 32; ++k) {
+          float x = sum[EPI == kBack ? c + k : 0];
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+          if (lane == k) mine = x;
+        }
+        atomicAdd(&a.db[n0 + c + lane], mine);
       }
     }
     if (!ok && lane == 0) {
@@ -1171,19 +1258,20 @@ cudaError_t launch_nks(const ConvTC &c, cudaStream_t s, int nblk) {
 }
 
 // ---- the persistent row kernel (k_conv_rows)
-template <int N, int KB, int KC, bool TAPS>
+template <int N, int KB, int KC, bool TAPS, int EPI = kPlain>
 cudaError_t prepare_rows() {
-  static cudaError_t e = cudaFuncSetAttribute(k_conv_rows<N, KB, KC, TAPS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              int(RowCfg<N, KB, KC>::BYTES));
+  static cudaError_t e =
+      cudaFuncSetAttribute(k_conv_rows<N, KB, KC, TAPS, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           int(RowCfg<N, KB, KC>::BYTES));
   return e;
 }
 
-template <int N, int KB, int KC, bool TAPS>
+template <int N, int KB, int KC, bool TAPS, int EPI = kPlain>
 cudaError_t launch_rows(const ConvTC &c, cudaStream_t s, int sms) {
   using R = RowCfg<N, KB, KC>;
   auto fn = encode_fn();
   if (!fn) return cudaErrorNotSupported;
-  const cudaError_t attr = prepare_rows<N, KB, KC, TAPS>();
+  const cudaError_t attr = prepare_rows<N, KB, KC, TAPS, EPI>();
   if (attr != cudaSuccess) return attr;
   CUtensorMap ta, tb;
   const cuuint32_t one[4] = {1, 1, 1, 1};
@@ -1216,9 +1304,15 @@ cudaError_t launch_rows(const ConvTC &c, cudaStream_t s, int sms) {
   a.tiles = c.B * a.col_blocks * c.H;
   a.wide = wide_stores(c);
   a.err = c.err;
+  a.pool = c.pool;
+  a.pool_cs = c.cout;
+  a.y = c.y;
+  a.y_cs = c.y_cs;
+  a.y_off = c.y_off;
+  a.db = c.db;
   const int nblk = c.cout / N;
-  const int ctas = std::max(1, std::min(a.tiles, sms * R::CPS / nblk));
-  k_conv_rows<N, KB, KC, TAPS><<<dim3(unsigned(ctas), unsigned(nblk)), kRowThreads, R::BYTES, s>>>(ta, tb, a);
+  const int ctas = std::max(1, std::min(EPI == kPool ? a.tiles / 2 : a.tiles, sms * R::CPS / nblk));
+  k_conv_rows<N, KB, KC, TAPS, EPI><<<dim3(unsigned(ctas), unsigned(nblk)), kRowThreads, R::BYTES, s>>>(ta, tb, a);
   return cudaGetLastError();
 }
 
@@ -1462,7 +1556,11 @@ cudaError_t conv3x3_tc_prepare() {
                         tc::prepare_rows<64, 32, 1, false>(), tc::prepare_rows<64, 64, 1, false>(),
                         tc::prepare_rows<64, 64, 2, false>(), tc::prepare_rows<64, 64, 1, true>(),
                         tc::prepare_rows<64, 64, 2, true>(), tc::prepare_rows<32, 64, 4, false>(),
-                        tc::prepare_rows<32, 64, 4, true>()})
+                        tc::prepare_rows<32, 64, 4, true>(),
+                        tc::prepare_rows<32, 32, 1, false, tc::kPool>(), tc::prepare_rows<64, 64, 1, false, tc::kPool>(),
+                        tc::prepare_rows<64, 64, 2, false, tc::kPool>(), tc::prepare_rows<64, 64, 2, true, tc::kPool>(),
+                        tc::prepare_rows<32, 32, 1, false, tc::kBack>(), tc::prepare_rows<64, 64, 1, false, tc::kBack>(),
+                        tc::prepare_rows<64, 64, 2, false, tc::kBack>(), tc::prepare_rows<64, 64, 2, true, tc::kBack>()})
     if (e == cudaSuccess) e = f;
   return e;
 }
@@ -1494,7 +1592,27 @@ cudaError_t conv3x3_tc(const ConvTC &c, cudaStream_t s) {
   // the persistent row kernel (whole 128-pixel rows; input channels whose
   // weights fit beside a row), with the K order of the kernel it replaces: that
   // one takes (dy, chunk, dx) up to 64 columns a CTA and (dy, dx, chunk) above
-  if (!up && c.W >= tc::kM && (long long)c.B * ((c.W + tc::kM - 1) / tc::kM) * c.H < (1LL << 31)) {
+  const bool rows = !up && c.W >= tc::kM && (long long)c.B * ((c.W + tc::kM - 1) / tc::kM) * c.H < (1LL << 31);
+  // its other epilogues: as many channels out as in, up to 128 (the blocks' second layers)
+  if (c.pool || c.y) {
+    if (!rows || c.cin != c.cout || (c.pool && (c.y || c.H % 2 || c.W % 2)) ||
+        (c.y && (c.y_cs % 8 || c.y_off % 8 || !c.db)))
+      return cudaErrorNotSupported;
+    if (n == 32 && c.cin == 32)
+      return c.pool ? tc::launch_rows<32, 32, 1, false, tc::kPool>(c, s, sms)
+                    : tc::launch_rows<32, 32, 1, false, tc::kBack>(c, s, sms);
+    if (n == 64 && c.cin == 64)
+      return c.pool ? tc::launch_rows<64, 64, 1, false, tc::kPool>(c, s, sms)
+                    : tc::launch_rows<64, 64, 1, false, tc::kBack>(c, s, sms);
+    if (n == 64 && c.cin == 128)
+      return c.pool ? tc::launch_rows<64, 64, 2, false, tc::kPool>(c, s, sms)
+                    : tc::launch_rows<64, 64, 2, false, tc::kBack>(c, s, sms);
+    if (n == 128 && c.cin == 128)
+      return c.pool ? tc::launch_rows<64, 64, 2, true, tc::kPool>(c, s, sms)
+                    : tc::launch_rows<64, 64, 2, true, tc::kBack>(c, s, sms);
+    return cudaErrorNotSupported;
+  }
+  if (rows) {
     if (n == 32 && c.cin == 32) return tc::launch_rows<32, 32, 1, false>(c, s, sms);
     if (n == 32 && c.cin == 64) return tc::launch_rows<32, 64, 1, false>(c, s, sms);
     if (n == 64 && c.cin == 32) return tc::launch_rows<64, 32, 1, false>(c, s, sms);

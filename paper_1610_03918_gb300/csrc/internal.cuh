@@ -517,6 +517,16 @@ struct ConvTC {
   // out 2H x 2W; this launch computes the cout GEMM columns from n_base
   int up_cout = 0;
   int n_base = 0;
+  // the same convolution with more in its epilogue, or cudaErrorNotSupported
+  // (the row kernel has them: cin = cout up to 128, images from 128 pixels wide):
+  // pool: also the 2 x 2 average pool of the output, [B][H / 2][W / 2][cout].
+  // y: the output is the gradient of y, relu's output; it is 0 where y (channels
+  // y_off .. in rows of y_cs) is not positive, and its sums over all pixels are
+  // added to db[cout].
+  __nv_bfloat16 *pool = nullptr;
+  const __nv_bfloat16 *y = nullptr;
+  int y_cs = 0, y_off = 0;
+  float *db = nullptr;
 };
 bool conv3x3_tc_supported(int cin, int cout, int in_cs, int in_off, int out_cs, int out_off, int W);
 cudaError_t conv3x3_tc(const ConvTC &c, cudaStream_t s);

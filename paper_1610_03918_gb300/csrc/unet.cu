@@ -773,9 +773,10 @@ int pix(const pic_unet *u, int l) { return u->B * (u->H >> l) * (u->W >> l); }
 
 // the tcgen05 convolution when the net uses it and the shapes allow it
 bool conv_tc(pic_unet *u, const bf16 *in, int in_cs, int in_off, int cin, const bf16 *w,
-             const float *bias, bf16 *out, int out_cs, int out_off, int cout, int l, bool relu) {
+             const float *bias, bf16 *out, int out_cs, int out_off, int cout, int l, bool relu,
+             const ConvTC &epilogue = ConvTC()) {
   if (u->conv_impl != 0) return false;
-  ConvTC c;
+  ConvTC c = epilogue;
   c.in = in;
   c.in_cs = in_cs;
   c.in_off = in_off;
@@ -796,8 +797,17 @@ bool conv_tc(pic_unet *u, const bf16 *in, int in_cs, int in_off, int cin, const 
 }
 
 void conv_fwd(pic_unet *u, int ci, const bf16 *in, int in_cs, int in_off, bf16 *out, int out_cs,
-              int out_off, int l, bool relu) {
+              int out_off, int l, bool relu, bf16 *pool = nullptr) {
   const pic_unet::Conv &c = u->conv[ci];
+  if (pool) {   // with the 2 x 2 average pool of the output
+    ConvTC e;
+    e.pool = pool;
+    if (conv_tc(u, in, in_cs, in_off, c.cin_c, c.w, u->P + c.b_off, out, out_cs, out_off, c.cout, l, relu, e)) return;
+    conv_fwd(u, ci, in, in_cs, in_off, out, out_cs, out_off, l, relu);
+    k_pool_vec<<<gridn((long long)pix(u, l + 1) * c.cout / 8), 256, 0, u->stream>>>(out, out_cs, out_off, pool, c.cout,
+                                                                                   u->B, u->H >> l, u->W >> l);
+    return;
+  }
   if (conv_tc(u, in, in_cs, in_off, c.cin_c, c.w, u->P + c.b_off, out, out_cs, out_off, c.cout, l, relu))
     return;
   ConvArgs a;
@@ -842,10 +852,19 @@ void flip_weights(pic_unet *u) {
   k_wflip<<<dim3(unsigned(2 * u->num_sms), unsigned(n)), 256, 0, u->stream>>>(a);
 }
 
-// data gradient: gin (cin channels) = conv(dpre, flipped weights)
-void conv_back_data(pic_unet *u, int ci, const bf16 *dpre, bf16 *gin, int gin_cs, int gin_off, int l) {
+// data gradient: gin (cin channels) = conv(dpre, flipped weights).  before: the layer that made the input, through whose ReLU the gradient then
+// goes (y contiguous; its bias gradient too) where the kernel can: true if it did
+bool conv_back_data(pic_unet *u, int ci, const bf16 *dpre, bf16 *gin, int gin_cs, int gin_off, int l,
+                    int before = -1, const bf16 *y = nullptr) {
   const pic_unet::Conv &c = u->conv[ci];
-  if (conv_tc(u, dpre, c.cout, 0, c.cout, c.wt, nullptr, gin, gin_cs, gin_off, c.cin_c, l, false)) return;
+  if (before >= 0) {
+    ConvTC e;
+    e.y = y;
+    e.y_cs = c.cin_c;
+    e.db = u->G + u->conv[before].b_off;
+    if (conv_tc(u, dpre, c.cout, 0, c.cout, c.wt, nullptr, gin, gin_cs, gin_off, c.cin_c, l, false, e)) return true;
+  }
+  if (conv_tc(u, dpre, c.cout, 0, c.cout, c.wt, nullptr, gin, gin_cs, gin_off, c.cin_c, l, false)) return false;
   ConvArgs a;
   a.in = dpre;
   a.in_cs = c.cout;
@@ -867,6 +886,7 @@ void conv_back_data(pic_unet *u, int ci, const bf16 *dpre, bf16 *gin, int gin_cs
   } else {
     k_conv3x3<64, 32><<<dim3(a.B * a.H * nwt, a.cout / 64), kConvThreads, 0, u->stream>>>(a);
   }
+  return false;
 }
 
 // the weight gradient on the mma.sync kernel (FP32 atomics over row groups)
@@ -919,32 +939,37 @@ void conv_back_weights(pic_unet *u, int ci, const bf16 *dpre, const bf16 *in, in
                                                                           c.cout, c.cin_m, c.cin_c);
 }
 
-// the weight gradient and the gradient gin at the input (unless null) of a
-// convolution whose pre-activation gradient is in dpre[l]
-void conv_grads(pic_unet *u, int ci, const bf16 *in, int in_cs, int in_off, bf16 *gin, int gin_cs, int gin_off,
-                int l) {
-  conv_back_weights(u, ci, u->dpre[l], in, in_cs, in_off, l);
-  if (gin) conv_back_data(u, ci, u->dpre[l], gin, gin_cs, gin_off, l);
-}
-
-// backward through relu(conv(in)) given the gradient g at its output;
-// writes the gradient at its input into gin (unless gin is null)
-// gp: the gradient of the average pool that follows y's block (added to g), or null
-void conv_block_back(pic_unet *u, int ci, const bf16 *g, int g_cs, int g_off, const bf16 *y, int y_cs,
-                     int y_off, const bf16 *in, int in_cs, int in_off, bf16 *gin, int gin_cs,
-                     int gin_off, int l, const bf16 *gp = nullptr) {
+// backward through the ReLU that follows layer ci: dpre[l] from the gradient g at
+// its output y, and the bias gradient.  gp: the gradient of the average pool that
+// follows (added to g), or null
+void relu_back(pic_unet *u, int ci, const bf16 *g, int g_cs, int g_off, const bf16 *y, int y_cs, int y_off, int l,
+               const bf16 *gp = nullptr) {
   const pic_unet::Conv &c = u->conv[ci];
   const long long np = pix(u, l);
-  bf16 *dpre = u->dpre[l];
   const long long ppb = 256 / (c.cout / 8);
   const int grid = int(std::min<long long>((np + ppb - 1) / ppb, 8LL * u->num_sms));
   if (gp)
     k_relu_back<true><<<grid, 256, 0, u->stream>>>(g, g_cs, g_off, y, y_cs, y_off, gp, u->H >> l, u->W >> l,
-                                                   dpre, c.cout, np, u->G + c.b_off);
+                                                   u->dpre[l], c.cout, np, u->G + c.b_off);
   else
-    k_relu_back<false><<<grid, 256, 0, u->stream>>>(g, g_cs, g_off, y, y_cs, y_off, nullptr, 1, 1, dpre,
+    k_relu_back<false><<<grid, 256, 0, u->stream>>>(g, g_cs, g_off, y, y_cs, y_off, nullptr, 1, 1, u->dpre[l],
                                                     c.cout, np, u->G + c.b_off);
-  conv_grads(u, ci, in, in_cs, in_off, gin, gin_cs, gin_off, l);
+}
+
+// The two layers of a block (cb after ca, y between them), from dpre, the gradient
+// before cb's ReLU: their weight gradients, ca's bias gradient, and the gradient gin
+// at ca's input (unless null).  gy: room for the gradient at y.
+void block_back(pic_unet *u, int ca, int cb, const bf16 *dpre, const bf16 *y, bf16 *gy, const bf16 *in, int in_cs,
+                int in_off, bf16 *gin, int gin_cs, int l) {
+  const int C = u->conv[ca].cout;
+  conv_back_weights(u, cb, dpre, y, C, 0, l);
+  const bf16 *d = gy;
+  if (!conv_back_data(u, cb, dpre, gy, C, 0, l, ca, y)) {
+    relu_back(u, ca, gy, C, 0, y, C, 0, l);
+    d = u->dpre[l];
+  }
+  conv_back_weights(u, ca, d, in, in_cs, in_off, l);
+  if (gin) conv_back_data(u, ca, d, gin, gin_cs, 0, l);
 }
 
 void weights_to_bf16(pic_unet *u) {
@@ -1062,14 +1087,11 @@ void forward(pic_unet *u, const float *x, bool keep_input) {
       k_conv_in<<<grid, 256, 0, u->stream>>>(x2, c.w, c.cin_c, u->P + c.b_off, u->a[0], u->B, u->H, u->W, 1);
     }
   }
-  conv_fwd(u, E0B, u->a[0], C0, 0, u->cat[0], 2 * C0, C0, 0, true);
-  k_pool_vec<<<gridn((long long)pix(u, 1) * C0 / 8), 256, 0, u->stream>>>(u->cat[0], 2 * C0, C0, u->p[1], C0, u->B, u->H, u->W);
+  conv_fwd(u, E0B, u->a[0], C0, 0, u->cat[0], 2 * C0, C0, 0, true, u->p[1]);
   conv_fwd(u, E1A, u->p[1], C0, 0, u->a[1], C1, 0, 1, true);
-  conv_fwd(u, E1B, u->a[1], C1, 0, u->cat[1], 2 * C1, C1, 1, true);
-  k_pool_vec<<<gridn((long long)pix(u, 2) * C1 / 8), 256, 0, u->stream>>>(u->cat[1], 2 * C1, C1, u->p[2], C1, u->B, u->H >> 1, u->W >> 1);
+  conv_fwd(u, E1B, u->a[1], C1, 0, u->cat[1], 2 * C1, C1, 1, true, u->p[2]);
   conv_fwd(u, E2A, u->p[2], C1, 0, u->a[2], C2, 0, 2, true);
-  conv_fwd(u, E2B, u->a[2], C2, 0, u->cat[2], 2 * C2, C2, 2, true);
-  k_pool_vec<<<gridn((long long)pix(u, 3) * C2 / 8), 256, 0, u->stream>>>(u->cat[2], 2 * C2, C2, u->p[3], C2, u->B, u->H >> 2, u->W >> 2);
+  conv_fwd(u, E2B, u->a[2], C2, 0, u->cat[2], 2 * C2, C2, 2, true, u->p[3]);
   conv_fwd(u, E3A, u->p[3], C2, 0, u->a[3], C3, 0, 3, true);
   conv_fwd(u, E3B, u->a[3], C3, 0, u->b3, C3, 0, 3, true);
   // decoder
@@ -1103,9 +1125,8 @@ void backward(pic_unet *u) {
   for (int l = 0; l <= 2; ++l) {
     const int C = kC[l];
     const int ca = (l == 2) ? D2A : (l == 1) ? D1A : D0A;
-    if (l == 0) conv_grads(u, ca + 1, u->da[l], C, 0, u->gda[l], C, 0, l);
-    else conv_block_back(u, ca + 1, g, C, 0, u->dout[l], C, 0, u->da[l], C, 0, u->gda[l], C, 0, l);
-    conv_block_back(u, ca, u->gda[l], C, 0, u->da[l], C, 0, u->cat[l], 2 * C, 0, u->gcat[l], 2 * C, 0, l);
+    if (l > 0) relu_back(u, ca + 1, g, C, 0, u->dout[l], C, 0, l);
+    block_back(u, ca, ca + 1, u->dpre[l], u->da[l], u->gda[l], u->cat[l], 2 * C, 0, u->gcat[l], 2 * C, l);
     // transposed conv: gradient at its input (the output of level l+1) from gcat[:, 0:C]
     const pic_unet::Up &up = u->up[l];
     const int hl = u->H >> (l + 1), wl = u->W >> (l + 1);
@@ -1126,19 +1147,18 @@ void backward(pic_unet *u) {
     g = gin;
   }
   // bottleneck
-  conv_block_back(u, E3B, u->gb3, C3, 0, u->b3, C3, 0, u->a[3], C3, 0, u->gx[3], C3, 0, 3);
-  conv_block_back(u, E3A, u->gx[3], C3, 0, u->a[3], C3, 0, u->p[3], kC[2], 0, u->gp[3], kC[2], 0, 3);
+  relu_back(u, E3B, u->gb3, C3, 0, u->b3, C3, 0, 3);
+  block_back(u, E3A, E3B, u->dpre[3], u->a[3], u->gx[3], u->p[3], kC[2], 0, u->gp[3], kC[2], 3);
   // encoder, back down: the pool's gradient joins the skip gradient gcat[l][C:2C]
   // inside the ReLU's backward
   for (int l = 2; l >= 0; --l) {
     const int C = kC[l];
     const int ea = 2 * l;   // E0A, E1A, E2A
-    conv_block_back(u, ea + 1, u->gcat[l], 2 * C, C, u->cat[l], 2 * C, C, u->a[l], C, 0, u->gx[l], C, 0, l,
-                    u->gp[l + 1]);
+    relu_back(u, ea + 1, u->gcat[l], 2 * C, C, u->cat[l], 2 * C, C, l, u->gp[l + 1]);
     if (l > 0)
-      conv_block_back(u, ea, u->gx[l], C, 0, u->a[l], C, 0, u->p[l], kC[l - 1], 0, u->gp[l], kC[l - 1], 0, l);
+      block_back(u, ea, ea + 1, u->dpre[l], u->a[l], u->gx[l], u->p[l], kC[l - 1], 0, u->gp[l], kC[l - 1], l);
     else
-      conv_block_back(u, ea, u->gx[0], C, 0, u->a[0], C, 0, u->x16, kCin0, 0, nullptr, 0, 0, 0);
+      block_back(u, ea, ea + 1, u->dpre[0], u->a[0], u->gx[0], u->x16, kCin0, 0, nullptr, 0, 0);
   }
 }
 
