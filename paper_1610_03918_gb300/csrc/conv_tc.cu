@@ -799,6 +799,246 @@ __global__ void __launch_bounds__(kRowThreads, RowCfg<N, KB, KC>::CPS)
   if (warp == 0) tmem_dealloc(tmem, C::NCOLS);
 }
 
+// ---------------------------------------------------------------- 2 x 2 transposed convolutions
+// The transposed convolution and its data gradient as persistent kernels: CTAs
+// of one tile of k_conv3x3_tc spend most of their few MMAs' time on starting, on
+// the weights and on an epilogue that nothing overlaps.  A CTA keeps the weights
+// of its N GEMM columns in shared memory and takes tiles of 128 pixels of the
+// small image one after another, KB channels a unit; units, accumulators and
+// epilogue overlap.
+//   kUp:      columns (2a + c) up_cout + co of the tile's 128 pixels go to child
+//             (2h + a, 2w + c); K = cin
+//   kUpBack:  the data gradient: K = the four children's channels (UPB above)
+//   kUpBackY: the same, on through the ReLU that made its target (kBack)
+//   warps 0-7  epilogue: warps 0-3 the lower, 4-7 the upper half of the columns
+//   warp 8     TMA        warp 9     MMA
+// K is summed in the order of k_conv3x3_tc: the same results bit for bit.  Bound
+// by memory: cold, batch 4, small image 516 x 256, 64 -> 32 channels 38.9 us (57.4
+// before; 203 MB), its gradient with the ReLU 65.8 (45.0 + 32.4; half of each
+// 128-byte line of the concatenation's gradient is its other half, 404 MB in all);
+// 128 -> 64 at 258 x 128 24.3 (38.5) and 27.9 (26.9 + 18.7).
+enum UpMode { kUp, kUpBack, kUpBackY };
+
+struct UpArgs {
+  bf16 *out;
+  int out_cs, out_off;
+  const float *bias;
+  int B, H, W;             // the small image
+  int log_bw;              // tile: 2^log_bw x 128 / 2^log_bw pixels
+  int tiles_w, tiles_h, tiles;
+  int in_off, kchunks, units;   // units of KB channels per tap and in all
+  int n_base;              // first GEMM column of CTA row 0
+  int up_cout;             // kUp: output channels
+  int ncols;               // kUpBack: weight rows per child
+  int stages;              // units in the ring
+  int wide;
+  const bf16 *y;
+  int y_cs, y_off;
+  float *db;
+  int *err;
+};
+constexpr int kUpStages = 8;
+
+template <int N, int KB, int MODE>
+__global__ void __launch_bounds__(kRowThreads, 1)
+    k_up_tiles(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, UpArgs a) {
+  constexpr int RING = N >= 256 ? 2 : 4;   // accumulators in TMEM
+  constexpr uint32_t UNIT = kM * KB * 2, W_TILE = N * KB * 2;
+  constexpr int HALF = N / 2;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  __shared__ __align__(8) uint64_t s_bar[2 * kUpStages + 1 + 2 * RING];
+  __shared__ uint32_t s_slot;
+  __shared__ int s_fail;
+  __shared__ float4 s_bias[N / 4];
+  const uint32_t S = a.stages;
+  const uint32_t sW = saddr(smem), sU = sW + a.units * W_TILE;
+  const uint32_t full = saddr(s_bar), empty = full + 8 * kUpStages, wbar = empty + 8 * kUpStages, tfull = wbar + 8,
+                 tempty = tfull + 8 * RING;
+  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
+  const int n0 = a.n_base + int(blockIdx.y) * N;
+  if (tid < N)
+    reinterpret_cast<float *>(s_bias)[tid] = a.bias ? a.bias[MODE == kUp ? (n0 + tid) % a.up_cout : n0 + tid] : 0.f;
+  if (tid == 0) {
+    for (int k = 0; k < kUpStages; ++k) {
+      mbar_init(full + 8 * k, 1);
+      mbar_init(empty + 8 * k, 1);
+    }
+    mbar_init(wbar, 1);
+    for (int k = 0; k < RING; ++k) {
+      mbar_init(tfull + 8 * k, 1);
+      mbar_init(tempty + 8 * k, 8);
+    }
+    s_fail = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) tmem_alloc(saddr(&s_slot), RING * N);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = s_slot;
+  volatile int *fail = &s_fail;
+  const int t0 = int((long long)a.tiles * blockIdx.x / gridDim.x);
+  const int t1 = int((long long)a.tiles * (blockIdx.x + 1) / gridDim.x);
+  const int bw = 1 << a.log_bw, bh = kM >> a.log_bw;
+
+  if (warp == 8) {
+    if (lane == 0) {
+      mbar_expect_tx(wbar, a.units * W_TILE);
+      for (int u = 0; u < a.units; ++u) {
+        const int tap = u / a.kchunks, c0 = (u - tap * a.kchunks) * KB;
+        tma_load_2d(sW + u * W_TILE, &tmB, c0, tap * a.ncols + n0, wbar);
+      }
+      uint32_t s = 0, ph = 1;   // next unit's slot, and the phase its release completes
+      bool ok = true;
+      for (int t = t0; t < t1 && ok && !*fail; ++t) {
+        const int r = t / a.tiles_w, w0 = (t - r * a.tiles_w) << a.log_bw;
+        const int b = r / a.tiles_h, h0 = (r - b * a.tiles_h) * bh;
+        for (int u = 0; u < a.units && ok; ++u) {
+          ok = mbar_wait(empty + 8 * s, ph);
+          if (!ok) break;
+          mbar_expect_tx(full + 8 * s, UNIT);
+          if (MODE == kUp) {
+            tma_load_4d(sU + s * UNIT, &tmA, a.in_off + u * KB, w0, h0, b, full + 8 * s);
+          } else {
+            const int tap = u / a.kchunks, c0 = (u - tap * a.kchunks) * KB;
+            tma_load_5d(sU + s * UNIT, &tmA, a.in_off + c0, tap & 1, w0, tap >> 1, b * a.H + h0, full + 8 * s);
+          }
+          if (++s == S) {
+            s = 0;
+            ph ^= 1;
+          }
+        }
+      }
+      if (!ok) {
+        atomicExch(&s_fail, 1);
+        atomicCAS(a.err, 0, 1);
+      }
+    }
+  } else if (warp == 9) {
+    const bool leader = elect_one();
+    constexpr uint32_t idesc = instr_desc<N>();
+    const uint64_t dw64 = smem_desc<KB>(sW);
+    const uint32_t dw = uint32_t(dw64), du = uint32_t(smem_desc<KB>(sU)), dhi = uint32_t(dw64 >> 32);
+    bool ok = mbar_wait_warp(wbar, 0);
+    uint32_t s = 0, ph = 0;
+    for (int t = t0; t < t1 && ok; ++t) {
+      const uint32_t i = t - t0, acc = i % RING;
+      ok = mbar_wait_warp(tempty + 8 * acc, ((i / RING) & 1) ^ 1) && !__any_sync(0xffffffffu, *fail);
+      for (int u = 0; u < a.units && ok; ++u) {
+        ok = mbar_wait_warp(full + 8 * s, ph);
+        if (!ok) break;
+        tc_fence_after();
+        if (leader) {
+#pragma unroll
+          for (int k = 0; k < KB / 16; ++k)
+            mma_bf16_lo(tmem + acc * N, du + s * (UNIT >> 4) + 2 * k, dw + u * (W_TILE >> 4) + 2 * k, dhi, idesc,
+                        (u | k) != 0 ? 1u : 0u);
+          mma_commit(empty + 8 * s);
+        }
+        if (++s == S) {
+          s = 0;
+          ph ^= 1;
+        }
+      }
+      if (ok && leader) mma_commit(tfull + 8 * acc);
+    }
+    if (!ok && leader) {
+      atomicExch(&s_fail, 1);
+      atomicCAS(a.err, 0, 2);
+    }
+  } else {
+    // thread (warp w, lane l) owns pixel 32 (w mod 4) + l of the tile, the accumulators' TMEM lane
+    const int quad = warp & 3, half = warp >> 2;
+    const int p = 32 * quad + lane, ph = p >> a.log_bw, pw = p & (bw - 1);
+    const int col0 = half * HALF;   // the warp's first column of the accumulator
+    const bool wide = a.wide != 0;
+    bool ok = true;
+    float sum[MODE == kUpBackY ? HALF : 1];
+    if (MODE == kUpBackY)
+#pragma unroll
+      for (int k = 0; k < HALF; ++k) sum[MODE == kUpBackY ? k : 0] = 0.f;
+    for (int t = t0; t < t1 && ok; ++t) {
+      const uint32_t i = t - t0, acc = i % RING;
+      const int r = t / a.tiles_w, w = ((t - r * a.tiles_w) << a.log_bw) + pw;
+      const int b = r / a.tiles_h, h = (r - b * a.tiles_h) * bh + ph;
+      const bool inside = h < a.H && w < a.W;
+      const size_t px = (size_t(b) * a.H + h) * a.W + w;
+      uint4 yv[MODE == kUpBackY ? HALF / 8 : 1];
+      if (MODE == kUpBackY) {
+        const uint4 *src = reinterpret_cast<const uint4 *>(a.y + px * a.y_cs + a.y_off + n0 + col0);
+#pragma unroll
+        for (int k = 0; k < HALF / 8; ++k) yv[MODE == kUpBackY ? k : 0] = inside ? src[k] : make_uint4(0u, 0u, 0u, 0u);
+      }
+      ok = __all_sync(0xffffffffu, mbar_wait(tfull + 8 * acc, (i / RING) & 1));
+      if (!ok) break;
+      tc_fence_after();
+      const uint32_t tl = tmem + (uint32_t(32 * quad) << 16) + acc * N + col0;
+      // kUp: a child's columns come together
+      int ac = MODE == kUp ? (n0 + col0) / a.up_cout : 0, co = n0 + col0 - ac * (MODE == kUp ? a.up_cout : 0);
+#pragma unroll
+      for (int c = 0; c < HALF; c += 16) {
+        uint32_t v[16];
+        tmem_ld16(tl + c, v);
+        if (c + 16 == HALF) {   // read out: the MMA may use the accumulator again
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(tempty + 8 * acc);
+        }
+        uint32_t o[8];
+#pragma unroll
+        for (int k = 0; k < 8; k += 2) {
+          const float4 bs = s_bias[(col0 + c + 2 * k) / 4];
+          const float *x = reinterpret_cast<const float *>(v + 2 * k);
+          o[k] = bf16_pair(x[0] + bs.x, x[1] + bs.y, false);
+          o[k + 1] = bf16_pair(x[2] + bs.z, x[3] + bs.w, false);
+        }
+        if (MODE == kUpBackY) {
+          const uint32_t *yy = reinterpret_cast<const uint32_t *>(yv + (MODE == kUpBackY ? c / 8 : 0));
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            o[k] &= __hgt2_mask(*reinterpret_cast<const __nv_bfloat162 *>(yy + k), __floats2bfloat162_rn(0.f, 0.f));
+            sum[MODE == kUpBackY ? c + 2 * k : 0] += __uint_as_float(o[k] << 16);
+            sum[MODE == kUpBackY ? c + 2 * k + 1 : 0] += __uint_as_float(o[k] & 0xffff0000u);
+          }
+        }
+        if (inside) {
+          const size_t q = MODE == kUp ? (size_t(b) * 2 * a.H + 2 * h + (ac >> 1)) * 2 * a.W + 2 * w + (ac & 1) : px;
+          store16(a.out + q * a.out_cs + a.out_off + co, o, wide);
+        }
+        co += 16;
+        if (MODE == kUp && co == a.up_cout) {
+          co = 0;
+          ac += 1;
+        }
+        __syncwarp();
+      }
+    }
+    if (MODE == kUpBackY) {
+#pragma unroll
+      for (int c = 0; c < HALF; c += 32) {
+        float mine = 0.f;
+#pragma unroll
+        for (int k = 0; k < 32; ++k) {
+          float x = sum[MODE == kUpBackY ? c + k : 0];
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+          if (lane == k) mine = x;
+        }
+        atomicAdd(&a.db[n0 + col0 + c + lane], mine);
+      }
+    }
+    if (!ok && lane == 0) {
+      atomicExch(&s_fail, 1);
+      atomicCAS(a.err, 0, 3);
+    }
+  }
+  __syncwarp();
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0) tmem_dealloc(tmem, RING * N);
+}
+
 // ---------------------------------------------------------------- first layer
 // The network's first 3x3 convolution (2 input channels -> 32) on the tensor
 // cores.  The 9 taps x 2 channels of a pixel, BF16-rounded, form one K row of
@@ -1535,6 +1775,122 @@ cudaError_t launch_upw(const UpWgradTC &g, cudaStream_t s, int sms) {
   return cudaGetLastError();
 }
 
+// The persistent transposed convolution (up_cout > 0: all 4 up_cout columns from
+// n_base 0 on, c.cout of them) and its data gradient; cudaErrorNotSupported for
+// channel counts that are no multiples of 32, or columns that 64 does not divide.
+constexpr int kUpSmem = 227 * 1024 - 2048;   // beside the static shared memory
+template <int N, int KB, int MODE>
+cudaError_t prepare_up() {
+  static cudaError_t e = cudaFuncSetAttribute(k_up_tiles<N, KB, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kUpSmem);
+  return e;
+}
+
+template <int N, int KB, int MODE>
+cudaError_t launch_up(const ConvTC &c, cudaStream_t s, int sms, const CUtensorMap &ta, UpArgs a) {
+  auto fn = encode_fn();
+  const cudaError_t attr = prepare_up<N, KB, MODE>();
+  if (attr != cudaSuccess) return attr;
+  // weights [rows][cin]: {cin, 4 up_cout} or {cin, 4 cout}; box {KB, N}
+  CUtensorMap tb;
+  const cuuint32_t one[2] = {1, 1};
+  const cuuint64_t bdim[2] = {cuuint64_t(c.cin), cuuint64_t(4) * (MODE == kUp ? c.up_cout : c.cout)};
+  const cuuint64_t bstr[1] = {cuuint64_t(c.cin) * 2};
+  const cuuint32_t bbox[2] = {cuuint32_t(KB), cuuint32_t(N)};
+  if (fn(&tb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<bf16 *>(c.w), bdim, bstr, bbox, one,
+         CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle_of(KB), CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+    return cudaErrorInvalidValue;
+  const int wbytes = a.units * N * KB * 2, unit = kM * KB * 2;
+  a.stages = std::min(kUpStages, (kUpSmem - 1024 - wbytes) / unit);
+  const int nblk = c.cout / N, ctas = std::max(1, std::min(a.tiles, sms / nblk));
+  k_up_tiles<N, KB, MODE><<<dim3(unsigned(ctas), unsigned(nblk)), kRowThreads, 1024 + wbytes + a.stages * unit, s>>>(
+      ta, tb, a);
+  return cudaGetLastError();
+}
+
+template <int KB, int MODE>
+cudaError_t launch_up_kb(const ConvTC &c, cudaStream_t s, int sms) {
+  auto fn = encode_fn();
+  if (!fn) return cudaErrorNotSupported;
+  UpArgs a;
+  a.out = c.out;
+  a.out_cs = c.out_cs;
+  a.out_off = c.out_off;
+  a.bias = c.bias;
+  a.B = c.B;
+  a.H = c.H;
+  a.W = c.W;
+  a.log_bw = c.W >= kM ? 7 : 31 - __builtin_clz(unsigned(c.W));
+  const int bw = 1 << a.log_bw, bh = kM >> a.log_bw;
+  a.tiles_w = (c.W + bw - 1) / bw;
+  a.tiles_h = (c.H + bh - 1) / bh;
+  const long long tiles = (long long)a.tiles_w * a.tiles_h * c.B;
+  if (tiles >= (1LL << 31)) return cudaErrorNotSupported;
+  a.tiles = int(tiles);
+  a.in_off = c.in_off;
+  a.kchunks = c.cin / KB;
+  a.units = (MODE == kUp ? 1 : 4) * a.kchunks;
+  a.n_base = c.n_base;
+  a.up_cout = c.up_cout;
+  a.ncols = MODE == kUp ? 0 : c.cout;
+  a.wide = wide_stores(c);
+  a.y = c.y;
+  a.y_cs = c.y_cs;
+  a.y_off = c.y_off;
+  a.db = c.db;
+  a.err = c.err;
+  // Columns a CTA: the fewest column-tiles in the longest CTA's sequence (a tile
+  // also costs about 32 columns' time for its pixels), wider on a tie; at least 3
+  // units beside the weights.
+  int best = 0;
+  long long best_cost = 0;
+  for (int n : {256, 128, 64}) {
+    if (c.cout % n || (MODE != kUp && n == 256) || c.cout / n > sms) continue;
+    if ((long long)a.units * n * KB * 2 + 3 * kM * KB * 2 + 1024 > kUpSmem) continue;
+    const long long per = sms / (c.cout / n), cost = (tiles + per - 1) / per * (n + 32);
+    if (!best || cost < best_cost) {
+      best = n;
+      best_cost = cost;
+    }
+  }
+  if (!best) return cudaErrorNotSupported;
+  CUtensorMap ta;
+  const cuuint32_t one[5] = {1, 1, 1, 1, 1};
+  const cuuint64_t e = 2, cs = c.in_cs;   // bytes per element
+  CUresult r;
+  if (MODE == kUp) {
+    // input {channels, W, H, B}; box {KB, bw, bh, 1}
+    const cuuint64_t dim[4] = {cs, cuuint64_t(c.W), cuuint64_t(c.H), cuuint64_t(c.B)};
+    const cuuint64_t str[3] = {cs * e, cs * e * c.W, cs * e * c.W * c.H};
+    const cuuint32_t box[4] = {cuuint32_t(KB), cuuint32_t(bw), cuuint32_t(bh), 1};
+    r = fn(&ta, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<bf16 *>(c.in), dim, str, box, one,
+           CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle_of(KB), CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  } else {
+    // the output gradient [B][2H][2W][in_cs] as {channels, c, x, a, B H}
+    const cuuint64_t dim[5] = {cs, 2, cuuint64_t(c.W), 2, cuuint64_t(c.B) * c.H};
+    const cuuint64_t str[4] = {cs * e, cs * e * 2, cs * e * 2 * c.W, cs * e * 4 * c.W};
+    const cuuint32_t box[5] = {cuuint32_t(KB), 1, cuuint32_t(bw), 1, cuuint32_t(bh)};
+    r = fn(&ta, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<bf16 *>(c.in), dim, str, box, one,
+           CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle_of(KB), CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  }
+  if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
+  if (best == 64) return launch_up<64, KB, MODE>(c, s, sms, ta, a);
+  if (MODE != kUp || best == 128) return launch_up<128, KB, MODE>(c, s, sms, ta, a);
+  if constexpr (MODE == kUp) return launch_up<256, KB, MODE>(c, s, sms, ta, a);
+  return cudaErrorNotSupported;
+}
+
+template <int KB>
+cudaError_t prepare_up_kb() {
+  for (cudaError_t e : {prepare_up<64, KB, kUp>(), prepare_up<128, KB, kUp>(), prepare_up<256, KB, kUp>(),
+                        prepare_up<64, KB, kUpBack>(), prepare_up<128, KB, kUpBack>(), prepare_up<64, KB, kUpBackY>(),
+                        prepare_up<128, KB, kUpBackY>()})
+    if (e != cudaSuccess) return e;
+  return cudaSuccess;
+}
+
 int sm_count() {
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
@@ -1546,6 +1902,8 @@ int sm_count() {
 
 cudaError_t conv3x3_tc_prepare() {
   cudaError_t e = tc::prepare_n<32>();
+  if (e == cudaSuccess) e = tc::prepare_up_kb<32>();
+  if (e == cudaSuccess) e = tc::prepare_up_kb<64>();
   if (e == cudaSuccess) e = tc::prepare_n<64>();
   if (e == cudaSuccess) e = tc::prepare_n<128>();
   if (e == cudaSuccess) e = tc::prepare_n<256>();
@@ -1644,12 +2002,41 @@ cudaError_t conv_in_tc(const float2 *x, const __nv_bfloat16 *w, int wcin, const 
   return cudaGetLastError();
 }
 
+cudaError_t conv_up_tc(const ConvTC &c, cudaStream_t s) {
+  const int total = 4 * c.up_cout, step = std::min(total, 256);
+  if (c.up_cout < 1 || c.up_cout % 16 || total % step || !conv3x3_tc_supported(c.cin, step, c.in_cs, c.in_off, c.out_cs, c.out_off, c.W))
+    return cudaErrorNotSupported;
+  ConvTC q = c;
+  q.cout = total;
+  q.n_base = 0;
+  if (total % 64 == 0 && c.cin % 32 == 0) {
+    const int sms = tc::sm_count();
+    if (sms < 1) return cudaErrorInvalidValue;
+    const cudaError_t e = c.cin % 64 == 0 ? tc::launch_up_kb<64, tc::kUp>(q, s, sms) : tc::launch_up_kb<32, tc::kUp>(q, s, sms);
+    if (e != cudaErrorNotSupported) return e;
+  }
+  for (q.n_base = 0; q.n_base < total; q.n_base += step) {
+    q.cout = step;
+    const cudaError_t e = conv3x3_tc(q, s);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
 cudaError_t conv_upback_tc(const ConvTC &c, cudaStream_t s) {
   if (!conv3x3_tc_supported(c.cin, c.cout, c.in_cs, c.in_off, c.out_cs, c.out_off, c.W) ||
       (long long)c.B * c.H >= (1LL << 31))
     return cudaErrorNotSupported;
   const int sms = tc::sm_count();
   if (sms < 1) return cudaErrorInvalidValue;
+  if (c.cin % 32 == 0 && c.cout % 64 == 0 && !(c.y && (c.y_cs % 8 || c.y_off % 8 || !c.db))) {
+    const cudaError_t e = c.cin % 64 == 0 ? (c.y ? tc::launch_up_kb<64, tc::kUpBackY>(c, s, sms)
+                                                 : tc::launch_up_kb<64, tc::kUpBack>(c, s, sms))
+                                          : (c.y ? tc::launch_up_kb<32, tc::kUpBackY>(c, s, sms)
+                                                 : tc::launch_up_kb<32, tc::kUpBack>(c, s, sms));
+    if (e != cudaErrorNotSupported) return e;
+  }
+  if (c.y) return cudaErrorNotSupported;
   const int BW = c.W >= tc::kM ? tc::kM : (1 << (31 - __builtin_clz(unsigned(c.W))));
   const long long tiles = (long long)((c.W + BW - 1) / BW) * ((c.H + tc::kM / BW - 1) / (tc::kM / BW)) * c.B;
   int n = c.cout, nblk = 1;

@@ -518,7 +518,8 @@ struct ConvTC {
   int up_cout = 0;
   int n_base = 0;
   // the same convolution with more in its epilogue, or cudaErrorNotSupported
-  // (the row kernel has them: cin = cout up to 128, images from 128 pixels wide):
+  // (the row kernel has them: cin = cout up to 128, images from 128 pixels wide; y
+  // also the transposed convolution's data gradient):
   // pool: also the 2 x 2 average pool of the output, [B][H / 2][W / 2][cout].
   // y: the output is the gradient of y, relu's output; it is 0 where y (channels
   // y_off .. in rows of y_cs) is not positive, and its sums over all pixels are
@@ -530,6 +531,8 @@ struct ConvTC {
 };
 bool conv3x3_tc_supported(int cin, int cout, int in_cs, int in_off, int out_cs, int out_off, int W);
 cudaError_t conv3x3_tc(const ConvTC &c, cudaStream_t s);
+// all 4 up_cout columns of the transposed convolution (cout and n_base are not used)
+cudaError_t conv_up_tc(const ConvTC &c, cudaStream_t s);
 // sets the kernels' shared-memory attributes (before any stream capture)
 cudaError_t conv3x3_tc_prepare();
 // data gradient of the 2x2 stride-2 transposed convolution on the tensor

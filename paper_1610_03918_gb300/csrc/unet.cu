@@ -986,11 +986,17 @@ void weights_to_bf16(pic_unet *u) {
 
 // data gradient of the transposed convolution of level l on the tensor cores:
 // a GEMM of the output gradient's 4 children per input pixel (K = 4 x cout)
-// with the master-order weights; false where the kernel does not apply
-bool up_back_tc(pic_unet *u, int l, bf16 *gin) {
+// with the master-order weights; false where the kernel does not apply.
+// before and y: as conv_back_data's
+bool up_back_tc(pic_unet *u, int l, bf16 *gin, int before = -1, const bf16 *y = nullptr) {
   if (u->conv_impl != 0) return false;
   const pic_unet::Up &up = u->up[l];
   ConvTC c;
+  if (before >= 0) {
+    c.y = y;
+    c.y_cs = up.cin;
+    c.db = u->G + u->conv[before].b_off;
+  }
   c.in = u->gcat[l];
   c.in_cs = 2 * kC[l];
   c.in_off = 0;
@@ -1035,8 +1041,8 @@ bool up_wgrad_tc(pic_unet *u, int l, const bf16 *hin) {
   return true;
 }
 
-// the transposed convolution of level l on the tensor cores (GEMM columns in
-// launches of at most 256); false where the kernel does not apply
+// the transposed convolution of level l on the tensor cores; false where the
+// kernels do not apply
 bool up_tc(pic_unet *u, int l, const bf16 *in, int in_cs) {
   if (u->conv_impl != 0) return false;
   const pic_unet::Up &up = u->up[l];
@@ -1056,14 +1062,7 @@ bool up_tc(pic_unet *u, int l, const bf16 *in, int in_cs) {
   c.relu = 0;
   c.err = u->d_err;
   c.up_cout = up.cout;
-  const int total = 4 * up.cout, step = total > 256 ? 256 : total;
-  if (!conv3x3_tc_supported(up.cin, step, in_cs, 0, c.out_cs, 0, c.W)) return false;
-  for (int n0 = 0; n0 < total; n0 += step) {
-    c.cout = step;
-    c.n_base = n0;
-    if (conv3x3_tc(c, u->stream) != cudaSuccess) return false;
-  }
-  return true;
+  return conv_up_tc(c, u->stream) == cudaSuccess;
 }
 
 // keep_input: also the BF16 copy of the input padded to kCin0 channels, which
@@ -1120,21 +1119,27 @@ void backward(pic_unet *u) {
   k_head_back<true><<<int(std::min<long long>((pix(u, 0) + 63) / 64, 8LL * u->num_sms)), 256, 0, u->stream>>>(
       u->dy, u->dout[0], u->P + u->head_w, u->dpre[0], u->G + u->head_w, u->G + u->head_b,
       u->G + u->conv[D0B].b_off, pix(u, 0));
-  // decoder, from the output up
-  bf16 *g = nullptr;
+  // decoder, from the output up; dpre: the gradient before the ReLU of the level's last layer
+  const bf16 *dpre = u->dpre[0];
   for (int l = 0; l <= 2; ++l) {
     const int C = kC[l];
     const int ca = (l == 2) ? D2A : (l == 1) ? D1A : D0A;
-    if (l > 0) relu_back(u, ca + 1, g, C, 0, u->dout[l], C, 0, l);
-    block_back(u, ca, ca + 1, u->dpre[l], u->da[l], u->gda[l], u->cat[l], 2 * C, 0, u->gcat[l], 2 * C, l);
+    block_back(u, ca, ca + 1, dpre, u->da[l], u->gda[l], u->cat[l], 2 * C, 0, u->gcat[l], 2 * C, l);
     // transposed conv: gradient at its input (the output of level l+1) from gcat[:, 0:C]
     const pic_unet::Up &up = u->up[l];
     const int hl = u->H >> (l + 1), wl = u->W >> (l + 1);
     const bf16 *hin = (l == 2) ? u->b3 : u->dout[l + 1];
     bf16 *gin = (l == 2) ? u->gb3 : u->gdout[l + 1];
-    if (!up_back_tc(u, l, gin))
-      k_up_back_data<<<gridn((long long)pix(u, l + 1) * up.cin), 256, 0, u->stream>>>(
-          u->gcat[l], 2 * C, 0, up.cout, u->P + up.w_off, gin, up.cin, u->B, hl, wl);
+    // and through the ReLU of that level's last layer
+    const int last = (l == 2) ? E3B : (l == 1) ? D2B : D1B;
+    dpre = gin;
+    if (!up_back_tc(u, l, gin, last, hin)) {
+      if (!up_back_tc(u, l, gin))
+        k_up_back_data<<<gridn((long long)pix(u, l + 1) * up.cin), 256, 0, u->stream>>>(
+            u->gcat[l], 2 * C, 0, up.cout, u->P + up.w_off, gin, up.cin, u->B, hl, wl);
+      relu_back(u, last, gin, up.cin, 0, hin, up.cin, 0, l + 1);
+      dpre = u->dpre[l + 1];
+    }
     if (!up_wgrad_tc(u, l, hin)) {
       const int rows = u->B * hl;
       const int tiles = ((up.cin + 31) / 32) * ((up.cout + 31) / 32) * 4;
@@ -1144,11 +1149,9 @@ void backward(pic_unet *u) {
       k_up_back_w<<<dim3(groups, ((up.cin + 31) / 32) * ((up.cout + 31) / 32), 4), 256, 0, u->stream>>>(
           hin, up.cin, u->gcat[l], 2 * C, 0, up.cout, u->G + up.w_off, u->G + up.b_off, u->B, hl, wl, rpc);
     }
-    g = gin;
   }
   // bottleneck
-  relu_back(u, E3B, u->gb3, C3, 0, u->b3, C3, 0, 3);
-  block_back(u, E3A, E3B, u->dpre[3], u->a[3], u->gx[3], u->p[3], kC[2], 0, u->gp[3], kC[2], 3);
+  block_back(u, E3A, E3B, dpre, u->a[3], u->gx[3], u->p[3], kC[2], 0, u->gp[3], kC[2], 3);
   // encoder, back down: the pool's gradient joins the skip gradient gcat[l][C:2C]
   // inside the ReLU's backward
   for (int l = 2; l >= 0; --l) {
@@ -1652,11 +1655,7 @@ pic_status pic_upconv_bf16(int32_t impl, int32_t B, int32_t H, int32_t W, const 
   c.err = err;
   c.up_cout = cout;
   pic_status st = cudaGetLastError() == cudaSuccess ? PIC_OK : PIC_ECUDA;
-  for (int n0 = 0; st == PIC_OK && n0 < total; n0 += step) {
-    c.cout = step;
-    c.n_base = n0;
-    if (picgb::conv3x3_tc(c, s) != cudaSuccess) st = PIC_ECUDA;
-  }
+  if (st == PIC_OK && picgb::conv_up_tc(c, s) != cudaSuccess) st = PIC_ECUDA;
   if (cudaStreamSynchronize(s) != cudaSuccess && st == PIC_OK) st = PIC_ECUDA;
   cudaFree(wt);
   return st == PIC_OK ? word.read("convolution") : st;

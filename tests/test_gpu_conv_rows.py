@@ -68,7 +68,14 @@ def test_store_width_changes_no_result(W, cin, cout):
         assert np.all(np.delete(out, np.s_[off:off + cout], axis=3) == 7.0)
 
 
-@pytest.mark.parametrize("H, W, cin, cout", [(5, 24, 64, 32), (3, 130, 128, 64), (4, 64, 256, 128)])
+@pytest.mark.parametrize("H, W, cin, cout", [
+    (5, 24, 64, 32), (3, 130, 128, 64), (4, 64, 256, 128),
+    (40, 300, 64, 32),      # several tiles a CTA, a ragged column block
+    (97, 128, 128, 64),     # 256 columns at once
+    (1, 8, 32, 16),         # a part of one tile; 64 columns, K = 32
+    (33, 9, 96, 32),        # three units, tiles of 8 x 16 pixels
+    (70, 90, 256, 128),     # 512 columns
+])
 def test_upconv_store_width_changes_no_result(H, W, cin, cout):
     import ctypes
     import torch
