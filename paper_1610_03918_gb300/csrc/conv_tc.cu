@@ -24,7 +24,7 @@
 // its TMEM) instead of hanging.
 //
 // The same kernel, in further modes, computes the 2x2 stride-2 transposed
-// convolution and its data gradient; k_wgrad_tc below computes the weight
+// convolution and its data gradient; k_wgrad_rows below computes the weight
 // gradients of both kinds of convolution with both operands MN-major.
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -141,6 +141,18 @@ __device__ __forceinline__ void mma_bf16_lo(uint32_t tmem_d, uint32_t da, uint32
       "mov.b64 b, {%2, %3};\n\t"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, p;\n\t}" ::"r"(tmem_d),
       "r"(da), "r"(db), "r"(hi), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+// the same with a high word for each operand
+__device__ __forceinline__ void mma_bf16_lo(uint32_t tmem_d, uint32_t da, uint32_t ha, uint32_t db, uint32_t hb,
+                                            uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\t"
+      "setp.ne.b32 p, %6, 0;\n\t"
+      "mov.b64 a, {%1, %2};\n\t"
+      "mov.b64 b, {%3, %4};\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n\t}" ::"r"(tmem_d),
+      "r"(da), "r"(ha), "r"(db), "r"(hb), "r"(idesc), "r"(accumulate)
       : "memory");
 }
 // One lane of a converged warp.  The MMA warps run their loops with all lanes
@@ -1172,40 +1184,55 @@ __global__ void __launch_bounds__(kThreads, 1)
 //    The three horizontal taps are three N chunks of CI channels whose
 //    starts lie one pixel row apart (LBO = one row), so N = 3 CI covers
 //    dx = 0, 1, 2 at once, each chunk being the input shifted by dx - 1.
-//  * A, the gradient: three slots, slot s the dpre row hq + 1 - s (pixels w0
-//    .. w0 + KP - 1, zero fill off the image), one slot per vertical tap
-//    (dpre row hq + 1 - dy meets input row hq at tap dy), and a fourth slot
-//    of zeros.  M = 128 rows of D are slots of CO channels at LBO = one slot:
-//    CO = 32, all four slots in one MMA; CO = 64, slots {0, 1} and {2, 3}.
-// D row (s, co), column (dx, ci) thus accumulates dW[co][3 s + dx][ci] over
+//  * A, the gradient: three consecutive slots, slot s the dpre row hq - 1 + s
+//    (pixels w0 .. w0 + KP - 1, zero fill off the image), one slot per vertical
+//    tap (dpre row hq + 1 - dy meets input row hq at tap dy).  M = 128 rows of D
+//    are slots of CO channels at LBO = one slot: CO = 32, four slots in one MMA;
+//    CO = 64, slots {0, 1} and {2, 3}.  The fourth is whatever lies there: its
+//    rows of D are not read.
+// D row (s, co), column (dx, ci) thus accumulates dW[co][3 (2 - s) + dx][ci] over
 // the CTA's K blocks; the epilogue adds it to dW with vector atomics (FP32,
 // so the sum order, not the terms, depends on the grid).
-// UPW: the weight gradient of the 2x2 stride-2 transposed convolution,
-// dW[a][c][ci][co] = sum over input pixels p of in[p][ci] g[child (a, c) of p][co],
-// g its output gradient.  The four slots of A are the four children's tiles
-// of g (5-D boxes {CO, 1, 64, 1, 1} of g viewed as {channels, c, x, a, rows}),
-// B is the input row without a shift (N = CI), and D row (t, co), column ci
-// holds dW[t][ci][co]; the epilogue adds it with scalar atomics, consecutive
-// lanes on consecutive co.
+// A CTA goes down the rows of a pixel column, and each dpre row serves three K
+// blocks: a segment of up to NR - 2 input rows starts at slot 0 of the NR with the
+// dpre row above it.  Rows come GA (dpre) and GB (input) to a TMA box, because
+// what set the pace before was neither the tensor core nor memory but the one
+// thread that loaded three dpre rows and an input row anew for every K block:
+// 160 cycles a box, 640 a K block of 224 (32 x 32) to 768 (64 x 64) cycles of MMA.
+// Cold, batch 4: 64 -> 64 at 516 x 256 51.6 -> 43.8 us (MMA alone 21), 32 -> 32 at
+// 1032 x 512 69.0 -> 51.0 (a read of both tensors 40), 256 -> 256 at 129 x 64 70.9 ->
+// 49.0.
 constexpr int kWKP = 64;   // pixels per K block
+constexpr int kWKPB = kWKP + 16;   // the input row with 8-pixel margins
 
-template <int CO, int CI, int STAGES, bool UPW = false>
-struct WLayout {
-  static constexpr int KPB = kWKP + 16;   // the input row with 8-pixel margins
+constexpr uint32_t tmem_cols(uint32_t n) {
+  return n <= 32 ? 32 : n <= 64 ? 64 : n <= 128 ? 128 : n <= 256 ? 256 : 512;
+}
+
+template <int CO, int CI>
+struct WRing {
   static constexpr uint32_t SLOT = kWKP * CO * 2;
-  static constexpr uint32_t A_BYTES = 4 * SLOT;
-  static constexpr uint32_t B_TX = KPB * CI * 2;
-  static constexpr uint32_t B_BYTES = ((B_TX + 1023) / 1024) * 1024;
-  static constexpr uint32_t STAGE = A_BYTES + B_BYTES;
-  static constexpr uint32_t BAR_OFF = STAGES * STAGE;
+  static constexpr uint32_t ROW = kWKPB * CI * 2;      // an input row; groups of 8 pixels stay whole
+  static constexpr int GA = 4, GB = 2;                 // rows per TMA box
+  static constexpr int NR = CO == 32 ? 16 : 12;        // dpre rows
+  static constexpr int NB = CI == 64 ? 4 : 3;          // boxes of input rows
+  static constexpr int NA = NR / GA;
+  static constexpr uint32_t B_OFF = NR * SLOT;
+  static constexpr uint32_t BAR_OFF = B_OFF + (NB * GB * ROW + 1023) / 1024 * 1024;
   // allocated, never written: keeps every address the descriptors of the last
-  // stage can form inside this CTA's shared memory (the widest reading of
+  // input row can form inside this CTA's shared memory (the widest reading of
   // the B tile spans 3 CI rows of 8-row groups from row 55)
   static constexpr uint32_t TAIL = 6 * CI * CI + 112 * CI;
-  static constexpr uint32_t BYTES = BAR_OFF + (2 * STAGES + 1) * 8 + 16 + TAIL + 1024;
+  static constexpr uint32_t BYTES = BAR_OFF + (2 * NA + 2 * NB + 1) * 8 + 16 + TAIL + 1024;
+  static_assert(BYTES <= 227 * 1024 - 64, "shared memory");
   static constexpr int NM = CO == 32 ? 1 : 2;   // MMAs along M per 16 pixels
-  static constexpr int N = UPW ? CI : 3 * CI;
-  static constexpr uint32_t NCOLS = NM * N <= 32 ? 32 : NM * N <= 64 ? 64 : NM * N <= 128 ? 128 : NM * N <= 256 ? 256 : 512;
+  static constexpr int N = 3 * CI;
+  // A CTA's K blocks in turn go to NACC accumulators, which the epilogue adds in
+  // FP32: the tensor core truncates each sum, so the error grows with the sums
+  // an accumulator takes (relative error of 32 -> 32 at 4 x 1032 x 512, over 453
+  // accumulators 2.2e-6, over 304 3.5e-6, over 608 1.5e-6).
+  static constexpr int NACC = NM * N > 256 ? 1 : 2;
+  static constexpr uint32_t NCOLS = tmem_cols(NACC * NM * N);
 };
 
 // descriptor of an MN-major tile in the swizzled layout TMA wrote with rows
@@ -1222,18 +1249,230 @@ __host__ __device__ constexpr uint32_t instr_desc_mn() {
   return instr_desc<N>() | (1u << 15) | (1u << 16);
 }
 
+struct WRowArgs {
+  float *dw;           // [cout][9][cin]
+  int cin, cout, in_off, H, nwc;
+  long long rows;      // B x nwc pixel columns x H input rows
+  int *err;
+};
+
+template <int CO, int CI>
+__global__ void __launch_bounds__(kThreads, 1)
+    k_wgrad_rows(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, WRowArgs a) {
+  using L = WRing<CO, CI>;
+  constexpr int NA = L::NA, NB = L::NB, GA = L::GA, GB = L::GB;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  const uint32_t s0 = saddr(smem), sB = s0 + L::B_OFF, bar0 = s0 + L::BAR_OFF;
+  // boxes of dpre rows full, empty; of input rows full, empty; all done
+  const uint32_t afull = bar0, aempty = afull + 8 * NA, bfull = aempty + 8 * NA, bempty = bfull + 8 * NB,
+                 done = bempty + 8 * NB;
+  uint32_t *slot = reinterpret_cast<uint32_t *>(smem + L::BAR_OFF + (2 * NA + 2 * NB + 1) * 8);
+  __shared__ int s_fail;
+  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
+  const int ncib = a.cin / CI;
+  const int co0 = int(blockIdx.y) / ncib * CO, ci0 = int(blockIdx.y) % ncib * CI;
+  const long long t0 = a.rows * blockIdx.x / gridDim.x, t1 = a.rows * (blockIdx.x + 1) / gridDim.x;
+  const int nacc = int(min(t1 - t0, (long long)L::NACC));   // accumulators in use
+  if (tid == 0) {
+    for (int k = 0; k < 2 * (NA + NB) + 1; ++k) mbar_init(bar0 + 8 * k, 1);
+    s_fail = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) tmem_alloc(saddr(slot), L::NCOLS);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *slot;
+  // the segments: n input rows from h0 of pixel column col
+  long long t = t0, col = 0;
+  int h0 = 0, n = 0;
+  auto next = [&]() {
+    if (t >= t1) return false;
+    col = t / a.H;
+    h0 = int(t - col * a.H);
+    n = int(min(min(t1 - t, (long long)(a.H - h0)), (long long)(L::NR - 2)));
+    t += n;
+    return true;
+  };
+
+  if (warp == 0) {
+    if (lane == 0) {
+      uint32_t phase = ~0u;   // per dpre box: the parity its next release completes (the first round waits for none)
+      uint32_t bs = 0, bph = 1;
+      bool ok = true;
+      while (ok && next()) {
+        const int b = int(col / a.nwc), w0 = int(col - (long long)b * a.nwc) * kWKP;
+        int g = 0;
+        auto load_a = [&]() {
+          ok = ok && mbar_wait(aempty + 8 * g, (phase >> g) & 1);
+          if (!ok) return;
+          phase ^= 1u << g;
+          mbar_expect_tx(afull + 8 * g, GA * L::SLOT);
+          tma_load_4d(s0 + g * (GA * L::SLOT), &tmA, co0, w0, h0 - 1 + GA * g, b, afull + 8 * g);
+          g += 1;
+        };
+        load_a();
+        for (int i = 0; i < n && ok; i += GB) {
+          // input rows up to i + GB - 1 need dpre slots up to i + GB + 1 (the last: n + 1)
+          if (min(i + GB + 1, n + 1) >= GA * g) load_a();
+          ok = ok && mbar_wait(bempty + 8 * bs, bph);
+          if (!ok) break;
+          mbar_expect_tx(bfull + 8 * bs, GB * L::ROW);
+          tma_load_4d(sB + bs * (GB * L::ROW), &tmB, a.in_off + ci0, w0 - 8, h0 + i, b, bfull + 8 * bs);
+          if (++bs == NB) {
+            bs = 0;
+            bph ^= 1;
+          }
+        }
+      }
+      if (!ok) {
+        atomicExch(&s_fail, 1);
+        atomicCAS(a.err, 0, 1);
+      }
+    }
+  } else if (warp == 1) {
+    const bool leader = elect_one();
+    constexpr uint32_t idesc = instr_desc_mn<L::N>();
+    // descriptors: only the address field (16-byte units) varies; input rows from
+    // pixel w0 - 1 on (row 7 of a box row), the tap dx = 0 chunk
+    const uint64_t a64 = mn_desc<CO>(s0, L::SLOT), b64 = mn_desc<CI>(sB + 7 * (CI * 2), CI * 2);
+    const uint32_t da = uint32_t(a64), ha = uint32_t(a64 >> 32), db = uint32_t(b64), hb = uint32_t(b64 >> 32);
+    uint32_t phase = 0;       // per dpre box: the parity its next load completes
+    uint32_t bs = 0, bph = 0;
+    uint32_t acc = 0, any = 0;             // the accumulator, whether it holds anything
+    long long rows = 0, until = (t1 - t0) / nacc;   // K blocks so far, those up to the next accumulator
+    bool ok = true;
+    while (ok && next()) {
+      int g = 0, freed = 0;   // dpre boxes that have arrived, that are released
+      for (int i = 0; i < n && ok; ++i) {
+        if (i + 2 >= GA * g) {
+          ok = mbar_wait_warp(afull + 8 * g, (phase >> g) & 1);
+          phase ^= 1u << g;
+          g += 1;
+        }
+        if (i % GB == 0) ok = ok && mbar_wait_warp(bfull + 8 * bs, bph);
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t ra = da + i * (L::SLOT >> 4), rb = db + (bs * GB + i % GB) * (L::ROW >> 4);
+        const bool box_done = i % GB == GB - 1 || i + 1 == n;
+        if (leader) {
+#pragma unroll
+          for (int k = 0; k < kWKP / 16; ++k)
+#pragma unroll
+            for (int m = 0; m < L::NM; ++m)
+              mma_bf16_lo(tmem + acc + m * L::N, ra + m * (2 * L::SLOT >> 4) + k * (CO * 2), ha, rb + k * (CI * 2), hb, idesc,
+                          any | k);
+          if (box_done) mma_commit(bempty + 8 * bs);
+          // a box's last row is slot 0 of this window
+          if (i % GA == GA - 1 && i + 1 < n) mma_commit(aempty + 8 * freed);
+          if (i + 1 == n)
+            for (int q = freed; q < g; ++q) mma_commit(aempty + 8 * q);
+        }
+        if (i % GA == GA - 1) freed += 1;
+        any = 1;
+        if (++rows == until && L::NACC > 1 && rows < t1 - t0) {
+          acc += L::NM * L::N;
+          any = 0;
+          until = t1 - t0;
+        }
+        if (box_done && ++bs == NB) {
+          bs = 0;
+          bph ^= 1;
+        }
+      }
+    }
+    if (leader) mma_commit(done);
+    if (!ok && leader) {
+      atomicExch(&s_fail, 1);
+      atomicCAS(a.err, 0, 2);
+    }
+  }
+
+  // epilogue: warp w reads D rows 32 w .. 32 w + 31 of each accumulator
+  __syncwarp();
+  const bool ok = mbar_wait(done, 0);
+  tc_fence_after();
+  if (!ok) atomicCAS(a.err, 0, 3);
+  const bool add = __all_sync(0xffffffffu, ok && !s_fail);
+#pragma unroll
+  for (int m = 0; m < L::NM; ++m) {
+    const int row = 32 * warp + lane;                       // D row of MMA m
+    const int sl = CO == 32 ? warp : 2 * m + (row >> 6);    // A slot: vertical tap 2 - sl
+    const int co = co0 + (CO == 32 ? lane : (row & 63));
+    if (sl == 3) continue;                                  // warp-uniform: no tap
+    const uint32_t tl = tmem + (uint32_t(32 * warp) << 16) + m * L::N;
+    const bool odd = lane & 1;
+#pragma unroll 1
+    for (int n0 = 0; n0 < L::N; n0 += 16) {
+      uint32_t v[16];
+      tmem_ld16(tl + n0, v);
+      if (L::NACC > 1 && nacc > 1) {
+        uint32_t u[16];
+        tmem_ld16(tl + L::NM * L::N + n0, u);
+#pragma unroll
+        for (int q = 0; q < 16; ++q) v[q] = __float_as_uint(__uint_as_float(v[q]) + __uint_as_float(u[q]));
+      }
+      const int dx = n0 / CI, ci = ci0 + (n0 - dx * CI);
+      // L2 adds 32-byte sectors: the lanes of a pair take the two halves of one row's
+      // sector, then of the other's (64 -> 64: 48.0 -> 43.5 us; a row a lane took 11.7)
+      float *dst = a.dw + (size_t(co & ~1) * 9 + 3 * (2 - sl) + dx) * a.cin + ci + (odd ? 4 : 0);
+#pragma unroll
+      for (int q = 0; q < 16; q += 8) {
+        float x[4], y[4];   // of the even lane's row, of the odd lane's
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const float lo = __uint_as_float(v[q + k]), hi = __uint_as_float(v[q + 4 + k]);
+          const float got = __shfl_xor_sync(0xffffffffu, odd ? lo : hi, 1);
+          x[k] = odd ? got : lo;
+          y[k] = odd ? hi : got;
+        }
+        if (add) {
+          atomicAdd(reinterpret_cast<float4 *>(dst + q), make_float4(x[0], x[1], x[2], x[3]));
+          atomicAdd(reinterpret_cast<float4 *>(dst + q + 9 * size_t(a.cin)), make_float4(y[0], y[1], y[2], y[3]));
+        }
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0) tmem_dealloc(tmem, L::NCOLS);
+}
+
+// The weight gradient of the 2x2 stride-2 transposed convolution,
+// dW[a][c][ci][co] = sum over input pixels p of in[p][ci] g[child (a, c) of p][co],
+// g its output gradient, K blocks as above.  The four slots of A are the four
+// children's tiles of g (5-D boxes {CO, 1, 64, 1, 1} of g viewed as {channels, c,
+// x, a, rows}), B is the input row without a shift (N = CI), and D row (t, co),
+// column ci holds dW[t][ci][co]; the epilogue adds it with scalar atomics,
+// consecutive lanes on consecutive co.
+template <int CO, int CI, int STAGES>
+struct WLayout {
+  static constexpr uint32_t SLOT = kWKP * CO * 2;
+  static constexpr uint32_t A_BYTES = 4 * SLOT;
+  static constexpr uint32_t B_TX = kWKPB * CI * 2;
+  static constexpr uint32_t B_BYTES = ((B_TX + 1023) / 1024) * 1024;
+  static constexpr uint32_t STAGE = A_BYTES + B_BYTES;
+  static constexpr uint32_t BAR_OFF = STAGES * STAGE;
+  static constexpr uint32_t TAIL = WRing<CO, CI>::TAIL;   // as there
+  static constexpr uint32_t BYTES = BAR_OFF + (2 * STAGES + 1) * 8 + 16 + TAIL + 1024;
+  static constexpr int NM = CO == 32 ? 1 : 2;   // MMAs along M per 16 pixels
+  static constexpr int N = CI;
+  static constexpr uint32_t NCOLS = tmem_cols(NM * N);
+};
+
 struct WArgs {
-  float *dw;           // [cout][9][cin]; UPW: [4][cin][cout]
-  int cin, cout, in_off, a_off, H, nwc;
+  float *dw;           // [4][cin][cout]
+  int cin, cout, a_off, H, nwc;
   long long nkb;       // K blocks: B H rows x nwc pixel chunks
   long long per_cta;   // K blocks per CTA along the grid's first index
   int *err;
 };
 
-template <int CO, int CI, int STAGES, bool UPW = false>
+template <int CO, int CI, int STAGES>
 __global__ void __launch_bounds__(kThreads, 1)
-    k_wgrad_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, WArgs a) {
-  using L = WLayout<CO, CI, STAGES, UPW>;
+    k_upwgrad_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, WArgs a) {
+  using L = WLayout<CO, CI, STAGES>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t s0 = saddr(smem);
@@ -1248,14 +1487,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   const long long k1 = k0 + a.per_cta < a.nkb ? k0 + a.per_cta : a.nkb;
   const int nk = int(k1 - k0);   // at least 1 (the host sizes the grid so)
 
-  // the fourth A slot of every stage holds zeros (the MMA's rows 96..127 for
-  // CO = 32, 64..127 of the second MMA for CO = 64; discarded)
-  if (!UPW) {
-    for (int st = 0; st < STAGES; ++st)
-      for (uint32_t o = 16 * tid; o < L::SLOT; o += 16 * kThreads)
-        *reinterpret_cast<uint4 *>(smem + st * L::STAGE + 3 * L::SLOT + o) = make_uint4(0, 0, 0, 0);
-    fence_async_smem();
-  }
   if (tid == 0) {
     for (int s = 0; s < STAGES; ++s) {
       mbar_init(bar0 + 8 * s, 1);
@@ -1286,15 +1517,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int w0 = int(g - r * a.nwc) * kWKP;
       const int b = int(r / a.H), hq = int(r - (long long)b * a.H);
       const uint32_t st = s0 + s * L::STAGE;
-      mbar_expect_tx(bar0 + 8 * s, (UPW ? 4 : 3) * L::SLOT + L::B_TX);
-      if (UPW) {
-        for (int t = 0; t < 4; ++t)
-          tma_load_5d(st + t * L::SLOT, &tmA, a.a_off + co0, t & 1, w0, t >> 1, int(r), bar0 + 8 * s);
-      } else {
-        for (int sl = 0; sl < 3; ++sl)
-          tma_load_4d(st + sl * L::SLOT, &tmA, co0, w0, hq + 1 - sl, b, bar0 + 8 * s);
-      }
-      tma_load_4d(st + L::A_BYTES, &tmB, a.in_off + ci0, w0 - 8, hq, b, bar0 + 8 * s);
+      mbar_expect_tx(bar0 + 8 * s, 4 * L::SLOT + L::B_TX);
+      for (int t = 0; t < 4; ++t)
+        tma_load_5d(st + t * L::SLOT, &tmA, a.a_off + co0, t & 1, w0, t >> 1, int(r), bar0 + 8 * s);
+      tma_load_4d(st + L::A_BYTES, &tmB, ci0, w0 - 8, hq, b, bar0 + 8 * s);
     }
   } else if (tid == 32) {
     constexpr uint32_t idesc = instr_desc_mn<L::N>();
@@ -1310,9 +1536,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       const uint32_t st = s0 + s * L::STAGE;
 #pragma unroll
       for (int k = 0; k < kWKP / 16; ++k) {
-        // input rows 7 + 16 k ..: pixel w0 - 1 + 16 k on, the tap dx = 0 chunk
-        // (UPW: rows 8 + 16 k .., pixel w0 + 16 k on)
-        const uint64_t db = mn_desc<CI>(st + L::A_BYTES + ((UPW ? 8 : 7) + 16 * k) * (CI * 2), CI * 2);
+        // input rows 8 + 16 k ..: pixel w0 + 16 k on
+        const uint64_t db = mn_desc<CI>(st + L::A_BYTES + (8 + 16 * k) * (CI * 2), CI * 2);
 #pragma unroll
         for (int m = 0; m < L::NM; ++m) {
           const uint64_t da = mn_desc<CO>(st + 2 * m * L::SLOT + 16 * k * (CO * 2), L::SLOT);
@@ -1332,28 +1557,18 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
   for (int m = 0; m < L::NM; ++m) {
     const int row = 32 * warp + lane;                       // D row of MMA m
-    const int sl = CO == 32 ? warp : 2 * m + (row >> 6);    // A slot: vertical tap (UPW: child)
+    const int sl = CO == 32 ? warp : 2 * m + (row >> 6);    // A slot: the child
     const int co = co0 + (CO == 32 ? lane : (row & 63));
-    if (!UPW && sl == 3) continue;                          // warp-uniform: the zero slot
     const uint32_t tl = tmem + (uint32_t(32 * warp) << 16) + m * L::N;
 #pragma unroll 1
     for (int n0 = 0; n0 < L::N; n0 += 16) {
       uint32_t v[16];
       tmem_ld16(tl + n0, v);
-      if (UPW) {
-        // consecutive lanes: consecutive co of one (t, ci) row of dW
-        if (ok && !s_fail) {
-          float *dst = a.dw + (size_t(sl) * a.cin + ci0 + n0) * a.cout + co;
+      // consecutive lanes: consecutive co of one (t, ci) row of dW
+      if (ok && !s_fail) {
+        float *dst = a.dw + (size_t(sl) * a.cin + ci0 + n0) * a.cout + co;
 #pragma unroll
-          for (int q = 0; q < 16; ++q) atomicAdd(dst + size_t(q) * a.cout, __uint_as_float(v[q]));
-        }
-      } else if (ok && !s_fail) {
-        const int dx = n0 / CI, ci = ci0 + (n0 - dx * CI);
-        float4 *dst = reinterpret_cast<float4 *>(a.dw + (size_t(co) * 9 + 3 * sl + dx) * a.cin + ci);
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-          atomicAdd(dst + q, make_float4(__uint_as_float(v[4 * q]), __uint_as_float(v[4 * q + 1]),
-                                         __uint_as_float(v[4 * q + 2]), __uint_as_float(v[4 * q + 3])));
+        for (int q = 0; q < 16; ++q) atomicAdd(dst + size_t(q) * a.cout, __uint_as_float(v[q]));
       }
     }
   }
@@ -1665,29 +1880,31 @@ cudaError_t launch_upb_n(const ConvTC &c, cudaStream_t s, int nblk) {
 }
 
 constexpr int kWStages = 3;
-template <int CO, int CI, bool UPW = false>
+template <int CO, int CI>
 cudaError_t prepare_wgrad() {
-  static cudaError_t e = cudaFuncSetAttribute(k_wgrad_tc<CO, CI, kWStages, UPW>,
+  static cudaError_t e = cudaFuncSetAttribute(k_wgrad_rows<CO, CI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              int(WRing<CO, CI>::BYTES));
+  return e;
+}
+template <int CO, int CI>
+cudaError_t prepare_upwgrad() {
+  static cudaError_t e = cudaFuncSetAttribute(k_upwgrad_tc<CO, CI, kWStages>,
                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              int(WLayout<CO, CI, kWStages, UPW>::BYTES));
+                                              int(WLayout<CO, CI, kWStages>::BYTES));
   return e;
 }
 
-// CTAs of one wave over yb (co, ci) blocks, each a run of K blocks (at least one)
+// CTAs of one wave over yb (co, ci) blocks, each a run of the n units (at least one)
 template <class L>
-long long wgrad_split(WArgs &a, int sms, int yb) {
+long long wave_split(long long n, int sms, int yb) {
   const int res_smem = int((227u * 1024u) / L::BYTES), res_tmem = int(512u / L::NCOLS);
   const int res = res_smem < res_tmem ? (res_smem > 0 ? res_smem : 1) : res_tmem;
-  long long splits = ((long long)sms * res + yb - 1) / yb;
-  if (splits > a.nkb) splits = a.nkb;
-  if (splits < 1) splits = 1;
-  a.per_cta = (a.nkb + splits - 1) / splits;
-  return (a.nkb + a.per_cta - 1) / a.per_cta;
+  return std::max(1LL, std::min(n, (long long)sms * res / yb));
 }
 
 template <int CO, int CI>
 cudaError_t launch_wgrad(const WgradTC &g, cudaStream_t s, int sms) {
-  using L = WLayout<CO, CI, kWStages>;
+  using L = WRing<CO, CI>;
   auto fn = encode_fn();
   if (!fn) return cudaErrorNotSupported;
   const cudaError_t attr = prepare_wgrad<CO, CI>();
@@ -1695,48 +1912,51 @@ cudaError_t launch_wgrad(const WgradTC &g, cudaStream_t s, int sms) {
   const cuuint64_t e = 2;
   const cuuint32_t one[4] = {1, 1, 1, 1};
   CUtensorMap ta, tb;
-  // the gradient [B][H][W][cout] as {cout, W, H, B}, boxes {CO, 64 pixels}
+  // the gradient [B][H][W][cout] as {cout, W, H, B}, boxes {CO, 64 pixels, GA rows}
   const cuuint64_t adim[4] = {cuuint64_t(g.cout), cuuint64_t(g.W), cuuint64_t(g.H), cuuint64_t(g.B)};
   const cuuint64_t astr[3] = {cuuint64_t(g.cout) * e, cuuint64_t(g.cout) * e * g.W, cuuint64_t(g.cout) * e * g.W * g.H};
-  const cuuint32_t abox[4] = {cuuint32_t(CO), cuuint32_t(kWKP), 1, 1};
+  const cuuint32_t abox[4] = {cuuint32_t(CO), cuuint32_t(kWKP), L::GA, 1};
   if (fn(&ta, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<bf16 *>(g.dpre), adim, astr, abox, one,
          CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle_of(CO), CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return cudaErrorInvalidValue;
-  // the input [B][H][W][in_cs] as {in_cs, W, H, B}, boxes {CI, 80 pixels}
+  // the input [B][H][W][in_cs] as {in_cs, W, H, B}, boxes {CI, 80 pixels, GB rows}
   const cuuint64_t bdim[4] = {cuuint64_t(g.in_cs), cuuint64_t(g.W), cuuint64_t(g.H), cuuint64_t(g.B)};
   const cuuint64_t bstr[3] = {cuuint64_t(g.in_cs) * e, cuuint64_t(g.in_cs) * e * g.W,
                               cuuint64_t(g.in_cs) * e * g.W * g.H};
-  const cuuint32_t bbox[4] = {cuuint32_t(CI), cuuint32_t(L::KPB), 1, 1};
+  const cuuint32_t bbox[4] = {cuuint32_t(CI), cuuint32_t(kWKPB), L::GB, 1};
   if (fn(&tb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<bf16 *>(g.in), bdim, bstr, bbox, one,
          CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle_of(CI), CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return cudaErrorInvalidValue;
-  WArgs a;
+  WRowArgs a;
   a.dw = g.dw;
   a.cin = g.cin;
   a.cout = g.cout;
   a.in_off = g.in_off;
-  a.a_off = 0;
   a.H = g.H;
   a.nwc = (g.W + kWKP - 1) / kWKP;
-  a.nkb = (long long)g.B * g.H * a.nwc;
+  a.rows = (long long)g.B * g.H * a.nwc;
   a.err = g.err;
   // one wave: the CTAs that fit on the SMs at once (shared memory, TMEM
-  // columns), shared out over the (co, ci) blocks, each a run of K blocks
+  // columns), shared out over the (co, ci) blocks; two waves where one does not
+  // come out even, so that no accumulator takes more than its share (256 -> 256 at
+  // 4 x 129 x 64, relative error: 1.55e-6 with 9 CTAs a block, 1.41e-6 with 10, in two
+  // waves of 19 6.5e-7; 40 and 49 us)
   const int yb = (g.cout / CO) * (g.cin / CI);
-  const long long splits = wgrad_split<L>(a, sms, yb);
-  k_wgrad_tc<CO, CI, kWStages><<<dim3(unsigned(splits), unsigned(yb)), kThreads, L::BYTES, s>>>(ta, tb, a);
+  const long long wave = wave_split<L>(1LL << 40, sms, 1);   // CTAs resident at once
+  const long long splits = wave_split<L>(a.rows, wave % yb && yb < wave ? 2 * sms : sms, yb);
+  k_wgrad_rows<CO, CI><<<dim3(unsigned(splits), unsigned(yb)), kThreads, L::BYTES, s>>>(ta, tb, a);
   return cudaGetLastError();
 }
 
 template <int CO>
 cudaError_t launch_upw(const UpWgradTC &g, cudaStream_t s, int sms) {
   constexpr int CI = 64;
-  using L = WLayout<CO, CI, kWStages, true>;
+  using L = WLayout<CO, CI, kWStages>;
   auto fn = encode_fn();
   if (!fn) return cudaErrorNotSupported;
-  const cudaError_t attr = prepare_wgrad<CO, CI, true>();
+  const cudaError_t attr = prepare_upwgrad<CO, CI>();
   if (attr != cudaSuccess) return attr;
   const cuuint64_t e = 2;
   const cuuint32_t one[5] = {1, 1, 1, 1, 1};
@@ -1754,7 +1974,7 @@ cudaError_t launch_upw(const UpWgradTC &g, cudaStream_t s, int sms) {
   // the input [B][H][W][cin] as {cin, W, H, B}, boxes {64, 80 pixels} from 8 before
   const cuuint64_t bdim[4] = {cuuint64_t(g.cin), cuuint64_t(g.W), cuuint64_t(g.H), cuuint64_t(g.B)};
   const cuuint64_t bstr[3] = {cuuint64_t(g.cin) * e, cuuint64_t(g.cin) * e * g.W, cuuint64_t(g.cin) * e * g.W * g.H};
-  const cuuint32_t bbox[4] = {cuuint32_t(CI), cuuint32_t(L::KPB), 1, 1};
+  const cuuint32_t bbox[4] = {cuuint32_t(CI), cuuint32_t(kWKPB), 1, 1};
   if (fn(&tb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<bf16 *>(g.in), bdim, bstr, bbox, one,
          CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle_of(CI), CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
@@ -1763,15 +1983,15 @@ cudaError_t launch_upw(const UpWgradTC &g, cudaStream_t s, int sms) {
   a.dw = g.dw;
   a.cin = g.cin;
   a.cout = g.cout;
-  a.in_off = 0;
   a.a_off = g.g_off;
   a.H = g.H;
   a.nwc = (g.W + kWKP - 1) / kWKP;
   a.nkb = (long long)g.B * g.H * a.nwc;
   a.err = g.err;
   const int yb = (g.cout / CO) * (g.cin / CI);
-  const long long splits = wgrad_split<L>(a, sms, yb);
-  k_wgrad_tc<CO, CI, kWStages, true><<<dim3(unsigned(splits), unsigned(yb)), kThreads, L::BYTES, s>>>(ta, tb, a);
+  const long long splits = wave_split<L>(a.nkb, sms, yb);
+  a.per_cta = (a.nkb + splits - 1) / splits;
+  k_upwgrad_tc<CO, CI, kWStages><<<dim3(unsigned((a.nkb + a.per_cta - 1) / a.per_cta), unsigned(yb)), kThreads, L::BYTES, s>>>(ta, tb, a);
   return cudaGetLastError();
 }
 
@@ -1909,7 +2129,7 @@ cudaError_t conv3x3_tc_prepare() {
   if (e == cudaSuccess) e = tc::prepare_n<256>();
   for (cudaError_t f : {tc::prepare_wgrad<32, 16>(), tc::prepare_wgrad<32, 32>(), tc::prepare_wgrad<32, 64>(),
                         tc::prepare_wgrad<64, 16>(), tc::prepare_wgrad<64, 32>(), tc::prepare_wgrad<64, 64>(),
-                        tc::prepare_wgrad<32, 64, true>(), tc::prepare_wgrad<64, 64, true>(),
+                        tc::prepare_upwgrad<32, 64>(), tc::prepare_upwgrad<64, 64>(),
                         tc::prepare_rows<32, 32, 1, false>(), tc::prepare_rows<32, 64, 1, false>(),
                         tc::prepare_rows<64, 32, 1, false>(), tc::prepare_rows<64, 64, 1, false>(),
                         tc::prepare_rows<64, 64, 2, false>(), tc::prepare_rows<64, 64, 1, true>(),
