@@ -314,6 +314,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) tmem_alloc(saddr(slot), L::NCOLS);
+  pdl_enter();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -552,7 +553,6 @@ __global__ void __launch_bounds__(kRowThreads, RowCfg<N, KB, KC>::CPS)
   const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
   __shared__ float4 s_bias[N / 4];
   const int n0 = int(blockIdx.y) * N;
-  if (tid < N) reinterpret_cast<float *>(s_bias)[tid] = a.bias ? a.bias[n0 + tid] : 0.f;
   if (tid == 0) {
     for (uint32_t s = 0; s < 2 * S; ++s) mbar_init(bar0 + 8 * s, 1);
     mbar_init(wbar, 1);
@@ -564,6 +564,8 @@ __global__ void __launch_bounds__(kRowThreads, RowCfg<N, KB, KC>::CPS)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) tmem_alloc(saddr(slot), C::NCOLS);
+  pdl_enter();
+  if (tid < N) reinterpret_cast<float *>(s_bias)[tid] = a.bias ? a.bias[n0 + tid] : 0.f;
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -869,8 +871,6 @@ __global__ void __launch_bounds__(kRowThreads, 1)
                  tempty = tfull + 8 * RING;
   const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
   const int n0 = a.n_base + int(blockIdx.y) * N;
-  if (tid < N)
-    reinterpret_cast<float *>(s_bias)[tid] = a.bias ? a.bias[MODE == kUp ? (n0 + tid) % a.up_cout : n0 + tid] : 0.f;
   if (tid == 0) {
     for (int k = 0; k < kUpStages; ++k) {
       mbar_init(full + 8 * k, 1);
@@ -885,6 +885,9 @@ __global__ void __launch_bounds__(kRowThreads, 1)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) tmem_alloc(saddr(&s_slot), RING * N);
+  pdl_enter();
+  if (tid < N)
+    reinterpret_cast<float *>(s_bias)[tid] = a.bias ? a.bias[MODE == kUp ? (n0 + tid) % a.up_cout : n0 + tid] : 0.f;
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -1087,6 +1090,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   __shared__ float sbias[kInN];
   __shared__ int s_fail;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  pdl_enter();
   // B[n][k] = w[n][tap][c], k = 2 tap + c < 18, else 0
   for (int i = tid; i < kInN * kInK; i += kThreads) {
     const int n = i / kInK, k = i - (i / kInK) * kInK;
@@ -1280,6 +1284,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) tmem_alloc(saddr(slot), L::NCOLS);
+  pdl_enter();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -1497,6 +1502,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) tmem_alloc(saddr(slot), L::NCOLS);
+  pdl_enter();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -1708,8 +1714,7 @@ cudaError_t launch_nks(const ConvTC &c, cudaStream_t s, int nblk) {
   const cudaError_t e = prepare_nks<N, KB, STAGES, UP, HALO>();
   if (e != cudaSuccess) return e;
   const long long tiles = (long long)a.tiles_w * a.tiles_h * c.B;
-  k<<<dim3(unsigned(tiles), unsigned(nblk)), kThreads, Layout<N, KB, STAGES, HALO>::BYTES, s>>>(ta, tb, a);
-  return cudaGetLastError();
+  return launch(k, dim3(unsigned(tiles), unsigned(nblk)), kThreads, Layout<N, KB, STAGES, HALO>::BYTES, s, ta, tb, a);
 }
 
 // ---- the persistent row kernel (k_conv_rows)
@@ -1767,8 +1772,8 @@ cudaError_t launch_rows(const ConvTC &c, cudaStream_t s, int sms) {
   a.db = c.db;
   const int nblk = c.cout / N;
   const int ctas = std::max(1, std::min(EPI == kPool ? a.tiles / 2 : a.tiles, sms * R::CPS / nblk));
-  k_conv_rows<N, KB, KC, TAPS, EPI><<<dim3(unsigned(ctas), unsigned(nblk)), kRowThreads, R::BYTES, s>>>(ta, tb, a);
-  return cudaGetLastError();
+  return launch(k_conv_rows<N, KB, KC, TAPS, EPI>, dim3(unsigned(ctas), unsigned(nblk)), kRowThreads, R::BYTES, s, ta, tb,
+                a);
 }
 
 template <int N, int KB, bool UP>
@@ -1867,9 +1872,8 @@ cudaError_t launch_upb(const ConvTC &c, cudaStream_t s, int nblk) {
   a.wide = wide_stores(c);
   a.err = c.err;
   const long long tiles = (long long)a.tiles_w * a.tiles_h * c.B;
-  k_conv3x3_tc<N, KB, STAGES, false, false, true>
-      <<<dim3(unsigned(tiles), unsigned(nblk)), kThreads, L::BYTES, s>>>(ta, tb, a);
-  return cudaGetLastError();
+  return launch(k_conv3x3_tc<N, KB, STAGES, false, false, true>, dim3(unsigned(tiles), unsigned(nblk)), kThreads, L::BYTES,
+                s, ta, tb, a);
 }
 
 template <int N>
@@ -1946,8 +1950,7 @@ cudaError_t launch_wgrad(const WgradTC &g, cudaStream_t s, int sms) {
   const int yb = (g.cout / CO) * (g.cin / CI);
   const long long wave = wave_split<L>(1LL << 40, sms, 1);   // CTAs resident at once
   const long long splits = wave_split<L>(a.rows, wave % yb && yb < wave ? 2 * sms : sms, yb);
-  k_wgrad_rows<CO, CI><<<dim3(unsigned(splits), unsigned(yb)), kThreads, L::BYTES, s>>>(ta, tb, a);
-  return cudaGetLastError();
+  return launch(k_wgrad_rows<CO, CI>, dim3(unsigned(splits), unsigned(yb)), kThreads, L::BYTES, s, ta, tb, a);
 }
 
 template <int CO>
@@ -1991,8 +1994,8 @@ cudaError_t launch_upw(const UpWgradTC &g, cudaStream_t s, int sms) {
   const int yb = (g.cout / CO) * (g.cin / CI);
   const long long splits = wave_split<L>(a.nkb, sms, yb);
   a.per_cta = (a.nkb + splits - 1) / splits;
-  k_upwgrad_tc<CO, CI, kWStages><<<dim3(unsigned((a.nkb + a.per_cta - 1) / a.per_cta), unsigned(yb)), kThreads, L::BYTES, s>>>(ta, tb, a);
-  return cudaGetLastError();
+  return launch(k_upwgrad_tc<CO, CI, kWStages>, dim3(unsigned((a.nkb + a.per_cta - 1) / a.per_cta), unsigned(yb)), kThreads,
+                L::BYTES, s, ta, tb, a);
 }
 
 // The persistent transposed convolution (up_cout > 0: all 4 up_cout columns from
@@ -2023,9 +2026,8 @@ cudaError_t launch_up(const ConvTC &c, cudaStream_t s, int sms, const CUtensorMa
   const int wbytes = a.units * N * KB * 2, unit = kM * KB * 2;
   a.stages = std::min(kUpStages, (kUpSmem - 1024 - wbytes) / unit);
   const int nblk = c.cout / N, ctas = std::max(1, std::min(a.tiles, sms / nblk));
-  k_up_tiles<N, KB, MODE><<<dim3(unsigned(ctas), unsigned(nblk)), kRowThreads, 1024 + wbytes + a.stages * unit, s>>>(
-      ta, tb, a);
-  return cudaGetLastError();
+  return launch(k_up_tiles<N, KB, MODE>, dim3(unsigned(ctas), unsigned(nblk)), kRowThreads,
+                1024 + wbytes + a.stages * unit, s, ta, tb, a);
 }
 
 template <int KB, int MODE>
@@ -2217,9 +2219,8 @@ cudaError_t conv_in_tc(const float2 *x, const __nv_bfloat16 *w, int wcin, const 
   if (npix < 1 || npix >= (1LL << 31)) return cudaErrorInvalidValue;
   const long long ntiles = (npix + tc::kM - 1) / tc::kM;
   const long long grid = ntiles < 8LL * sms ? ntiles : 8LL * sms;   // 8 CTAs per SM, tiles in turn
-  tc::k_conv_in_tc<<<unsigned(grid), tc::kThreads, 0, s>>>(x, w, wcin, bias, out, B, H, W, relu,
-                                                           (reinterpret_cast<uintptr_t>(out) & 31) == 0, err);
-  return cudaGetLastError();
+  return launch(tc::k_conv_in_tc, dim3(unsigned(grid)), tc::kThreads, 0, s, x, w, wcin, bias, out, B, H, W, relu,
+                (reinterpret_cast<uintptr_t>(out) & 31) == 0 ? 1 : 0, err);
 }
 
 cudaError_t conv_up_tc(const ConvTC &c, cudaStream_t s) {

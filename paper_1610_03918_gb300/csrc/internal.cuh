@@ -258,7 +258,7 @@ struct BoxPoisson {
   size_t solve_smem = 0, add_smem = 0;
 };
 
-// Programmatic dependent launch.  The solver's kernels wait for the grid
+// Programmatic dependent launch.  The solver's and the network's kernels wait for the grid
 // before them (its results are then visible) and at once let the next kernel
 // of the stream be scheduled, so that kernel's blocks are resident and waiting
 // when this one ends instead of being launched only then.  Both instructions
@@ -294,9 +294,9 @@ void launch_cluster(void (*k)(P...), int ctas, int block, size_t smem, cudaStrea
 }
 
 template <typename... P, typename... A>
-void launch(void (*k)(P...), int grid, int block, size_t smem, cudaStream_t s, A... args) {
+cudaError_t launch(void (*k)(P...), dim3 grid, int block, size_t smem, cudaStream_t s, A... args) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(unsigned(grid));
+  cfg.gridDim = grid;
   cfg.blockDim = dim3(unsigned(block));
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
@@ -305,7 +305,7 @@ void launch(void (*k)(P...), int grid, int block, size_t smem, cudaStream_t s, A
   at.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &at;
   cfg.numAttrs = kPdl ? 1 : 0;
-  cudaLaunchKernelEx(&cfg, k, args...);
+  return cudaLaunchKernelEx(&cfg, k, args...);
 }
 
 }  // namespace picgb

@@ -291,6 +291,7 @@ template <bool POOL>
 __global__ void __launch_bounds__(256) k_relu_back(const bf16 *g, int g_cs, int g_off, const bf16 *y, int y_cs,
                                                    int y_off, const bf16 *gp, int H, int W, bf16 *dpre, int C,
                                                    long long npix, float *db) {
+  pdl_enter();
   const int G = C >> 3, grp = threadIdx.x % G, ppb = blockDim.x / G;
   float s[8];
 #pragma unroll
@@ -342,6 +343,7 @@ struct FlipArgs {
   int cout[kFlips], cin[kFlips];   // multiples of 32
 };
 __global__ void __launch_bounds__(256) k_wflip(FlipArgs a) {
+  pdl_enter();
   __shared__ bf16 tile[32][34];
   const int q = blockIdx.y, cout = a.cout[q], cin = a.cin[q], nci = cin / 32;
   const int tiles = 9 * (cout / 32) * nci, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -442,6 +444,7 @@ __global__ void __launch_bounds__(256) k_up_back_w(const bf16 *in, int cin, cons
 // MSE: dy = 2 (y - t) / n, loss partial sums in FP64, one atomic per CTA (one
 // per warp, on the one address, made 25 us of 2.1M pixels; now 16.5, the FP64 adds)
 __global__ void __launch_bounds__(256) k_mse(const float *y, const float *t, float *dy, long long n, double *loss) {
+  pdl_enter();
   __shared__ double part[8];
   double s = 0.0;
   GSTRIDE(p, n) {
@@ -467,6 +470,7 @@ __global__ void __launch_bounds__(256) k_mse(const float *y, const float *t, flo
 template <bool RELU>
 __global__ void __launch_bounds__(256) k_head_back(const float *dy, const bf16 *hin, const float *w, bf16 *gh,
                                                    float *dw, float *db, float *dbh, long long npix) {
+  pdl_enter();
   constexpr int G = kC0 / 8, PPB = 256 / G;
   const int grp = threadIdx.x % G;
   float wk[8], s[8], sh[8], bs = 0.f;
@@ -525,6 +529,7 @@ __global__ void __launch_bounds__(256) k_head_back(const float *dy, const bf16 *
 // g_off multiples of 8, C at most 256
 __global__ void __launch_bounds__(256) k_colsum(const bf16 *g, int g_cs, int g_off, int C, long long npix,
                                                 float *db) {
+  pdl_enter();
   const int G = C >> 3, grp = threadIdx.x % G, ppb = blockDim.x / G;
   float s[8];
 #pragma unroll
@@ -572,6 +577,7 @@ __global__ void k_w_to_bf16(const float *m, bf16 *w, int cout, int ci_m, int ci_
 
 // gradient of an expanded conv weight folded back to the master layout
 __global__ void k_w_fold(const float *gc, float *gm, int cout, int ci_m, int ci_c) {
+  pdl_enter();
   GSTRIDE(i, (long long)cout * 9 * ci_m) {
     const int ci = int(i % ci_m);
     const long long ct = i / ci_m;
@@ -610,6 +616,7 @@ __global__ void k_to_bf16(const float *a, bf16 *b, long long n) {
 }
 
 __global__ void k_input_vec(const float2 *x, uint4 *out, long long npix) {
+  pdl_enter();
   GSTRIDE(p, npix) {
     const float2 v = x[p];
     __align__(16) bf16 o[8] = {__float2bfloat16(v.x), __float2bfloat16(v.y)};
@@ -680,6 +687,7 @@ __global__ void __launch_bounds__(256) k_conv_in(const float2 *x, const bf16 *w,
 
 // 2x2 average pool, 8 channels (16 bytes) per thread
 __global__ void k_pool_vec(const bf16 *in, int in_cs, int in_off, bf16 *out, int C, int B, int H, int W) {
+  pdl_enter();
   const int Ho = H / 2, Wo = W / 2, C8 = C / 8;
   GSTRIDE(i, (long long)B * Ho * Wo * C8) {
     const int c = int(i % C8) * 8;
@@ -701,6 +709,7 @@ __global__ void k_pool_vec(const bf16 *in, int in_cs, int in_off, bf16 *out, int
 
 // head with 16-byte loads of the 32 input channels
 __global__ void k_head_vec(const bf16 *hin, const float *w, const float *b, float *y, long long npix) {
+  pdl_enter();
   GSTRIDE(p, npix) {
     const uint4 *src = reinterpret_cast<const uint4 *>(hin + p * kC0);
     float s = b[0];
@@ -804,8 +813,8 @@ void conv_fwd(pic_unet *u, int ci, const bf16 *in, int in_cs, int in_off, bf16 *
     e.pool = pool;
     if (conv_tc(u, in, in_cs, in_off, c.cin_c, c.w, u->P + c.b_off, out, out_cs, out_off, c.cout, l, relu, e)) return;
     conv_fwd(u, ci, in, in_cs, in_off, out, out_cs, out_off, l, relu);
-    k_pool_vec<<<gridn((long long)pix(u, l + 1) * c.cout / 8), 256, 0, u->stream>>>(out, out_cs, out_off, pool, c.cout,
-                                                                                   u->B, u->H >> l, u->W >> l);
+    launch(k_pool_vec, gridn((long long)pix(u, l + 1) * c.cout / 8), 256, 0, u->stream, out, out_cs, out_off, pool,
+           c.cout, u->B, u->H >> l, u->W >> l);
     return;
   }
   if (conv_tc(u, in, in_cs, in_off, c.cin_c, c.w, u->P + c.b_off, out, out_cs, out_off, c.cout, l, relu))
@@ -849,7 +858,7 @@ void flip_weights(pic_unet *u) {
     a.cin[n] = c.cin_c;
     n += 1;
   }
-  k_wflip<<<dim3(unsigned(2 * u->num_sms), unsigned(n)), 256, 0, u->stream>>>(a);
+  launch(k_wflip, dim3(unsigned(2 * u->num_sms), unsigned(n)), 256, 0, u->stream, a);
 }
 
 // data gradient: gin (cin channels) = conv(dpre, flipped weights).  before: the layer that made the input, through whose ReLU the gradient then
@@ -935,8 +944,8 @@ void conv_back_weights(pic_unet *u, int ci, const bf16 *dpre, const bf16 *in, in
   }
   if (!done) wgrad_mma(u->B, H, W, c.cin_c, c.cout, dpre, in, in_cs, in_off, dw, u->stream);
   if (c.cin_c != c.cin_m)
-    k_w_fold<<<gridn((long long)c.cout * 9 * c.cin_m), 256, 0, u->stream>>>(u->g0tmp, u->G + c.w_off,
-                                                                          c.cout, c.cin_m, c.cin_c);
+    launch(k_w_fold, gridn((long long)c.cout * 9 * c.cin_m), 256, 0, u->stream, u->g0tmp, u->G + c.w_off, c.cout,
+           c.cin_m, c.cin_c);
 }
 
 // backward through the ReLU that follows layer ci: dpre[l] from the gradient g at
@@ -949,11 +958,11 @@ void relu_back(pic_unet *u, int ci, const bf16 *g, int g_cs, int g_off, const bf
   const long long ppb = 256 / (c.cout / 8);
   const int grid = int(std::min<long long>((np + ppb - 1) / ppb, 8LL * u->num_sms));
   if (gp)
-    k_relu_back<true><<<grid, 256, 0, u->stream>>>(g, g_cs, g_off, y, y_cs, y_off, gp, u->H >> l, u->W >> l,
-                                                   u->dpre[l], c.cout, np, u->G + c.b_off);
+    launch(k_relu_back<true>, grid, 256, 0, u->stream, g, g_cs, g_off, y, y_cs, y_off, gp, u->H >> l, u->W >> l,
+           u->dpre[l], c.cout, np, u->G + c.b_off);
   else
-    k_relu_back<false><<<grid, 256, 0, u->stream>>>(g, g_cs, g_off, y, y_cs, y_off, nullptr, 1, 1, u->dpre[l],
-                                                    c.cout, np, u->G + c.b_off);
+    launch(k_relu_back<false>, grid, 256, 0, u->stream, g, g_cs, g_off, y, y_cs, y_off, nullptr, 1, 1, u->dpre[l],
+           c.cout, np, u->G + c.b_off);
 }
 
 // The two layers of a block (cb after ca, y between them), from dpre, the gradient
@@ -1036,8 +1045,8 @@ bool up_wgrad_tc(pic_unet *u, int l, const bf16 *hin) {
   if (conv_upwgrad_tc(g, u->stream) != cudaSuccess) return false;
   const long long np = pix(u, l);
   const long long ppb = 256 / (up.cout / 8);
-  k_colsum<<<int(std::min<long long>((np + ppb - 1) / ppb, 8LL * u->num_sms)), 256, 0, u->stream>>>(
-      u->gcat[l], 2 * kC[l], 0, up.cout, np, u->G + up.b_off);
+  launch(k_colsum, int(std::min<long long>((np + ppb - 1) / ppb, 8LL * u->num_sms)), 256, 0, u->stream, u->gcat[l],
+         2 * kC[l], 0, up.cout, np, u->G + up.b_off);
   return true;
 }
 
@@ -1066,12 +1075,13 @@ bool up_tc(pic_unet *u, int l, const bf16 *in, int in_cs) {
 }
 
 // keep_input: also the BF16 copy of the input padded to kCin0 channels, which
-// the weight gradient of the first convolution reads
-void forward(pic_unet *u, const float *x, bool keep_input) {
+// the weight gradient of the first convolution reads.  y: where the output goes
+// (null: u->y)
+void forward(pic_unet *u, const float *x, bool keep_input, float *y = nullptr) {
   const int C0 = kC[0], C1 = kC[1], C2 = kC[2], C3 = kC[3];
   if (keep_input)
-    k_input_vec<<<gridn(pix(u, 0)), 256, 0, u->stream>>>(reinterpret_cast<const float2 *>(x),
-                                                         reinterpret_cast<uint4 *>(u->x16), pix(u, 0));
+    launch(k_input_vec, gridn(pix(u, 0)), 256, 0, u->stream, reinterpret_cast<const float2 *>(x),
+           reinterpret_cast<uint4 *>(u->x16), pix(u, 0));
   // encoder; each level's output is written into the skip half of its concat buffer
   {
     // the first convolution on the tensor cores (K = 9 taps x 2 channels
@@ -1108,7 +1118,8 @@ void forward(pic_unet *u, const float *x, bool keep_input) {
     h = u->dout[l];
     hc = kC[l];
   }
-  k_head_vec<<<gridn(pix(u, 0)), 256, 0, u->stream>>>(u->dout[0], u->P + u->head_w, u->P + u->head_b, u->y, pix(u, 0));
+  launch(k_head_vec, gridn(pix(u, 0)), 256, 0, u->stream, u->dout[0], u->P + u->head_w, u->P + u->head_b, y ? y : u->y,
+         pix(u, 0));
 }
 
 void backward(pic_unet *u) {
@@ -1116,9 +1127,9 @@ void backward(pic_unet *u) {
   cudaMemsetAsync(u->G, 0, size_t(u->nparam) * 4, u->stream);
   flip_weights(u);
   // the head, and through the ReLU of the layer before it
-  k_head_back<true><<<int(std::min<long long>((pix(u, 0) + 63) / 64, 8LL * u->num_sms)), 256, 0, u->stream>>>(
-      u->dy, u->dout[0], u->P + u->head_w, u->dpre[0], u->G + u->head_w, u->G + u->head_b,
-      u->G + u->conv[D0B].b_off, pix(u, 0));
+  launch(k_head_back<true>, int(std::min<long long>((pix(u, 0) + 63) / 64, 8LL * u->num_sms)), 256, 0, u->stream,
+         u->dy, u->dout[0], u->P + u->head_w, u->dpre[0], u->G + u->head_w, u->G + u->head_b,
+         u->G + u->conv[D0B].b_off, pix(u, 0));
   // decoder, from the output up; dpre: the gradient before the ReLU of the level's last layer
   const bf16 *dpre = u->dpre[0];
   for (int l = 0; l <= 2; ++l) {
@@ -1170,6 +1181,7 @@ void backward(pic_unet *u) {
 }  // namespace picgb
 
 using namespace picgb::unet;
+using picgb::launch;
 
 extern "C" {
 
@@ -1312,9 +1324,7 @@ pic_status pic_unet_get_params(pic_unet *u, float *host) {
 
 pic_status pic_unet_forward(pic_unet *u, const float *x, float *y) {
   if (!u || !x || !y) return PIC_EINVAL;
-  forward(u, x, false);
-  if (cudaMemcpyAsync(y, u->y, size_t(u->B) * u->H * u->W * 4, cudaMemcpyDeviceToDevice, u->stream) != cudaSuccess)
-    return PIC_ECUDA;
+  forward(u, x, false, y);
   return cudaGetLastError() == cudaSuccess ? PIC_OK : PIC_ECUDA;
 }
 
@@ -1323,7 +1333,7 @@ pic_status pic_unet_gradients(pic_unet *u, const float *x, const float *t, float
   forward(u, x, true);
   cudaMemsetAsync(u->d_loss, 0, 8, u->stream);
   const long long n = (long long)u->B * u->H * u->W;
-  k_mse<<<std::min(1024, gridn(n)), 256, 0, u->stream>>>(u->y, t, u->dy, n, u->d_loss);
+  launch(k_mse, std::min(1024, gridn(n)), 256, 0, u->stream, u->y, t, u->dy, n, u->d_loss);
   backward(u);
   if (host_grad &&
       cudaMemcpyAsync(host_grad, u->G, size_t(u->nparam) * 4, cudaMemcpyDeviceToHost, u->stream) != cudaSuccess)
@@ -1342,7 +1352,7 @@ pic_status pic_unet_train_step(pic_unet *u, const float *x, const float *t, floa
   forward(u, x, true);
   cudaMemsetAsync(u->d_loss, 0, 8, u->stream);
   const long long n = (long long)u->B * u->H * u->W;
-  k_mse<<<std::min(1024, gridn(n)), 256, 0, u->stream>>>(u->y, t, u->dy, n, u->d_loss);
+  launch(k_mse, std::min(1024, gridn(n)), 256, 0, u->stream, u->y, t, u->dy, n, u->d_loss);
   backward(u);
   u->step += 1;
   const float b1 = 0.9f, b2 = 0.999f;
@@ -1565,8 +1575,8 @@ pic_status pic_avgpool2_bf16(int32_t B, int32_t H, int32_t W, const void *in, in
       (long long)B * H * W >= (1LL << 31))
     return PIC_EINVAL;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  k_pool_vec<<<gridn((long long)B * (H / 2) * (W / 2) * (C / 8)), 256, 0, s>>>(
-      static_cast<const bf16 *>(in), in_cs, in_off, static_cast<bf16 *>(out), C, B, H, W);
+  launch(k_pool_vec, gridn((long long)B * (H / 2) * (W / 2) * (C / 8)), 256, 0, s, static_cast<const bf16 *>(in),
+         in_cs, in_off, static_cast<bf16 *>(out), C, B, H, W);
   if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) return PIC_ECUDA;
   return PIC_OK;
 }
@@ -1574,7 +1584,7 @@ pic_status pic_avgpool2_bf16(int32_t B, int32_t H, int32_t W, const void *in, in
 pic_status pic_head_bf16(int64_t npix, const void *hin, const float *w, const float *b, float *y, void *stream) {
   if (!hin || !w || !b || !y || npix < 1 || !aligned16(hin)) return PIC_EINVAL;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  k_head_vec<<<gridn(npix), 256, 0, s>>>(static_cast<const bf16 *>(hin), w, b, y, npix);
+  launch(k_head_vec, gridn(npix), 256, 0, s, static_cast<const bf16 *>(hin), w, b, y, npix);
   if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) return PIC_ECUDA;
   return PIC_OK;
 }
@@ -1585,8 +1595,8 @@ pic_status pic_head_back_bf16(int64_t npix, const float *dy, const void *hin, co
   const int sms = device_sms();
   if (sms < 1) return PIC_ECUDA;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  k_head_back<false><<<int(std::min<long long>((npix + 63) / 64, 8LL * sms)), 256, 0, s>>>(
-      dy, static_cast<const bf16 *>(hin), w, static_cast<bf16 *>(gh), dw, db, nullptr, npix);
+  launch(k_head_back<false>, int(std::min<long long>((npix + 63) / 64, 8LL * sms)), 256, 0, s, dy,
+         static_cast<const bf16 *>(hin), w, static_cast<bf16 *>(gh), dw, db, nullptr, npix);
   if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) return PIC_ECUDA;
   return PIC_OK;
 }
@@ -1606,11 +1616,11 @@ pic_status pic_relu_back_bf16(int32_t B, int32_t H, int32_t W, const void *g, in
   const int grid = int(std::min<long long>((np + ppb - 1) / ppb, 8LL * sms));
   const bf16 *bg = static_cast<const bf16 *>(g), *by = static_cast<const bf16 *>(y);
   if (gp)
-    k_relu_back<true><<<grid, 256, 0, s>>>(bg, g_cs, g_off, by, y_cs, y_off, static_cast<const bf16 *>(gp), H, W,
-                                           static_cast<bf16 *>(dpre), C, np, db);
+    launch(k_relu_back<true>, grid, 256, 0, s, bg, g_cs, g_off, by, y_cs, y_off, static_cast<const bf16 *>(gp), H, W,
+           static_cast<bf16 *>(dpre), C, np, db);
   else
-    k_relu_back<false><<<grid, 256, 0, s>>>(bg, g_cs, g_off, by, y_cs, y_off, nullptr, 1, 1,
-                                            static_cast<bf16 *>(dpre), C, np, db);
+    launch(k_relu_back<false>, grid, 256, 0, s, bg, g_cs, g_off, by, y_cs, y_off, nullptr, 1, 1,
+           static_cast<bf16 *>(dpre), C, np, db);
   if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) return PIC_ECUDA;
   return PIC_OK;
 }
@@ -1704,8 +1714,8 @@ pic_status pic_upconv_wgrad_bf16(int32_t impl, int32_t B, int32_t H, int32_t W, 
   g.err = err;
   if (picgb::conv_upwgrad_tc(g, s) != cudaSuccess) return PIC_ECUDA;
   const long long np = 4LL * B * H * W, ppb = 256 / (cout / 8);
-  k_colsum<<<int(std::min<long long>((np + ppb - 1) / ppb, 8LL * sms)), 256, 0, s>>>(bg, gout_cs, gout_off, cout,
-                                                                                   np, db);
+  launch(k_colsum, int(std::min<long long>((np + ppb - 1) / ppb, 8LL * sms)), 256, 0, s, bg, gout_cs, gout_off, cout,
+         np, db);
   if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) return PIC_ECUDA;
   return word.read("weight gradient");
 }
