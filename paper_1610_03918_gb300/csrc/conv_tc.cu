@@ -471,6 +471,7 @@ struct RowArgs {
   const bf16 *y;           // kBack: [B][H][W][y_cs], channels from y_off
   int y_cs, y_off;
   float *db;
+  int db_n;                // kSum: the first db_n output channels are summed
 };
 
 // kPool: also the 2 x 2 average pool of the output (H and W even).  kBack: the
@@ -479,7 +480,9 @@ struct RowArgs {
 // output (k_pool_vec, k_relu_back), which is as long as the convolution: batch 4,
 // 32 -> 32 at 1032 x 512 46.8 + 42.5 us -> 55.5 and 45.5 + 64.4 -> 62; 64 -> 64 at
 // 516 x 256 32.8 + 13.3 -> 36 and 32.7 + 32.5 -> 48.
-enum Epilogue { kPlain, kPool, kBack };
+// kSum: only the sums, of the output's first channels (the bias gradient of the
+// transposed convolution whose output they are; k_colsum took 70 us a pass for it).
+enum Epilogue { kPlain, kPool, kBack, kSum };
 
 constexpr int kRowThreads = 320;
 constexpr int kRing = 8;                     // accumulators (output rows) in TMEM
@@ -698,11 +701,13 @@ __global__ void __launch_bounds__(kRowThreads, RowCfg<N, KB, KC>::CPS)
     uint32_t i = 0;
     bool ok = true;
     Runs<EPI == kPool> r(a);
-    float sum[EPI == kBack ? N : 1];         // kBack: the thread's columns' sums
+    constexpr bool SUMS = EPI == kBack || EPI == kSum;
+    const bool sums = EPI == kBack || (EPI == kSum && n0 < a.db_n);
+    float sum[SUMS ? N : 1];                 // the thread's columns' sums
     uint32_t above[EPI == kPool ? N / 2 : 1];   // kPool: the output above
-    if (EPI == kBack)
+    if (SUMS)
 #pragma unroll
-      for (int k = 0; k < N; ++k) sum[EPI == kBack ? k : 0] = 0.f;
+      for (int k = 0; k < N; ++k) sum[SUMS ? k : 0] = 0.f;
     while (ok && r.next()) {
       const int w = r.cb * kM + 32 * quad + lane;
       const size_t p0 = (size_t(r.b) * a.H + r.h0) * a.W + w;
@@ -749,8 +754,13 @@ __global__ void __launch_bounds__(kRowThreads, RowCfg<N, KB, KC>::CPS)
 #pragma unroll
               for (int k = 0; k < 8; ++k) {
                 o[k] &= __hgt2_mask(*reinterpret_cast<const __nv_bfloat162 *>(yy + k), __floats2bfloat162_rn(0.f, 0.f));
-                sum[EPI == kBack ? c + q + 2 * k : 0] += __uint_as_float(o[k] << 16);
-                sum[EPI == kBack ? c + q + 2 * k + 1 : 0] += __uint_as_float(o[k] & 0xffff0000u);
+              }
+            }
+            if (sums && (EPI == kBack || w < a.W)) {   // (the mask is 0 off the image)
+#pragma unroll
+              for (int k = 0; k < 8; ++k) {
+                sum[SUMS ? c + q + 2 * k : 0] += __uint_as_float(o[k] << 16);
+                sum[SUMS ? c + q + 2 * k + 1 : 0] += __uint_as_float(o[k] & 0xffff0000u);
               }
             }
             if (w < a.W) store16(dst + c + q, o, wide);
@@ -788,18 +798,18 @@ __global__ void __launch_bounds__(kRowThreads, RowCfg<N, KB, KC>::CPS)
         }
       }
     }
-    if (EPI == kBack) {
+    if (sums) {
 #pragma unroll
       for (int c = 0; c < N; c += 32) {
         float mine = 0.f;
 #pragma unroll
         for (int k = 0; k < 32; ++k) {
-          float x = sum[EPI == kBack ? c + k : 0];
+          float x = sum[SUMS ? c + k : 0];
 #pragma unroll
           for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
           if (lane == k) mine = x;
         }
-        atomicAdd(&a.db[n0 + c + lane], mine);
+        if (EPI == kBack || n0 + c + lane < a.db_n) atomicAdd(&a.db[n0 + c + lane], mine);
       }
     }
     if (!ok && lane == 0) {
@@ -1770,6 +1780,7 @@ cudaError_t launch_rows(const ConvTC &c, cudaStream_t s, int sms) {
   a.y_cs = c.y_cs;
   a.y_off = c.y_off;
   a.db = c.db;
+  a.db_n = c.db_n;
   const int nblk = c.cout / N;
   const int ctas = std::max(1, std::min(EPI == kPool ? a.tiles / 2 : a.tiles, sms * R::CPS / nblk));
   return launch(k_conv_rows<N, KB, KC, TAPS, EPI>, dim3(unsigned(ctas), unsigned(nblk)), kRowThreads, R::BYTES, s, ta, tb,
@@ -2139,6 +2150,9 @@ cudaError_t conv3x3_tc_prepare() {
                         tc::prepare_rows<32, 64, 4, true>(),
                         tc::prepare_rows<32, 32, 1, false, tc::kPool>(), tc::prepare_rows<64, 64, 1, false, tc::kPool>(),
                         tc::prepare_rows<64, 64, 2, false, tc::kPool>(), tc::prepare_rows<64, 64, 2, true, tc::kPool>(),
+                        tc::prepare_rows<64, 32, 1, false, tc::kSum>(), tc::prepare_rows<64, 64, 1, false, tc::kSum>(),
+                        tc::prepare_rows<64, 64, 2, false, tc::kSum>(), tc::prepare_rows<64, 64, 1, true, tc::kSum>(),
+                        tc::prepare_rows<64, 64, 2, true, tc::kSum>(),
                         tc::prepare_rows<32, 32, 1, false, tc::kBack>(), tc::prepare_rows<64, 64, 1, false, tc::kBack>(),
                         tc::prepare_rows<64, 64, 2, false, tc::kBack>(), tc::prepare_rows<64, 64, 2, true, tc::kBack>()})
     if (e == cudaSuccess) e = f;
@@ -2190,6 +2204,15 @@ cudaError_t conv3x3_tc(const ConvTC &c, cudaStream_t s) {
     if (n == 128 && c.cin == 128)
       return c.pool ? tc::launch_rows<64, 64, 2, true, tc::kPool>(c, s, sms)
                     : tc::launch_rows<64, 64, 2, true, tc::kBack>(c, s, sms);
+    return cudaErrorNotSupported;
+  }
+  if (c.db) {   // the concatenations' gradients: twice as many channels out as in
+    if (!rows || c.cout != 2 * c.cin || c.db_n != c.cin) return cudaErrorNotSupported;
+    if (n == 64 && c.cin == 32) return tc::launch_rows<64, 32, 1, false, tc::kSum>(c, s, sms);
+    if (n == 64 && c.cin == 64) return tc::launch_rows<64, 64, 1, false, tc::kSum>(c, s, sms);
+    if (n == 64 && c.cin == 128) return tc::launch_rows<64, 64, 2, false, tc::kSum>(c, s, sms);
+    if (n >= 128 && c.cin == 64) return tc::launch_rows<64, 64, 1, true, tc::kSum>(c, s, sms);
+    if (n >= 128 && c.cin == 128) return tc::launch_rows<64, 64, 2, true, tc::kSum>(c, s, sms);
     return cudaErrorNotSupported;
   }
   if (rows) {

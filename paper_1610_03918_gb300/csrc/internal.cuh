@@ -530,6 +530,9 @@ struct ConvTC {
   const __nv_bfloat16 *y = nullptr;
   int y_cs = 0, y_off = 0;
   float *db = nullptr;
+  // db without y: the sums of the first db_n = cin output channels are added to db
+  // (cout = 2 cin up to 256)
+  int db_n = 0;
 };
 bool conv3x3_tc_supported(int cin, int cout, int in_cs, int in_off, int out_cs, int out_off, int W);
 cudaError_t conv3x3_tc(const ConvTC &c, cudaStream_t s);

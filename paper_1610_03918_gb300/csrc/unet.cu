@@ -861,16 +861,23 @@ void flip_weights(pic_unet *u) {
   launch(k_wflip, dim3(unsigned(2 * u->num_sms), unsigned(n)), 256, 0, u->stream, a);
 }
 
-// data gradient: gin (cin channels) = conv(dpre, flipped weights).  before: the layer that made the input, through whose ReLU the gradient then
-// goes (y contiguous; its bias gradient too) where the kernel can: true if it did
+// data gradient: gin (cin channels) = conv(dpre, flipped weights).  before: the layer
+// that made the input, through whose ReLU the gradient then goes (y contiguous; its
+// bias gradient too); lead: where the sums of gin's first half of channels are added;
+// either only where the kernel can: true if it did
 bool conv_back_data(pic_unet *u, int ci, const bf16 *dpre, bf16 *gin, int gin_cs, int gin_off, int l,
-                    int before = -1, const bf16 *y = nullptr) {
+                    int before = -1, const bf16 *y = nullptr, float *lead = nullptr) {
   const pic_unet::Conv &c = u->conv[ci];
-  if (before >= 0) {
+  if (before >= 0 || lead) {
     ConvTC e;
-    e.y = y;
-    e.y_cs = c.cin_c;
-    e.db = u->G + u->conv[before].b_off;
+    if (lead) {
+      e.db = lead;
+      e.db_n = c.cout;
+    } else {
+      e.y = y;
+      e.y_cs = c.cin_c;
+      e.db = u->G + u->conv[before].b_off;
+    }
     if (conv_tc(u, dpre, c.cout, 0, c.cout, c.wt, nullptr, gin, gin_cs, gin_off, c.cin_c, l, false, e)) return true;
   }
   if (conv_tc(u, dpre, c.cout, 0, c.cout, c.wt, nullptr, gin, gin_cs, gin_off, c.cin_c, l, false)) return false;
@@ -967,9 +974,10 @@ void relu_back(pic_unet *u, int ci, const bf16 *g, int g_cs, int g_off, const bf
 
 // The two layers of a block (cb after ca, y between them), from dpre, the gradient
 // before cb's ReLU: their weight gradients, ca's bias gradient, and the gradient gin
-// at ca's input (unless null).  gy: room for the gradient at y.
-void block_back(pic_unet *u, int ca, int cb, const bf16 *dpre, const bf16 *y, bf16 *gy, const bf16 *in, int in_cs,
-                int in_off, bf16 *gin, int gin_cs, int l) {
+// at ca's input (unless null).  gy: room for the gradient at y.  lead: where the sums
+// of gin's first half of channels are added if the kernel can: true if it did.
+bool block_back(pic_unet *u, int ca, int cb, const bf16 *dpre, const bf16 *y, bf16 *gy, const bf16 *in, int in_cs,
+                int in_off, bf16 *gin, int gin_cs, int l, float *lead = nullptr) {
   const int C = u->conv[ca].cout;
   conv_back_weights(u, cb, dpre, y, C, 0, l);
   const bf16 *d = gy;
@@ -978,7 +986,7 @@ void block_back(pic_unet *u, int ca, int cb, const bf16 *dpre, const bf16 *y, bf
     d = u->dpre[l];
   }
   conv_back_weights(u, ca, d, in, in_cs, in_off, l);
-  if (gin) conv_back_data(u, ca, d, gin, gin_cs, 0, l);
+  return gin && conv_back_data(u, ca, d, gin, gin_cs, 0, l, -1, nullptr, lead);
 }
 
 void weights_to_bf16(pic_unet *u) {
@@ -1025,9 +1033,9 @@ bool up_back_tc(pic_unet *u, int l, bf16 *gin, int before = -1, const bf16 *y = 
 }
 
 // weight and bias gradients of the transposed convolution of level l (input
-// hin) on the tensor cores and a vector column sum; false where the kernel does
-// not apply
-bool up_wgrad_tc(pic_unet *u, int l, const bf16 *hin) {
+// hin) on the tensor cores and, unless the bias gradient is there already, a vector
+// column sum; false where the kernel does not apply
+bool up_wgrad_tc(pic_unet *u, int l, const bf16 *hin, bool bias_done) {
   if (u->conv_impl != 0) return false;
   const pic_unet::Up &up = u->up[l];
   UpWgradTC g;
@@ -1043,6 +1051,7 @@ bool up_wgrad_tc(pic_unet *u, int l, const bf16 *hin) {
   g.W = u->W >> (l + 1);
   g.err = u->d_err;
   if (conv_upwgrad_tc(g, u->stream) != cudaSuccess) return false;
+  if (bias_done) return true;
   const long long np = pix(u, l);
   const long long ppb = 256 / (up.cout / 8);
   launch(k_colsum, int(std::min<long long>((np + ppb - 1) / ppb, 8LL * u->num_sms)), 256, 0, u->stream, u->gcat[l],
@@ -1135,9 +1144,10 @@ void backward(pic_unet *u) {
   for (int l = 0; l <= 2; ++l) {
     const int C = kC[l];
     const int ca = (l == 2) ? D2A : (l == 1) ? D1A : D0A;
-    block_back(u, ca, ca + 1, dpre, u->da[l], u->gda[l], u->cat[l], 2 * C, 0, u->gcat[l], 2 * C, l);
-    // transposed conv: gradient at its input (the output of level l+1) from gcat[:, 0:C]
     const pic_unet::Up &up = u->up[l];
+    const bool bias_done = block_back(u, ca, ca + 1, dpre, u->da[l], u->gda[l], u->cat[l], 2 * C, 0, u->gcat[l],
+                                      2 * C, l, u->conv_impl == 0 ? u->G + up.b_off : nullptr);
+    // transposed conv: gradient at its input (the output of level l+1) from gcat[:, 0:C]
     const int hl = u->H >> (l + 1), wl = u->W >> (l + 1);
     const bf16 *hin = (l == 2) ? u->b3 : u->dout[l + 1];
     bf16 *gin = (l == 2) ? u->gb3 : u->gdout[l + 1];
@@ -1151,7 +1161,8 @@ void backward(pic_unet *u) {
       relu_back(u, last, gin, up.cin, 0, hin, up.cin, 0, l + 1);
       dpre = u->dpre[l + 1];
     }
-    if (!up_wgrad_tc(u, l, hin)) {
+    if (!up_wgrad_tc(u, l, hin, bias_done)) {   // the fallback sums the bias gradient itself
+      if (bias_done) cudaMemsetAsync(u->G + up.b_off, 0, size_t(up.cout) * 4, u->stream);
       const int rows = u->B * hl;
       const int tiles = ((up.cin + 31) / 32) * ((up.cout + 31) / 32) * 4;
       int groups = std::max(1, std::min(rows, 2048 / tiles));
