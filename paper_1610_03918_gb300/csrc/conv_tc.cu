@@ -7,6 +7,11 @@
 // with BF16 tensors in NHWC (channel slices given by a channel stride and
 // offset), FP32 accumulation, act = ReLU or identity, zero padding.
 //
+// Images at least 128 pixels wide whose channels fit run on the row kernel
+// (k_conv_rows), the transposed convolutions and their data gradients on
+// k_up_tiles, both persistent; the weight gradients on k_wgrad_rows and
+// k_upwgrad_tc, with both operands MN-major; the rest on the tile kernel:
+//
 // One CTA computes a tile of M = 128 output pixels (a BH x BW block of one
 // image, BW = min(W, 128) rounded down to a power of two) for a block of N
 // output channels: all of them, or, for layers with fewer pixel tiles than
@@ -24,8 +29,7 @@
 // its TMEM) instead of hanging.
 //
 // The same kernel, in further modes, computes the 2x2 stride-2 transposed
-// convolution and its data gradient; k_wgrad_rows below computes the weight
-// gradients of both kinds of convolution with both operands MN-major.
+// convolution and its data gradient where the channels are no multiples of 32.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>

@@ -8,14 +8,20 @@
 // copy is made.  The input has 2 channels (rho / s, conductor mask) padded to
 // 16 so that every convolution's K is a multiple of 16.
 //
-// 3x3 convolutions (forward and data gradient) are implicit GEMMs on the
-// tensor cores (mma.sync m16n8k16 BF16 -> FP32, ldmatrix fragments, cp.async
-// double-buffered tiles): M = pixels of one row segment, N = output
-// channels, K = 9 taps x input channels.  The data gradient is the same
-// kernel with the weights flipped in space and transposed in channels.  The
-// weight gradient is a tensor-core GEMM over pixels (M = out channels,
-// N = in channels per tap) accumulated with FP32 atomics.  The transposed
-// convolutions, pooling, head, loss and Adam are small CUDA-core kernels.
+// Every contraction runs on the tcgen05 kernels of conv_tc.cu, which also pool
+// the encoder's outputs, take the gradients through the ReLUs and sum the bias
+// gradients in their epilogues where the shapes allow it; the head, the loss, Adam
+// and what the epilogues do not take are CUDA-core kernels here.  The kernels of a
+// pass are launched programmatically (pdl_enter).
+//
+// With conv_impl = 1, or where a shape does not fit, the 3x3 convolutions
+// (forward and data gradient) are implicit GEMMs with mma.sync (m16n8k16 BF16 ->
+// FP32, ldmatrix fragments, cp.async double-buffered tiles): M = pixels of one row
+// segment, N = output channels, K = 9 taps x input channels.  The data gradient is
+// the same kernel with the weights flipped in space and transposed in channels.
+// The weight gradient is a GEMM over pixels (M = out channels, N = in channels per
+// tap) accumulated with FP32 atomics; the transposed convolutions run on the CUDA
+// cores.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
