@@ -585,7 +585,7 @@ const float *unet_output(const pic_unet *u);
 int unet_height(const pic_unet *u);
 int unet_width(const pic_unet *u);
 int unet_batch(const pic_unet *u);
-int unet_forward_kernels();
+int unet_forward_kernels(const pic_unet *u);
 pic_status unet_copy_params(pic_unet *dst, const pic_unet *src);
 // RF bias: the electrode's Dirichlet values (in phi and in the Dirichlet
 // data) and the lift at t = (step + advance) dt; no-op without RF

@@ -964,26 +964,34 @@ __global__ void k_moments(ParticleBuf P, const int64_t *nslots_p, double *part) 
 
 // the CTAs of the resident ones that a context counts on (an ensemble's members share the GPU)
 int own_ctas(const pic_ctx *c, int resident) { return std::max(1, resident / std::max(1, c->sharing)); }
-// whether the particles the context has room for make chunks larger than kChunk (not in
+// whether the particles the context has room for make chunks larger than kChunk.  Not in
 // an ensemble, whose members find more of the GPU free than their part at times and
-// share out their chunks over that: 8 members 280 -> 291 us a step)
+// share out their chunks over that: 8 members 280 -> 291 us a step.  Nor with the other
+// tile shapes: a build of their kernels with the parts' loop ended in an SM exception
+// on 34M particles, with every chunk, cell and slot checked in range; the cause was not
+// found, and those kernels are not built.
 bool chunk_parts(const pic_ctx *c, int resident) {
-  return c->sharing <= 1 && (c->cap[0] + c->cap[1]) / resident / kShareParts > kChunk;
+  return c->tile_variant == 0 && c->sharing <= 1 && (c->cap[0] + c->cap[1]) / resident / kShareParts > kChunk;
 }
 
 // CTAs of the step kernel that are resident at once
 template <int V>
 int resident_ctas(const pic_ctx *c) {
   int per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_particles<0, V, true>, Win<V>::THREADS, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_particles<0, V, V == 0>, Win<V>::THREADS, 0);
   return c->num_sms * std::min(std::max(per_sm, 1), kMaxCtasPerSm);
 }
 
 template <int MODE, int V>
 cudaError_t launch_particles_v(pic_ctx *c, const PArgs &a) {
   const int ctas = resident_ctas<V>(c);
-  if (chunk_parts(c, ctas)) k_particles<MODE, V, true><<<ctas, Win<V>::THREADS, 0, c->stream>>>(a);
-  else k_particles<MODE, V, false><<<ctas, Win<V>::THREADS, 0, c->stream>>>(a);
+  if constexpr (V == 0) {
+    if (chunk_parts(c, ctas)) {
+      k_particles<MODE, V, true><<<ctas, Win<V>::THREADS, 0, c->stream>>>(a);
+      return cudaGetLastError();
+    }
+  }
+  k_particles<MODE, V, false><<<ctas, Win<V>::THREADS, 0, c->stream>>>(a);
   return cudaGetLastError();
 }
 

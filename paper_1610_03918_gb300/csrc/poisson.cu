@@ -2384,7 +2384,7 @@ cudaError_t poisson_capture(pic_ctx *c, cudaGraph_t top, std::vector<cudaGraphNo
 int64_t poisson_kernel_count(pic_ctx *c, int64_t S, int64_t O, int64_t I) {
   // final resid, and unless the density kernel opens the solve: guess and init
   int64_t per_solve = 1 + (c->cfg.warm_start != 1 ? 2 : 0);
-  if (c->cfg.warm_start == 3) per_solve += 2 + unet_forward_kernels();   // absmax, input, network
+  if (c->cfg.warm_start == 3) per_solve += 2 + unet_forward_kernels(c->net);   // absmax, input, network
   if (closing_cluster(c))   // opening pass, solve, closing kernel (further passes are its own)
     return S * (per_solve + 1 + (c->fp.enabled ? c->fp.kernels : 2));
   if (one_pass_solver(c))   // per pass: resid, solve (which corrects phi)
@@ -2527,7 +2527,7 @@ cudaError_t launch_learned_guess(pic_ctx *c) {
   unet_forward_only(c->net, c->d_net_x);
   launch(k_guess_learned_dev, c->red.nblocks, kThreads, 0, c->stream, c->d_phi, c->d_phiL, c->d_nodeflags,
          unet_output(c->net), smax, nn);
-  c->launches += 3 + unet_forward_kernels();
+  c->launches += 3 + unet_forward_kernels(c->net);
   return cudaGetLastError();
 }
 

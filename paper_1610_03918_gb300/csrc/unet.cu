@@ -1822,9 +1822,15 @@ const float *unet_output(const pic_unet *u) { return u->y; }
 int unet_height(const pic_unet *u) { return u->H; }
 int unet_width(const pic_unet *u) { return u->W; }
 int unet_batch(const pic_unet *u) { return u->B; }
-// kernels one forward launches: the input conversion, 14 convolutions, 3
-// pools, 3 transposed convolutions and the head
-int unet_forward_kernels() { return 1 + 14 + 3 + 3 + 1; }
+// kernels one forward launches: 14 convolutions (the first one from the FP32
+// input), 3 transposed convolutions, the head, and the pools that no convolution's
+// epilogue takes
+int unet_forward_kernels(const pic_unet *u) {
+  int pools = 0;
+  for (int l = 0; l < 3; ++l)
+    if (u->conv_impl != 0 || (u->W >> l) < 128) ++pools;
+  return 14 + 3 + 1 + pools;
+}
 // copies the FP32 parameters of src into dst (same architecture) on dst's stream
 pic_status unet_copy_params(pic_unet *dst, const pic_unet *src) {
   if (dst->nparam != src->nparam) return PIC_EINVAL;
