@@ -39,11 +39,11 @@ BYTES_PER_PARTICLE_STEP = 40
 # capture (dram__bytes_read.sum + dram__bytes_write.sum over the launch),
 # valid for the kernel source whose hash is recorded with it.
 NCU_TRAFFIC = {
-    # k_particles<0, 0>, 512x1024 trench at 20 ppc (16.96M particles, 0.4 GB of
-    # state, larger than L2), launches 3 and 4: 354.4 MB read + 287.4 / 284.2
-    # MB written
-    "source_sha256": "15dc1fe1b005f98e3c89cc6f7b48311bb7e7475cd7c9646380bd9e7e747d9204",
-    "bytes_per_particle": 37.76,
+    # k_particles<0, 0, true>, 512x1024 trench at 40 ppc (33.91M particles, 0.8 GB
+    # of state, larger than L2, chunks in parts as at 100 ppc), launches 3 and 4:
+    # 694.5 MB read + 626.3 / 622.9 MB written
+    "source_sha256": "4a4e9716966d035f1260111005724054abc81cd0390e64e01fe9a6d0b0f25fa6",
+    "bytes_per_particle": 38.9,
 }
 
 
