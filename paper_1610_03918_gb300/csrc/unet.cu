@@ -17,7 +17,8 @@
 // With conv_impl = 1, or where a shape does not fit, the 3x3 convolutions
 // (forward and data gradient) are implicit GEMMs with mma.sync (m16n8k16 BF16 ->
 // FP32, ldmatrix fragments, cp.async double-buffered tiles): M = pixels of one row
-// segment, N = output channels, K = 9 taps x input channels.  The data gradient is
+// segment (up to 48 pixels wide: pixels of several rows), N = output channels, K = 9
+// taps x input channels.  The data gradient is
 // the same kernel with the weights flipped in space and transposed in channels.
 // The weight gradient is a GEMM over pixels (M = out channels, N = in channels per
 // tap) accumulated with FP32 atomics; the transposed convolutions run on the CUDA
@@ -202,6 +203,104 @@ __global__ void __launch_bounds__(kConvThreads) k_conv3x3(ConvArgs a) {
   }
 }
 
+// The same layer on narrow images: tiles of 32 pixels in the order of the batch's
+// pixels, whatever row they lie in, by 32 output channels, where the kernel above has
+// a row's few pixels in a tile of 128.  A layer of few pixels is bound by the latency
+// of its K steps in turn: steps of 64 channels, the loads four steps ahead, small
+// tiles for more CTAs.  K is summed in the same order by the same instruction: the
+// same results bit for bit.  A call of 256 -> 256 channels at 64 x 3 pixels 62 -> 22 us,
+// at 4 x 129 x 7 295 -> 45 us.
+constexpr int kPxM = 32, kPxN = 32, kPxK = 64, kPxStages = 5, kPxThreads = 128;
+
+__global__ void __launch_bounds__(kPxThreads) k_conv3x3_px(ConvArgs a) {
+  constexpr int LD = kPxK + 8;             // padded rows: conflict-free ldmatrix
+  constexpr int CH = kPxK / 8, ROWS = kPxThreads / CH, NR = kPxM / ROWS;
+  __shared__ __align__(16) bf16 As[kPxStages][kPxM * LD];
+  __shared__ __align__(16) bf16 Bs[kPxStages][kPxN * LD];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int wm = warp >> 1, wn = warp & 1;
+  const int np = a.B * a.H * a.W;
+  const int p0 = blockIdx.x * kPxM, n0 = blockIdx.y * kPxN;
+  const int kchunks = a.cin / kPxK, nk = 9 * kchunks;
+  pdl_enter();
+
+  // this thread's 16-byte chunk of NR pixels and of as many weight rows
+  const int row = tid / CH, cc = (tid % CH) * 8;
+  int px[NR], py[NR];
+#pragma unroll
+  for (int r = 0; r < NR; ++r) {
+    const int p = p0 + row + r * ROWS;
+    px[r] = p % a.W;
+    py[r] = p < np ? (p / a.W) % a.H : -2;   // past the last pixel: no tap is inside
+  }
+  auto load = [&](int ks) {
+    if (ks < nk) {
+      const int st = ks % kPxStages, tap = ks / kchunks, c = (ks - tap * kchunks) * kPxK + cc;
+      const int di = tap / 3 - 1, dj = tap % 3 - 1;
+#pragma unroll
+      for (int r = 0; r < NR; ++r) {
+        const int m = row + r * ROWS, hh = py[r] + di, ww = px[r] + dj;
+        const bool ok = hh >= 0 && hh < a.H && ww >= 0 && ww < a.W;
+        const bf16 *src = ok ? a.in + size_t(p0 + m + di * a.W + dj) * a.in_cs + a.in_off + c : a.in;
+        cp_async16(&As[st][m * LD + cc], src, ok);
+        cp_async16(&Bs[st][m * LD + cc], a.w + (size_t(n0 + m) * 9 + tap) * a.cin + c, true);
+      }
+    }
+    cp_async_commit();                       // a group a step, the last ones empty
+  };
+
+  float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+  for (int ks = 0; ks < kPxStages - 1; ++ks) load(ks);
+  for (int ks = 0; ks < nk; ++ks) {
+    const int st = ks % kPxStages;
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(kPxStages - 2));
+    __syncthreads();                         // step ks is here, step ks - 1's stage is free
+    load(ks + kPxStages - 1);
+#pragma unroll
+    for (int kk = 0; kk < kPxK; kk += 16) {
+      unsigned a0, a1, a2, a3, b0, b1, b2, b3;
+      ldsm_x4(a0, a1, a2, a3, &As[st][(wm * 16 + (lane & 15)) * LD + kk + (lane >> 4) * 8]);
+      const int mi = lane >> 3;
+      ldsm_x4(b0, b1, b2, b3,
+              &Bs[st][(wn * 16 + (lane & 7) + ((mi >> 1) << 3)) * LD + kk + ((mi & 1) << 3)]);
+      mma16816(acc[0], a0, a1, a2, a3, b0, b1);
+      mma16816(acc[1], a0, a1, a2, a3, b2, b3);
+    }
+  }
+#pragma unroll
+  for (int nf = 0; nf < 2; ++nf) {
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+      const int p = p0 + wm * 16 + (lane >> 2) + half * 8;
+      const int n = n0 + wn * 16 + nf * 8 + (lane & 3) * 2;
+      if (p >= np) continue;
+      float v0 = acc[nf][half * 2 + 0], v1 = acc[nf][half * 2 + 1];
+      if (a.bias) {
+        v0 += a.bias[n];
+        v1 += a.bias[n + 1];
+      }
+      if (a.relu) {
+        v0 = fmaxf(v0, 0.f);
+        v1 = fmaxf(v1, 0.f);
+      }
+      bf16 *dst = a.out + size_t(p) * a.out_cs + a.out_off + n;
+      *reinterpret_cast<__nv_bfloat162 *>(dst) = __floats2bfloat162_rn(v0, v1);
+    }
+  }
+}
+
+// True if it was launched: images up to kPxMaxW wide, channels in whole tiles and steps.
+// The line: at 48 pixels small and large layers gain (1 x 128 x 48, 64 channels 22.6 -> 17.1
+// us; 4 x 516 x 48, 128 channels 290 -> 218), at 64, half of the row tile, the small one
+// does (22.9 -> 16.1) and the large one not (4 x 1032 x 64, 64 channels 160 -> 179).
+constexpr int kPxMaxW = 48;
+bool conv_px(const ConvArgs &a, cudaStream_t s) {
+  const long long np = (long long)a.B * a.H * a.W;
+  if (a.W > kPxMaxW || a.cin % kPxK || a.cout % kPxN || np + kPxM >= (1LL << 31) || a.cout / kPxN > 65535) return false;
+  return launch(k_conv3x3_px, dim3(unsigned((np + kPxM - 1) / kPxM), unsigned(a.cout / kPxN)), kPxThreads, 0, s, a) ==
+         cudaSuccess;
+}
+
 // ---------------------------------------------------------------- 3x3 weight gradient
 // dW[co][tap][ci] += sum_p dpre[p][co] * in[p + off(tap)][ci] over a group of
 // rows; 32 x 32 tile of (co, ci) per CTA, 4 warps of 16 x 16.
@@ -364,40 +463,95 @@ __global__ void __launch_bounds__(256) k_wflip(FlipArgs a) {
   }
 }
 
-// transposed 2x2 stride-2 convolution: out (2h x 2w) from in (h x w); W [2][2][ci][co] FP32
-__global__ void k_up_fwd(const bf16 *in, int cin, const float *w, const float *bias, bf16 *out,
-                         int out_cs, int out_off, int cout, int B, int h, int wd) {
-  const int H = 2 * h, W = 2 * wd;
-  GSTRIDE(i, (long long)B * H * W * cout) {
-    const int co = int(i % cout);
-    const long long p = i / cout;
-    const int x = int(p % W), y = int((p / W) % H), b = int(p / ((long long)W * H));
-    const int a = y & 1, c = x & 1;
-    const bf16 *src = in + ((size_t(b) * h + (y >> 1)) * wd + (x >> 1)) * cin;
-    const float *wk = w + (size_t(a * 2 + c) * cin) * cout + co;
-    float s = bias[co];
-    for (int ci = 0; ci < cin; ++ci) s = fmaf(__bfloat162float(src[ci]), wk[size_t(ci) * cout], s);
-    out[p * out_cs + out_off + co] = __float2bfloat16(s);
+// The transposed 2x2 stride-2 convolution on CUDA cores, where the tensor-core kernels
+// do not apply: out (2h x 2w) from in (h x w), W [2][2][cin][cout] FP32; BACK: its data
+// gradient, gin (h x w, cin) from gout (2h x 2w, cout).  A CTA takes 16 pixels of the
+// small image by 32 result channels (forward: of one of the four children, blockIdx.y)
+// and goes through K 32 values a step, weights and pixels staged in shared memory, the
+// next step's loads in flight meanwhile; an output is one thread's chain of FMAs in the
+// order of K.  With a thread an output and W from memory: 50 us forward for 256 -> 128
+// channels at 4 x 32 x 3 pixels and 203 us for its gradient, whose lanes read W a row
+// apart; now 13 and 28 us (bound by the latency of 8 and 16 steps); a pass of forward and gradients at 4 x 256 x 24 1951 -> 716 us with this and
+// k_conv3x3_px, a forward pass at 2 x 416 x 24 427 -> 143.
+constexpr int kUpPx = 16;
+
+template <bool BACK>
+__global__ void __launch_bounds__(256) k_up(const bf16 *src, int src_cs, int src_off, const float *w, const float *bias,
+                                            bf16 *dst, int dst_cs, int dst_off, int cin, int cout, int B, int h, int wd) {
+  __shared__ float ws[32][33];               // [k][n]
+  __shared__ __align__(16) float xs[kUpPx][36];   // [pixel][k]
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int N = BACK ? cin : cout, K = BACK ? cout : cin;
+  const int nb = (N + 31) / 32, n0 = int(blockIdx.x % nb) * 32;
+  const long long np = (long long)B * h * wd, p0 = (long long)(blockIdx.x / nb) * kUpPx;
+  const int steps = (K + 31) / 32, total = (BACK ? 4 : 1) * steps;
+  pdl_enter();
+
+  // the child t of pixel p in the large image, as a pixel number
+  auto child = [&](long long p, int t) {
+    const int x = int(p % wd);
+    return (2 * (p / wd) + (t >> 1)) * (2 * wd) + 2 * x + (t & 1);   // rows of all images in turn
+  };
+  float wr[4], xr[2];
+  auto fetch = [&](int it) {
+    const int t = BACK ? it / steps : int(blockIdx.y), k0 = (it % steps) * 32;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int q = ty + 8 * r;              // the row of W that this warp reads
+      const int ci = BACK ? n0 + q : k0 + q, co = BACK ? k0 + tx : n0 + tx;
+      wr[r] = ci < cin && co < cout ? w[(size_t(t) * cin + ci) * cout + co] : 0.f;
+    }
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      const long long p = p0 + ty + 8 * r;
+      xr[r] = p < np && k0 + tx < K
+                  ? __bfloat162float(src[size_t(BACK ? child(p, t) : p) * src_cs + src_off + k0 + tx]) : 0.f;
+    }
+  };
+  float s[2];
+  s[0] = s[1] = !BACK && n0 + tx < N ? bias[n0 + tx] : 0.f;
+  fetch(0);
+  for (int it = 0; it < total; ++it) {
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      if (BACK) ws[tx][ty + 8 * r] = wr[r];
+      else ws[ty + 8 * r][tx] = wr[r];
+    }
+#pragma unroll
+    for (int r = 0; r < 2; ++r) xs[ty + 8 * r][tx] = xr[r];
+    __syncthreads();
+    if (it + 1 < total) fetch(it + 1);
+    const int kn = min(32, K - (it % steps) * 32);
+    if (kn == 32) {
+#pragma unroll
+      for (int k = 0; k < 32; k += 4) {
+        const float4 u = *reinterpret_cast<const float4 *>(&xs[ty][k]), v = *reinterpret_cast<const float4 *>(&xs[ty + 8][k]);
+        const float w0 = ws[k][tx], w1 = ws[k + 1][tx], w2 = ws[k + 2][tx], w3 = ws[k + 3][tx];
+        s[0] = fmaf(u.w, w3, fmaf(u.z, w2, fmaf(u.y, w1, fmaf(u.x, w0, s[0]))));
+        s[1] = fmaf(v.w, w3, fmaf(v.z, w2, fmaf(v.y, w1, fmaf(v.x, w0, s[1]))));
+      }
+    } else {
+      for (int k = 0; k < kn; ++k) {
+        s[0] = fmaf(xs[ty][k], ws[k][tx], s[0]);
+        s[1] = fmaf(xs[ty + 8][k], ws[k][tx], s[1]);
+      }
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    const long long p = p0 + ty + 8 * r;
+    if (p < np && n0 + tx < N)
+      dst[size_t(BACK ? p : child(p, int(blockIdx.y))) * dst_cs + dst_off + n0 + tx] = __float2bfloat16(s[r]);
   }
 }
 
-// data gradient of the transposed convolution: gin (h x w, cin) from gout (2h x 2w, cout)
-__global__ void k_up_back_data(const bf16 *gout, int gout_cs, int gout_off, int cout, const float *w,
-                               bf16 *gin, int cin, int B, int h, int wd) {
-  const int W = 2 * wd;
-  GSTRIDE(i, (long long)B * h * wd * cin) {
-    const int ci = int(i % cin);
-    const long long p = i / cin;
-    const int x = int(p % wd), y = int((p / wd) % h), b = int(p / ((long long)wd * h));
-    float s = 0.f;
-    for (int a = 0; a < 2; ++a)
-      for (int c = 0; c < 2; ++c) {
-        const bf16 *g = gout + ((size_t(b) * 2 * h + 2 * y + a) * W + 2 * x + c) * gout_cs + gout_off;
-        const float *wk = w + (size_t(a * 2 + c) * cin + ci) * cout;
-        for (int co = 0; co < cout; ++co) s = fmaf(__bfloat162float(g[co]), wk[co], s);
-      }
-    gin[i] = __float2bfloat16(s);
-  }
+template <bool BACK>
+void launch_up(const bf16 *src, int src_cs, int src_off, const float *w, const float *bias, bf16 *dst, int dst_cs,
+               int dst_off, int cin, int cout, int B, int h, int wd, cudaStream_t s) {
+  const long long px = ((long long)B * h * wd + kUpPx - 1) / kUpPx, nb = ((BACK ? cin : cout) + 31) / 32;
+  launch(k_up<BACK>, dim3(unsigned(px * nb), BACK ? 1 : 4), 256, 0, s, src, src_cs, src_off, w, bias, dst, dst_cs,
+         dst_off, cin, cout, B, h, wd);
 }
 
 // weight gradient of the transposed convolution: dw[a][c][ci][co] += sum over input pixels
@@ -840,6 +994,7 @@ void conv_fwd(pic_unet *u, int ci, const bf16 *in, int in_cs, int in_off, bf16 *
   a.H = u->H >> l;
   a.W = u->W >> l;
   a.relu = relu ? 1 : 0;
+  if (conv_px(a, u->stream)) return;
   const int nwt = (a.W + kTM - 1) / kTM;
   if (c.cout == 32) {
     dim3 g(a.B * a.H * nwt, 1);
@@ -902,6 +1057,7 @@ bool conv_back_data(pic_unet *u, int ci, const bf16 *dpre, bf16 *gin, int gin_cs
   a.H = u->H >> l;
   a.W = u->W >> l;
   a.relu = 0;
+  if (conv_px(a, u->stream)) return false;
   const int nwt = (a.W + kTM - 1) / kTM;
   if (a.cout == 32) {
     k_conv3x3<32, 32><<<dim3(a.B * a.H * nwt, 1), kConvThreads, 0, u->stream>>>(a);
@@ -1125,8 +1281,8 @@ void forward(pic_unet *u, const float *x, bool keep_input, float *y = nullptr) {
     const pic_unet::Up &up = u->up[l];
     const int hl = u->H >> (l + 1), wl = u->W >> (l + 1);
     if (!up_tc(u, l, h, hc))
-      k_up_fwd<<<gridn((long long)pix(u, l) * up.cout), 256, 0, u->stream>>>(
-          h, hc, u->P + up.w_off, u->P + up.b_off, u->cat[l], 2 * kC[l], 0, up.cout, u->B, hl, wl);
+      launch_up<false>(h, hc, 0, u->P + up.w_off, u->P + up.b_off, u->cat[l], 2 * kC[l], 0, hc, up.cout, u->B, hl, wl,
+                       u->stream);
     const int ca = (l == 2) ? D2A : (l == 1) ? D1A : D0A;
     conv_fwd(u, ca, u->cat[l], 2 * kC[l], 0, u->da[l], kC[l], 0, l, true);
     conv_fwd(u, ca + 1, u->da[l], kC[l], 0, u->dout[l], kC[l], 0, l, true);
@@ -1162,8 +1318,8 @@ void backward(pic_unet *u) {
     dpre = gin;
     if (!up_back_tc(u, l, gin, last, hin)) {
       if (!up_back_tc(u, l, gin))
-        k_up_back_data<<<gridn((long long)pix(u, l + 1) * up.cin), 256, 0, u->stream>>>(
-            u->gcat[l], 2 * C, 0, up.cout, u->P + up.w_off, gin, up.cin, u->B, hl, wl);
+        launch_up<true>(u->gcat[l], 2 * C, 0, u->P + up.w_off, nullptr, gin, up.cin, 0, up.cin, up.cout, u->B, hl, wl,
+                        u->stream);
       relu_back(u, last, gin, up.cin, 0, hin, up.cin, 0, l + 1);
       dpre = u->dpre[l + 1];
     }
@@ -1528,7 +1684,9 @@ pic_status pic_conv3x3_bf16(int32_t impl, int32_t B, int32_t H, int32_t W, const
   a.W = W;
   a.relu = relu ? 1 : 0;
   const int nwt = (W + kTM - 1) / kTM;
-  if (cout == 32 && cin == 16)
+  if ((cout == 32 || cout % 64 == 0) && conv_px(a, s))
+    ;
+  else if (cout == 32 && cin == 16)
     k_conv3x3<32, 16><<<dim3(B * H * nwt, 1), kConvThreads, 0, s>>>(a);
   else if (cout == 32 && cin % 32 == 0)
     k_conv3x3<32, 32><<<dim3(B * H * nwt, 1), kConvThreads, 0, s>>>(a);
@@ -1652,7 +1810,7 @@ pic_status pic_upconv_bf16(int32_t impl, int32_t B, int32_t H, int32_t W, const 
   const bf16 *bi = static_cast<const bf16 *>(in);
   bf16 *bo = static_cast<bf16 *>(out);
   if (impl == 1) {
-    k_up_fwd<<<gridn(4LL * B * H * W * cout), 256, 0, s>>>(bi, cin, w, bias, bo, out_cs, out_off, cout, B, H, W);
+    launch_up<false>(bi, cin, 0, w, bias, bo, out_cs, out_off, cin, cout, B, H, W, s);
     if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) return PIC_ECUDA;
     return PIC_OK;
   }
@@ -1747,8 +1905,7 @@ pic_status pic_upconv_back_bf16(int32_t impl, int32_t B, int32_t H, int32_t W, c
   const bf16 *bg = static_cast<const bf16 *>(gout);
   bf16 *bin = static_cast<bf16 *>(gin);
   if (impl == 1) {
-    k_up_back_data<<<gridn((long long)B * H * W * cin), 256, 0, s>>>(bg, gout_cs, gout_off, cout, w, bin, cin,
-                                                                    B, H, W);
+    launch_up<true>(bg, gout_cs, gout_off, w, nullptr, bin, cin, 0, cin, cout, B, H, W, s);
     if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) return PIC_ECUDA;
     return PIC_OK;
   }
