@@ -17,9 +17,9 @@
 // With conv_impl = 1, or where a shape does not fit, the 3x3 convolutions
 // (forward and data gradient) are implicit GEMMs with mma.sync (m16n8k16 BF16 ->
 // FP32, ldmatrix fragments, cp.async double-buffered tiles): M = pixels of one row
-// segment (up to 48 pixels wide: pixels of several rows), N = output channels, K = 9
-// taps x input channels.  The data gradient is
-// the same kernel with the weights flipped in space and transposed in channels.
+// segment (on images up to 48 wide, of several rows), N = output channels, K = 9 taps
+// x input channels.  The data gradient is the same kernel with the weights flipped in
+// space and transposed in channels.
 // The weight gradient is a GEMM over pixels (M = out channels, N = in channels per
 // tap) accumulated with FP32 atomics; the transposed convolutions run on the CUDA
 // cores.
@@ -469,10 +469,11 @@ __global__ void __launch_bounds__(256) k_wflip(FlipArgs a) {
 // small image by 32 result channels (forward: of one of the four children, blockIdx.y)
 // and goes through K 32 values a step, weights and pixels staged in shared memory, the
 // next step's loads in flight meanwhile; an output is one thread's chain of FMAs in the
-// order of K.  With a thread an output and W from memory: 50 us forward for 256 -> 128
-// channels at 4 x 32 x 3 pixels and 203 us for its gradient, whose lanes read W a row
-// apart; now 13 and 28 us (bound by the latency of 8 and 16 steps); a pass of forward and gradients at 4 x 256 x 24 1951 -> 716 us with this and
-// k_conv3x3_px, a forward pass at 2 x 416 x 24 427 -> 143.
+// order of K.  With a thread an output and W from memory it took 50 us forward for 256
+// -> 128 channels at 4 x 32 x 3 pixels and 203 us for its gradient, whose lanes read W a
+// row apart; now 13 and 28 us, the latency of 8 and 16 steps.  A pass of forward and
+// gradients at 4 x 256 x 24 went from 1951 to 716 us with this and k_conv3x3_px, a
+// forward pass at 2 x 416 x 24 from 427 to 143.
 constexpr int kUpPx = 16;
 
 template <bool BACK>
@@ -525,7 +526,8 @@ __global__ void __launch_bounds__(256) k_up(const bf16 *src, int src_cs, int src
     if (kn == 32) {
 #pragma unroll
       for (int k = 0; k < 32; k += 4) {
-        const float4 u = *reinterpret_cast<const float4 *>(&xs[ty][k]), v = *reinterpret_cast<const float4 *>(&xs[ty + 8][k]);
+        const float4 u = *reinterpret_cast<const float4 *>(&xs[ty][k]);
+        const float4 v = *reinterpret_cast<const float4 *>(&xs[ty + 8][k]);
         const float w0 = ws[k][tx], w1 = ws[k + 1][tx], w2 = ws[k + 2][tx], w3 = ws[k + 3][tx];
         s[0] = fmaf(u.w, w3, fmaf(u.z, w2, fmaf(u.y, w1, fmaf(u.x, w0, s[0]))));
         s[1] = fmaf(v.w, w3, fmaf(v.z, w2, fmaf(v.y, w1, fmaf(v.x, w0, s[1]))));
