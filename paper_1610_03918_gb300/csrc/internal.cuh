@@ -35,9 +35,7 @@ constexpr TileVariant kTileVariants[kNumTileVariants] = {
     {5, 5, 4, 256},    // 32 x 32
 };
 constexpr int kMinTileLog2 = 4;  // the smallest tile (16 x 16) sizes the tile arrays
-constexpr int kChunk = 4092;     // particles whose sums fit 32 bits (multiple of 4, <= 4095)
-constexpr int kMaxChunk = 4 * kChunk;   // particles per work item
-constexpr int kShareParts = 4;   // a resident CTA's share of the particles, in work items at least
+constexpr int kChunk = 4092;     // particles per work item (multiple of 4, <= 4095)
 constexpr int kRunSteps = 8;     // most steps of one graph launch
 constexpr int kMinChunk = 512;   // one pass of the particle kernel's smaller CTA
 constexpr int kMaxCtasPerSm = 16;

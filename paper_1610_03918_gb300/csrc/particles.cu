@@ -50,7 +50,6 @@ struct SortArgs {
   Geom g;
   int ntiles;
   int ctas;                // CTAs of the particle kernel resident at once
-  int max_chunk;           // particles of a chunk at most (kChunk or kMaxChunk)
 };
 
 // The counting passes take 4 consecutive slots per lane and vector (16-byte
@@ -147,10 +146,6 @@ __device__ uint2 block_exscan(uint2 v, uint2 *total) {
 // 13M particles in 16 x 16 tiles 2.6 chunks a CTA, which run as long as 3.
 // Equal parts, because a remainder costs a whole window: 4096 particles a tile
 // (16 per cell) made a chunk of 4092 and one of 4 (512 x 512: 80.3 -> 71.7 us).
-// Where a CTA's share is worth it, up to kMaxChunk and a kShareParts-th of the
-// share (k_particles' PARTS), but for the last quarter of the particles, whose
-// chunks stay at `most`, so that the CTAs end together (1024 x 512 with 84.5M:
-// 560 us; with an eighth of the share 585, a sixteenth 604).
 __global__ void __launch_bounds__(1024) k_sort_scan(SortArgs a) {
   __shared__ uint32_t s_first[1024];   // first chunk of each tile of the round
   __shared__ uint32_t s_off[1024], s_padded[1024];
@@ -158,17 +153,13 @@ __global__ void __launch_bounds__(1024) k_sort_scan(SortArgs a) {
   const int64_t share = (a.nslots[0] + a.nslots[1] + a.ctas - 1) / a.ctas;
   const int64_t rounds = max(int64_t(1), (share + kChunk - 1) / kChunk), part = (share + rounds - 1) / rounds;
   const uint32_t most = uint32_t(min(int64_t(kChunk), max(int64_t(kMinChunk), (part + kMinChunk - 1) / kMinChunk * kMinChunk)));
-  const uint32_t big = uint32_t(max(int64_t(most), min(int64_t(a.max_chunk), share / kShareParts)));
-  auto chunks_of = [&](uint32_t padded, int sp, int t) {
-    const uint32_t cap = sp == 1 && 2 * t >= a.ntiles ? most : big;
-    return (padded + cap - 1) / cap;
-  };
+  auto chunks_of = [&](uint32_t padded) { return (padded + most - 1) / most; };
   uint32_t slot_base = 0, chunk_base = 0;
   if (s == 1)
     for (int t0 = 0; t0 < a.ntiles; t0 += 1024) {
       const int t = t0 + threadIdx.x;
       uint2 tot;
-      block_exscan(make_uint2(0u, t < a.ntiles ? chunks_of((a.count[t] + 3u) & ~3u, 0, t) : 0u), &tot);
+      block_exscan(make_uint2(0u, t < a.ntiles ? chunks_of((a.count[t] + 3u) & ~3u) : 0u), &tot);
       chunk_base += tot.y;
     }
   uint32_t *cur = a.cursor + int64_t(s) * a.ntiles;
@@ -182,7 +173,7 @@ __global__ void __launch_bounds__(1024) k_sort_scan(SortArgs a) {
       padded = (n + 3u) & ~3u;
     }
     uint2 tot;
-    const uint2 ex = block_exscan(make_uint2(padded, chunks_of(padded, s, t)), &tot);
+    const uint2 ex = block_exscan(make_uint2(padded, chunks_of(padded)), &tot);
     const uint32_t off = ex.x + slot_base;
     s_first[threadIdx.x] = ex.y;
     s_off[threadIdx.x] = off;
@@ -201,7 +192,7 @@ __global__ void __launch_bounds__(1024) k_sort_scan(SortArgs a) {
         if (s_first[mid] <= c) lo = mid; else hi = mid;
       }
       const uint32_t q = c - s_first[lo], pad = s_padded[lo];
-      const uint32_t parts = chunks_of(pad, s, t0 + lo), per = ((pad + parts - 1) / parts + 3u) & ~3u;
+      const uint32_t parts = chunks_of(pad), per = ((pad + parts - 1) / parts + 3u) & ~3u;
       const uint32_t b0 = s_off[lo] + min(pad, q * per);
       const uint32_t b1 = s_off[lo] + min(pad, (q + 1) * per);
       reinterpret_cast<int4 *>(a.chunks)[chunk_base + c] = make_int4(s, t0 + lo, int(b0), int(b1));
@@ -682,28 +673,16 @@ __device__ __forceinline__ void prefetch_l2(const void *p, unsigned bytes) {
 // registers and 10 CTAs: 677 us): 5.74 TB/s of algorithmic traffic, 0.85 of a
 // copy's.  Sparing the particles of all-interior windows the cell mask's look
 // (+3%), the next chunk's first state prefetched across the chunk boundary
-// (+1.6%), loads past L1 (+11%) and plain stores (+0.4%) did not pay.
-//
-// PARTS: chunks of up to kMaxChunk particles.  A chunk costs its window whatever
-// it holds (625 nodes staged, cleared and added with 64-bit atomics), and above
-// kChunk particles the 32-bit sums have to be carried between parts: 84.5M
-// particles, 20.6k a tile, 589 us in chunks of 4.1k, 560 in halves of a tile.  The
-// loop over the parts costs 1% where there is one (8.4M: 107.8 -> 108.7 us), so it
-// is for loads whose chunks come out larger (chunk_parts).
-template <int MODE, int V, bool PARTS>
+// (+1.6%), loads past L1 (+11%) and plain stores (+0.4%) did not pay.  Chunks of up
+// to four times kChunk, their sums carried between parts of kChunk, gave 560 us with
+// these tiles, but the same loop with the larger ones ended in an SM exception that
+// reading and range checks did not explain: there is no such loop.
+template <int MODE, int V>
 __global__ void __launch_bounds__(Win<V>::THREADS, Win<V>::THREADS == 128 ? 9 : 4) k_particles(PArgs a) {
   constexpr int NWX = Win<V>::NWX, NWY = Win<V>::NWY, THREADS = Win<V>::THREADS;
   __shared__ float2 sE[NWX * NWY];
   __shared__ uint32_t sAcc[NWX * NWY];
-  __shared__ int16_t sHigh[PARTS ? NWX * NWY : 1];   // what earlier parts of a chunk added, in units of 2^20
   __shared__ double sRed[THREADS / 32];
-  // A node's sum over kChunk particles, on top of less than 2^20 of earlier ones,
-  // lies in [-kChunk, (kChunk + 1) 2^20): each adds a share in [-1, 2^20].  That
-  // range is narrower than 2^32, so the 32-bit sum decodes uniquely; values from
-  // (kChunk + 1) 2^20 on are the negative ones.
-  auto decode = [](uint32_t v) {
-    return v >= uint32_t(kChunk + 1) * kQ ? (long long)v - (1ll << 32) : (long long)v;
-  };
   const Geom g = a.g;
   const int nch = *a.nchunks;
   const int nnodes = g.nxn * g.nyn;
@@ -753,10 +732,7 @@ __global__ void __launch_bounds__(Win<V>::THREADS, Win<V>::THREADS == 128 ? 9 : 
       }
     };
     for (int d = 0; d < kPrefetchAhead; ++d) prefetch(int64_t(ch.begin) + d * step);
-    int p0 = ch.begin;
-    for (;;) {
-    const int p1 = PARTS ? min(p0 + kChunk, ch.end) : ch.end;
-    for (int64_t base = p0 + 4 * threadIdx.x; base < p1; base += 4 * blockDim.x) {
+    for (int64_t base = ch.begin + 4 * threadIdx.x; base < ch.end; base += 4 * blockDim.x) {
       prefetch(base - 4 * threadIdx.x + kPrefetchAhead * step);
       int4 c4 = *reinterpret_cast<const int4 *>(P.cell + base);
       float4 fx4 = *reinterpret_cast<const float4 *>(P.fx + base);
@@ -782,25 +758,18 @@ __global__ void __launch_bounds__(Win<V>::THREADS, Win<V>::THREADS == 128 ? 9 : 
       }
     }
     __syncthreads();
-    if (!PARTS || p1 == ch.end) break;
-    // between the parts a sum keeps its low 20 bits, the rest moves to the 16 beside it
     if (MODE != 2) {
       for (int k = threadIdx.x; k < NWX * NWY; k += blockDim.x) {
-        const long long x = decode(sAcc[k]);
-        sHigh[k] = int16_t((p0 > ch.begin ? sHigh[k] : 0) + int(x >> 20));
-        sAcc[k] = uint32_t(x) & (kQ - 1u);
-      }
-      __syncthreads();
-    }
-    p0 = p1;
-    }
-    if (MODE != 2) {
-      for (int k = threadIdx.x; k < NWX * NWY; k += blockDim.x) {
-        const long long x = decode(sAcc[k]) + (PARTS && p0 > ch.begin ? (long long)sHigh[k] << 20 : 0ll);
-        if (x) {
+        const uint32_t v = sAcc[k];
+        if (v) {
           const int wi = k / NWY, wj = k - (k / NWY) * NWY;
           int gi = wi0 + wi, gj = wj0 + wj;
           wrap_node(gi, gj);
+          // The node's sum over the chunk lies in [-kChunk, kChunk * 2^20]: each of
+          // at most kChunk particles adds a share in [-1, 2^20].  That range is
+          // narrower than 2^32, so the 32-bit sum decodes uniquely; values above
+          // kChunk * 2^20 are the negative ones.
+          const long long x = v > uint32_t(kChunk) * kQ ? (long long)v - (1ll << 32) : (long long)v;
           if (gi >= 0 && gi < g.nxn && gj >= 0 && gj < g.nyn)
             atomicAdd(&acc[gi * g.nyn + gj], (unsigned long long)x);
         }
@@ -962,36 +931,17 @@ __global__ void k_moments(ParticleBuf P, const int64_t *nslots_p, double *part) 
   }
 }
 
-// the CTAs of the resident ones that a context counts on (an ensemble's members share the GPU)
-int own_ctas(const pic_ctx *c, int resident) { return std::max(1, resident / std::max(1, c->sharing)); }
-// whether the particles the context has room for make chunks larger than kChunk.  Not in
-// an ensemble, whose members find more of the GPU free than their part at times and
-// share out their chunks over that: 8 members 280 -> 291 us a step.  Nor with the other
-// tile shapes: a build of their kernels with the parts' loop ended in an SM exception
-// on 34M particles, with every chunk, cell and slot checked in range; the cause was not
-// found, and those kernels are not built.
-bool chunk_parts(const pic_ctx *c, int resident) {
-  return c->tile_variant == 0 && c->sharing <= 1 && (c->cap[0] + c->cap[1]) / resident / kShareParts > kChunk;
-}
-
 // CTAs of the step kernel that are resident at once
 template <int V>
 int resident_ctas(const pic_ctx *c) {
   int per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_particles<0, V, V == 0>, Win<V>::THREADS, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_particles<0, V>, Win<V>::THREADS, 0);
   return c->num_sms * std::min(std::max(per_sm, 1), kMaxCtasPerSm);
 }
 
 template <int MODE, int V>
 cudaError_t launch_particles_v(pic_ctx *c, const PArgs &a) {
-  const int ctas = resident_ctas<V>(c);
-  if constexpr (V == 0) {
-    if (chunk_parts(c, ctas)) {
-      k_particles<MODE, V, true><<<ctas, Win<V>::THREADS, 0, c->stream>>>(a);
-      return cudaGetLastError();
-    }
-  }
-  k_particles<MODE, V, false><<<ctas, Win<V>::THREADS, 0, c->stream>>>(a);
+  k_particles<MODE, V><<<resident_ctas<V>(c), Win<V>::THREADS, 0, c->stream>>>(a);
   return cudaGetLastError();
 }
 
@@ -1027,8 +977,7 @@ cudaError_t launch_sort(pic_ctx *c) {
     case 3: a.ctas = resident_ctas<3>(c); break;
     default: a.ctas = resident_ctas<0>(c); break;
   }
-  a.max_chunk = chunk_parts(c, a.ctas) ? kMaxChunk : kChunk;
-  a.ctas = own_ctas(c, a.ctas);
+  a.ctas = std::max(1, a.ctas / std::max(1, c->sharing));   // an ensemble's members share the GPU
   const dim3 grid(c->num_sms * 4, 2);   // 8 CTAs of 256 threads per SM: one wave
   if (a.ntiles <= kHistSmemTiles)
     k_sort_hist<true><<<grid, 256, size_t(a.ntiles) * 4, c->stream>>>(a);
