@@ -110,6 +110,12 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map
       "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(bar)
       : "memory");
 }
+// tcgen05.alloc waits, without a limit, for columns that other CTAs of the SM hold.
+// So a kernel here takes its columns in warp 0, waits for the grid before it
+// (pdl_wait), and lets the next grid's CTAs in (pdl_release) only after a barrier
+// behind the allocation: when they become resident, every CTA of this grid holds its
+// columns.  Released earlier, they could take the SM's last columns and wait for
+// this grid's end while a CTA of this grid waits for columns.
 __device__ __forceinline__ void tmem_alloc(uint32_t slot, uint32_t ncols) {
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(slot), "r"(ncols)
                : "memory");
@@ -318,10 +324,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) tmem_alloc(saddr(slot), L::NCOLS);
-  pdl_enter();
+  pdl_wait();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_release();
   const uint32_t tmem = *slot;
   const int kchunks = a.cin / KB;
   const int nk = (UP ? 1 : (HALO ? 3 : (UPB ? 4 : 9))) * kchunks;
@@ -571,11 +578,12 @@ __global__ void __launch_bounds__(kRowThreads, RowCfg<N, KB, KC>::CPS)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) tmem_alloc(saddr(slot), C::NCOLS);
-  pdl_enter();
+  pdl_wait();
   if (tid < N) reinterpret_cast<float *>(s_bias)[tid] = a.bias ? a.bias[n0 + tid] : 0.f;
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_release();
   const uint32_t tmem = *slot;
   volatile int *fail = &s_fail;
 
@@ -899,12 +907,13 @@ __global__ void __launch_bounds__(kRowThreads, 1)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) tmem_alloc(saddr(&s_slot), RING * N);
-  pdl_enter();
+  pdl_wait();
   if (tid < N)
     reinterpret_cast<float *>(s_bias)[tid] = a.bias ? a.bias[MODE == kUp ? (n0 + tid) % a.up_cout : n0 + tid] : 0.f;
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_release();
   const uint32_t tmem = s_slot;
   volatile int *fail = &s_fail;
   const int t0 = int((long long)a.tiles * blockIdx.x / gridDim.x);
@@ -1104,7 +1113,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   __shared__ float sbias[kInN];
   __shared__ int s_fail;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  pdl_enter();
+  if (warp == 0) tmem_alloc(saddr(&slot), kInN);
+  pdl_wait();
   // B[n][k] = w[n][tap][c], k = 2 tap + c < 18, else 0
   for (int i = tid; i < kInN * kInK; i += kThreads) {
     const int n = i / kInK, k = i - (i / kInK) * kInK;
@@ -1117,10 +1127,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     s_fail = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 0) tmem_alloc(saddr(&slot), kInN);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_release();
   const uint32_t tmem = slot;
   constexpr uint32_t idesc = instr_desc<kInN>();
   const unsigned npix = unsigned(B) * unsigned(H) * unsigned(W);
@@ -1298,10 +1308,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) tmem_alloc(saddr(slot), L::NCOLS);
-  pdl_enter();
+  pdl_wait();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_release();
   const uint32_t tmem = *slot;
   // the segments: n input rows from h0 of pixel column col
   long long t = t0, col = 0;
@@ -1516,10 +1527,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) tmem_alloc(saddr(slot), L::NCOLS);
-  pdl_enter();
+  pdl_wait();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_release();
   const uint32_t tmem = *slot;
 
   if (tid == 0) {

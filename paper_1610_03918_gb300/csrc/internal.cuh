@@ -261,10 +261,14 @@ struct BoxPoisson {
 // Programmatic dependent launch.  The solver's and the network's kernels wait for the grid
 // before them (its results are then visible) and at once let the next kernel
 // of the stream be scheduled, so that kernel's blocks are resident and waiting
-// when this one ends instead of being launched only then.  Both instructions
-// are no-ops for a kernel launched without the attribute.
+// when this one ends instead of being launched only then (kernels that take tensor
+// memory after their allocation: tmem_alloc in conv_tc.cu).  Both instructions are
+// no-ops for a kernel launched without the attribute.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_enter() {
-  asm volatile("griddepcontrol.wait;\n\tgriddepcontrol.launch_dependents;" ::: "memory");
+  pdl_wait();
+  pdl_release();
 }
 
 #ifndef PICGB_NO_PDL
