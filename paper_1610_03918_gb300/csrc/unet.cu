@@ -27,15 +27,14 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
 #include <new>
 #include <string>
-#include <thread>
 #include <vector>
 
+#include "errword.h"
 #include "internal.cuh"
 #include "philox.cuh"
 
@@ -1588,49 +1587,46 @@ pic_status pic_unet_load(pic_unet *u, const char *path) {
 
 namespace {
 // Error words of the layer entry points' tcgen05 kernels (a bounded wait gave
-// up).  A kernel writes its word only then, so the words stay zero and need no
-// clearing before a launch; they are managed memory, which the host reads in
-// place once the stream has ended: against a device word that is cleared
-// before and copied back after the kernel, a call of a 10 us kernel takes 19.2
-// instead of 28.6 us.  Each call in progress has a word of its own.
+// up; errword.h).  They are managed memory, which the host clears and reads in
+// place: against a device word that is cleared before and copied back after the
+// kernel, a call of a 10 us kernel takes 19.2 instead of 28.6 us.
 constexpr int kErrWords = 64;
 __managed__ int g_layer_err[kErrWords];
-std::atomic<uint64_t> g_err_taken{0};
+picgb::ErrWords g_err_pool;
+
+// waits for a call's launches on its stream (a stream in capture cannot be waited
+// for and drops what it holds)
+struct StreamDrain {
+  cudaStream_t s;
+  picgb::Drain operator()() const {
+    const cudaError_t e = cudaStreamSynchronize(s);
+    if (e == cudaSuccess) return picgb::Drain::kEnded;
+    return e == cudaErrorStreamCaptureUnsupported || e == cudaErrorStreamCaptureInvalidated ? picgb::Drain::kNotRun
+                                                                                         : picgb::Drain::kUnknown;
+  }
+};
 
 class ErrWord {
  public:
-  ErrWord() {
-    uint64_t t = g_err_taken.load(std::memory_order_relaxed);
-    for (;;) {
-      if (t == ~uint64_t(0)) {   // 64 calls in progress: until one of them returns
-        std::this_thread::yield();
-        t = g_err_taken.load(std::memory_order_relaxed);
-        continue;
-      }
-      k_ = __builtin_ctzll(~t);
-      if (g_err_taken.compare_exchange_weak(t, t | (uint64_t(1) << k_), std::memory_order_acquire)) return;
-    }
-  }
-  ~ErrWord() { g_err_taken.fetch_and(~(uint64_t(1) << k_), std::memory_order_release); }
-  ErrWord(const ErrWord &) = delete;
-  ErrWord &operator=(const ErrWord &) = delete;
+  explicit ErrWord(cudaStream_t s) : lease_(g_err_pool, g_layer_err, StreamDrain{s}) {}
   int *device() const {
     int *p = nullptr;
-    return cudaGetSymbolAddress((void **)&p, g_layer_err) == cudaSuccess ? p + k_ : nullptr;
+    return lease_.index() >= 0 && cudaGetSymbolAddress((void **)&p, g_layer_err) == cudaSuccess ? p + lease_.index()
+                                                                                               : nullptr;
   }
-  // after the stream's synchronisation: the call's status (1 producer, 2 MMA,
-  // 3 epilogue wait gave up, for pic_last_error); the word is zero again
-  pic_status read(const char *what) const {
-    volatile int *w = g_layer_err + k_;
-    const int e = *w;
-    if (!e) return PIC_OK;
-    *w = 0;
+  // the end of the call, whose launches returned st: waits for them and returns the
+  // call's status (1 producer, 2 MMA, 3 epilogue wait gave up, for pic_last_error)
+  pic_status end(pic_status st, const char *what) {
+    const int e = lease_.end();
+    if (st != PIC_OK) return st;
+    if (e < 0) return PIC_ECUDA;
+    if (e == 0) return PIC_OK;
     picgb::note(cudaErrorTimeout, (std::string("tcgen05 ") + what + " wait " + std::to_string(e)).c_str());
     return PIC_ETIMEOUT;
   }
 
  private:
-  int k_ = 0;
+  picgb::ErrLease<StreamDrain> lease_;
 };
 }  // namespace
 
@@ -1646,10 +1642,10 @@ pic_status pic_conv3x3_bf16(int32_t impl, int32_t B, int32_t H, int32_t W, const
   const bf16 *bin = static_cast<const bf16 *>(in), *bw = static_cast<const bf16 *>(w);
   bf16 *bout = static_cast<bf16 *>(out);
   if (impl == 0) {
-    const ErrWord word;
+    if (!picgb::conv3x3_tc_supported(cin, cout, in_cs, in_off, out_cs, out_off, W)) return PIC_EINVAL;
+    ErrWord word(s);
     int *err = word.device();
     if (!err) return PIC_ECUDA;
-    if (!picgb::conv3x3_tc_supported(cin, cout, in_cs, in_off, out_cs, out_off, W)) return PIC_EINVAL;
     picgb::ConvTC c;
     c.in = bin;
     c.in_cs = in_cs;
@@ -1666,8 +1662,7 @@ pic_status pic_conv3x3_bf16(int32_t impl, int32_t B, int32_t H, int32_t W, const
     c.W = W;
     c.relu = relu ? 1 : 0;
     c.err = err;
-    if (picgb::conv3x3_tc(c, s) != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) return PIC_ECUDA;
-    return word.read("convolution");
+    return word.end(picgb::conv3x3_tc(c, s) == cudaSuccess ? PIC_OK : PIC_ECUDA, "convolution");
   }
   // the mma.sync implicit GEMM: cout 32 (cin 16 or a multiple of 32) or a multiple of 64
   ConvArgs a;
@@ -1715,7 +1710,7 @@ pic_status pic_conv3x3_wgrad_bf16(int32_t impl, int32_t B, int32_t H, int32_t W,
     return PIC_OK;
   }
   if (!picgb::conv_wgrad_tc_supported(cin, cout, in_cs, in_off, dw)) return PIC_EINVAL;
-  const ErrWord word;
+  ErrWord word(s);
   int *err = word.device();
   if (!err) return PIC_ECUDA;
   picgb::WgradTC g;
@@ -1730,8 +1725,7 @@ pic_status pic_conv3x3_wgrad_bf16(int32_t impl, int32_t B, int32_t H, int32_t W,
   g.H = H;
   g.W = W;
   g.err = err;
-  if (picgb::conv_wgrad_tc(g, s) != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) return PIC_ECUDA;
-  return word.read("weight gradient");
+  return word.end(picgb::conv_wgrad_tc(g, s) == cudaSuccess ? PIC_OK : PIC_ECUDA, "weight gradient");
 }
 
 namespace {
@@ -1819,11 +1813,14 @@ pic_status pic_upconv_bf16(int32_t impl, int32_t B, int32_t H, int32_t W, const 
   const int total = 4 * cout, step = total > 256 ? 256 : total;
   if (total % step || cout % 16 || !picgb::conv3x3_tc_supported(cin, step, cin, 0, out_cs, out_off, W))
     return PIC_EINVAL;
-  const ErrWord word;
-  int *err = word.device();
-  if (!err) return PIC_ECUDA;
   bf16 *wt = nullptr;
   if (cudaMalloc(&wt, size_t(total) * cin * 2) != cudaSuccess) return PIC_ENOMEM;
+  ErrWord word(s);
+  int *err = word.device();
+  if (!err) {
+    cudaFree(wt);
+    return PIC_ECUDA;
+  }
   k_upw_to_bf16<<<gridn(4LL * cout * cin), 256, 0, s>>>(w, wt, cin, cout);
   picgb::ConvTC c;
   c.in = bi;
@@ -1843,9 +1840,9 @@ pic_status pic_upconv_bf16(int32_t impl, int32_t B, int32_t H, int32_t W, const 
   c.up_cout = cout;
   pic_status st = cudaGetLastError() == cudaSuccess ? PIC_OK : PIC_ECUDA;
   if (st == PIC_OK && picgb::conv_up_tc(c, s) != cudaSuccess) st = PIC_ECUDA;
-  if (cudaStreamSynchronize(s) != cudaSuccess && st == PIC_OK) st = PIC_ECUDA;
+  st = word.end(st, "convolution");
   cudaFree(wt);
-  return st == PIC_OK ? word.read("convolution") : st;
+  return st;
 }
 
 pic_status pic_upconv_wgrad_bf16(int32_t impl, int32_t B, int32_t H, int32_t W, const void *in, int32_t cin,
@@ -1874,7 +1871,7 @@ pic_status pic_upconv_wgrad_bf16(int32_t impl, int32_t B, int32_t H, int32_t W, 
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return PIC_ECUDA;
-  const ErrWord word;
+  ErrWord word(s);
   int *err = word.device();
   if (!err) return PIC_ECUDA;
   picgb::UpWgradTC g;
@@ -1889,12 +1886,11 @@ pic_status pic_upconv_wgrad_bf16(int32_t impl, int32_t B, int32_t H, int32_t W, 
   g.H = H;
   g.W = W;
   g.err = err;
-  if (picgb::conv_upwgrad_tc(g, s) != cudaSuccess) return PIC_ECUDA;
+  if (picgb::conv_upwgrad_tc(g, s) != cudaSuccess) return word.end(PIC_ECUDA, "weight gradient");
   const long long np = 4LL * B * H * W, ppb = 256 / (cout / 8);
   launch(k_colsum, int(std::min<long long>((np + ppb - 1) / ppb, 8LL * sms)), 256, 0, s, bg, gout_cs, gout_off, cout,
          np, db);
-  if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) return PIC_ECUDA;
-  return word.read("weight gradient");
+  return word.end(cudaGetLastError() == cudaSuccess ? PIC_OK : PIC_ECUDA, "weight gradient");
 }
 
 pic_status pic_upconv_back_bf16(int32_t impl, int32_t B, int32_t H, int32_t W, const void *gout,
@@ -1912,12 +1908,15 @@ pic_status pic_upconv_back_bf16(int32_t impl, int32_t B, int32_t H, int32_t W, c
     return PIC_OK;
   }
   if (!picgb::conv3x3_tc_supported(cout, cin, gout_cs, gout_off, cin, 0, W)) return PIC_EINVAL;
-  const ErrWord word;
-  int *err = word.device();
-  if (!err) return PIC_ECUDA;
   const long long nw = 4LL * cin * cout;
   bf16 *wb = nullptr;
   if (cudaMalloc(&wb, size_t(nw) * 2) != cudaSuccess) return PIC_ENOMEM;
+  ErrWord word(s);
+  int *err = word.device();
+  if (!err) {
+    cudaFree(wb);
+    return PIC_ECUDA;
+  }
   picgb::ConvTC c;
   c.in = bg;
   c.in_cs = gout_cs;
@@ -1935,12 +1934,10 @@ pic_status pic_upconv_back_bf16(int32_t impl, int32_t B, int32_t H, int32_t W, c
   c.relu = 0;
   c.err = err;
   k_to_bf16<<<gridn(nw), 256, 0, s>>>(w, wb, nw);
-  pic_status st = PIC_OK;
-  if (cudaGetLastError() != cudaSuccess || picgb::conv_upback_tc(c, s) != cudaSuccess ||
-      cudaStreamSynchronize(s) != cudaSuccess)
-    st = PIC_ECUDA;
+  const bool launched = cudaGetLastError() == cudaSuccess && picgb::conv_upback_tc(c, s) == cudaSuccess;
+  const pic_status st = word.end(launched ? PIC_OK : PIC_ECUDA, "convolution");
   cudaFree(wb);
-  return st == PIC_OK ? word.read("convolution") : st;
+  return st;
 }
 
 pic_status pic_unet_set_conv_impl(pic_unet *u, int32_t impl) {
