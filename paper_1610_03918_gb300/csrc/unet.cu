@@ -896,6 +896,7 @@ inline int gridn(long long n, int t = 256) {
 // ============================================================================
 struct pic_unet {
   int B, H, W;
+  int dev = 0;
   int num_sms = 1;
   cudaStream_t stream = nullptr;
   std::vector<void *> allocs;
@@ -1368,13 +1369,10 @@ pic_status pic_unet_create(int32_t batch, int32_t height, int32_t width, void *s
   u->H = height;
   u->W = width;
   u->stream = static_cast<cudaStream_t>(stream);
-  {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&u->num_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-      delete u;
-      return PIC_ECUDA;
-    }
+  if (cudaGetDevice(&u->dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&u->num_sms, cudaDevAttrMultiProcessorCount, u->dev) != cudaSuccess) {
+    delete u;
+    return PIC_ECUDA;
   }
   // parameter layout (the order of the layer list)
   long long off = 0;
@@ -1498,7 +1496,17 @@ pic_status pic_unet_get_params(pic_unet *u, float *host) {
 
 pic_status pic_unet_forward(pic_unet *u, const float *x, float *y) {
   if (!u || !x || !y) return PIC_EINVAL;
-  forward(u, x, false, y);
+  // the head stores into the caller's array where that is this device's memory and
+  // its floats are aligned; a copy takes any other
+  cudaPointerAttributes at = {};
+  if (cudaPointerGetAttributes(&at, y) != cudaSuccess) cudaGetLastError();
+  if (reinterpret_cast<uintptr_t>(y) % alignof(float) == 0 && at.type == cudaMemoryTypeDevice && at.device == u->dev) {
+    forward(u, x, false, y);
+  } else {
+    forward(u, x, false);
+    if (cudaMemcpyAsync(y, u->y, size_t(u->B) * u->H * u->W * 4, cudaMemcpyDeviceToDevice, u->stream) != cudaSuccess)
+      return PIC_ECUDA;
+  }
   return cudaGetLastError() == cudaSuccess ? PIC_OK : PIC_ECUDA;
 }
 
