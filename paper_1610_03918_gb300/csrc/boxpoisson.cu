@@ -299,7 +299,7 @@ cudaError_t box_poisson_setup(pic_ctx *c) {
   const Geom &g = c->g;
   if (c->cfg.poisson_method != 0) return cudaSuccess;
   // beside the FFT solve only for the passes its closing kernel may add
-  if (c->fp.enabled && c->g.nxn * c->g.nyn > kTailNodes) return cudaSuccess;
+  if (c->fp.enabled && (c->g.nxn * c->g.nyn > kTailNodes || c->g.nyn > kFftOnceCols)) return cudaSuccess;
   const int nyn = g.nyn, nxn = g.nxn, col0 = g.py ? 0 : 1, n = g.py ? nyn : nyn - 2;
   if (n < 2 || n > kMaxCols) return cudaSuccess;
   auto free_at = [&](int i, int j) { return (c->h_nodeflags[size_t(i) * nyn + j] & kFree) != 0; };

@@ -284,6 +284,19 @@ inline size_t box_solve_smem(const BoxBlock &b) { return (4 * size_t(b.n) + 2 * 
 // node's cost beyond what all of them take (384 x 384: the same step time, 512 x
 // 512: 123 -> 131 us).
 constexpr int kTailNodes = 81920;
+// On a grid of the FFT solve the cluster's further passes are transforms by a dense
+// basis on 16 SMs, where a conditional node would run the FFT kernels on all of them.
+// With one pass a step the cluster gains on every such grid (128 x 64: 57 -> 35 us a step,
+// 312 x 256: 67 -> 55, 72 x 1024: 80 -> 64), with two only on the smaller ones (640 x 32: 87
+// -> 67, 128 x 64: 80 -> 64, 160 x 128: 88 -> 88; but 1248 x 64: 105 -> 134, 312 x 256: 99
+// -> 196, 72 x 1024: 118 -> 522).  So the FFT grids have it up to kFftTailNodes nodes and
+// kFftTailCols columns, and beyond where a second pass is rare: up to kFftOnceRows rows
+// and kFftOnceCols columns, a tolerance of kFftOnceRtol or more and a guess from the
+// steps before (passes a step on 320 rows: 1.00 to 1.08 from the potential of the step
+// before, 2.00 from 0; on 640 rows up to 1.42; on 1248 up to 1.77).
+constexpr int kFftTailNodes = 21504, kFftTailCols = 128;
+constexpr int kFftOnceRows = 320, kFftOnceCols = 256;
+constexpr double kFftOnceRtol = 1e-6;
 // launch arguments for a context's transform solve of A e = r (its tables set up)
 BoxArgs box_args(pic_ctx *c, const float *r, float2 *pot, PoissonState *ps);
 

@@ -2276,7 +2276,12 @@ static void launch_first_pass(pic_ctx *c, const FineArgs &a, bool bb_later) {
 }
 
 
-bool closing_cluster(const pic_ctx *c) { return c->box.tail != 0; }
+bool closing_cluster(const pic_ctx *c) {
+  if (!c->box.tail || !c->fp.enabled) return c->box.tail != 0;
+  const int rows = c->box.b[0].m, cols = c->box.b[0].n, ws = c->cfg.warm_start;
+  return (c->g.nxn * c->g.nyn <= kFftTailNodes && cols <= kFftTailCols) ||
+         (rows <= kFftOnceRows && cols <= kFftOnceCols && c->cfg.poisson_rtol >= kFftOnceRtol && (ws == 1 || ws == 2));
+}
 
 // The solve of a grid whose closing cluster checks and repeats by itself, into
 // the capture in progress:
