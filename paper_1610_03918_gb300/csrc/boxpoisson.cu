@@ -43,6 +43,19 @@ constexpr int kMaxCols = 1024;         // columns of the basis (V is n x n)
 constexpr int kMaxRows = 4096;
 constexpr int kMaxSlot = 512;          // interface columns (their Schur complement is inverted on the host)
 
+// Multiply-adds of a transform (rows x columns^2) above which multigrid is the faster
+// one.  A pass here grows with that product, a V-cycle with the nodes; one, two and
+// three passes stand against 5, 7 to 9 and 10 to 12 V-cycles at tolerances of 1e-6, 1e-8
+// to 1e-10 and 1e-12, two against 6 at 1e-6 from a guess of 0.  Four walls, us a step
+// here : there at 1e-6, 1e-8, 1e-12 and from 0: 1024 x 1024 553 : 779, 908 : 1018, 1258 :
+// 1385, 917 : 919; 2048 x 1024 1044 : 1153, 1675 : 1485, 2328 : 2094, 1669 : 1354.  A
+// coarsest level of more than 160 unknowns is swept in one CTA, 0.06 us a node and
+// V-cycle: the line rises with it.  Doubly periodic boxes' V-cycles take longer (1024 x
+// 1024 539 : 817, 869 : 1055, 1190 : 1423, 871 : 964; 2048 x 1024 979 : 1238, 1573 : 1588,
+// 2170 : 2194, 1581 : 1447); with such a coarsest level multigrid is slow on any box
+// periodic in y (4096 x 960 between plates 1427 : 4970).
+constexpr double kMaxWorkWalls = 1.1e9, kMaxWorkCoarsest = 1.2e6, kMaxWorkPeriodic = 1.7e9;
+
 int pad4(int n) { return (n + 3) & ~3; }
 int pad8(int n) { return (n + 7) & ~7; }
 
@@ -308,6 +321,12 @@ cudaError_t box_poisson_setup(pic_ctx *c) {
     for (int j = 0; j < nyn; ++j) q += free_at(i, j);
     return q;
   };
+  auto too_large = [&](int m) {
+    const MGLevel &L = c->lev.back();
+    return double(m) * n * n > (!g.py           ? kMaxWorkWalls + kMaxWorkCoarsest * L.nxn * L.nyn
+                                : c->ncoarse > 0 ? kMaxWorkPeriodic
+                                                 : HUGE_VAL);
+  };
   BoxBlock &R = p.b[0], &S = p.b[1];
   R.col0 = col0;
   R.n = n;
@@ -317,6 +336,7 @@ cudaError_t box_poisson_setup(pic_ctx *c) {
     if (nxn < 3 || nxn > kMaxRows) return cudaSuccess;
     for (int i = 0; i < nxn; ++i)
       if (row_count(i) != n) return cudaSuccess;
+    if (too_large(nxn)) return cudaSuccess;
     R.row0 = 0;
     R.m = nxn;
     if ((e = build_block(c, R, g.py != 0, -1, true, tr)) != cudaSuccess) return e;
@@ -325,7 +345,7 @@ cudaError_t box_poisson_setup(pic_ctx *c) {
     int xs = 1;
     while (xs < nxn - 1 && row_count(xs) == n) ++xs;
     const int m = xs - 1;
-    if (m < 1 || m > kMaxRows) return cudaSuccess;
+    if (m < 1 || m > kMaxRows || too_large(m)) return cudaSuccess;
     bool slot = false;
     for (int r = xs; r < nxn; ++r) slot = slot || row_count(r) > 0;
     int first = -1, last = -1, ms = 0;
