@@ -284,8 +284,12 @@ inline size_t box_solve_smem(const BoxBlock &b) { return (4 * size_t(b.n) + 2 * 
 // node's cost beyond what all of them take (384 x 384: the same step time, 512 x
 // 512: 123 -> 131 us).
 constexpr int kTailNodes = 81920;
-// On a grid of the FFT solve the cluster's further passes are transforms by a dense
-// basis on 16 SMs, where a conditional node would run the FFT kernels on all of them.
+// Its further passes are transforms by a dense basis on 16 SMs, which grow with the
+// columns squared.  Two passes a step against multigrid (1e-8): 128 x 512 between walls
+// 237 against 494 us, 64 x 1024 547 against 483 (1e-6 from a guess of 0: 547 against 428);
+// so a box of more than kTailCols columns repeats its two kernels on all SMs under the node.
+constexpr int kTailCols = 512;
+// On a grid of the FFT solve a conditional node runs the FFT kernels on all SMs instead.
 // With one pass a step the cluster gains on every such grid (128 x 64: 57 -> 35 us a step,
 // 312 x 256: 67 -> 55, 72 x 1024: 80 -> 64), with two only on the smaller ones (640 x 32: 87
 // -> 67, 128 x 64: 80 -> 64, 160 x 128: 88 -> 88; but 1248 x 64: 105 -> 134, 312 x 256: 99

@@ -2032,7 +2032,7 @@ constexpr int kTailCtas = 16;
 cudaError_t box_tail_setup(pic_ctx *c) {
   BoxPoisson &p = c->box;
   const int nn = c->g.nxn * c->g.nyn;
-  p.tail = nn <= kTailNodes ? 1 : 0;
+  p.tail = nn <= kTailNodes && p.b[0].n <= kTailCols ? 1 : 0;
   if (!p.tail) return cudaSuccess;
   p.tail_smem = std::max(p.solve_smem, size_t(p.b[0].n) * 8 * sizeof(float));
   if (p.slot) p.tail_smem = std::max(p.tail_smem, size_t(p.b[1].n) * 8 * sizeof(float));
