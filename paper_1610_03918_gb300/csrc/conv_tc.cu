@@ -2103,6 +2103,12 @@ cudaError_t launch_up_kb(const ConvTC &c, cudaStream_t s, int sms) {
     }
   }
   if (!best) return cudaErrorNotSupported;
+  // Four column blocks of 64 each load all of the pixels; with few units beside the
+  // weights, on many tiles, that costs more than one pass of the tile kernel (a call
+  // with 256 channels from 256 at 1032 tiles 231 us against 223, at 774 203 against 210;
+  // from 320 at 400 tiles 178 against 174, at 1032 279 against 243; from 192 never).
+  if (MODE == kUpBack && c.cout / best >= 4 && tiles * (a.units * KB / 64 - 12) > 20LL * sms)
+    return cudaErrorNotSupported;
   CUtensorMap ta;
   const cuuint32_t one[5] = {1, 1, 1, 1, 1};
   const cuuint64_t e = 2, cs = c.in_cs;   // bytes per element
