@@ -357,14 +357,15 @@ const char *pic_last_error(void);
  * Sec. III-C run as a batch).  Each member is a full context built from
  * cfgs[k] (its own grid size, trench, particles and tallies); all members
  * share one CUDA stream (`stream`, or a library-owned one when NULL) and one
- * tile-sort schedule (equal sort_every, else PIC_EINVAL).  The members form up
- * to eight groups of about equal particle counts, each stepped on a stream of its
- * own, after what `stream` holds at the call, and `stream` waits for all of them at
- * the call's last step (at every step with cfgs[0].timing).  A group's step is one
- * launch of a captured CUDA graph in which every member's step (sort when due,
- * particle kernel, rho, Poisson solve with its own device-side convergence loop,
- * field) is an independent branch, so the members' phases overlap on the GPU and no
- * group waits for another's solves.  Load and read members with pic_load / pic_diag on
+ * tile-sort schedule (equal sort_every, else PIC_EINVAL).  In calls of four steps
+ * and more (two with 16 members, one with 24) the members form up to eight groups of
+ * about equal particle counts, each stepped on a stream of its own, after what `stream`
+ * holds at the call, and `stream` waits for all of them at the call's last step; in
+ * shorter calls, and with cfgs[0].timing, all members form one group on `stream`.  A
+ * group's step is one launch of a captured CUDA graph in which every member's step
+ * (sort when due, particle kernel, rho, Poisson solve with its own device-side
+ * convergence loop, field) is an independent branch, so the members' phases overlap on
+ * the GPU and no group waits for another's solves.  Load and read members with pic_load / pic_diag on
  * pic_batch_member(b, k); advance them only through pic_batch_step. */
 typedef struct pic_batch pic_batch;
 
@@ -380,7 +381,7 @@ pic_ctx *pic_batch_member(pic_batch *b, int32_t k);
 pic_status pic_batch_step(pic_batch *b, int32_t nsteps);
 
 /* out[0] = ensemble steps and out[1] = their device milliseconds (CUDA
- * events around all groups' launches of a step) since the last call. */
+ * events around the launch of a step) since the last call. */
 pic_status pic_batch_timing(pic_batch *b, double *out);
 
 /* Release the batch and all its members. */

@@ -568,9 +568,9 @@ def exchange_sum(sims):
 
 
 class Batch:
-    """An ensemble of independent runs advanced together: captured CUDA graphs,
-    one for each of up to eight groups of members, with every member's step as a
-    parallel branch.
+    """An ensemble of independent runs advanced together: captured CUDA graphs, one
+    for each of up to eight groups of members (one for all of them in calls of few
+    steps and with timing), with every member's step as a parallel branch.
     ``members[k]`` is a Sim view of member k for loading and diagnostics."""
 
     def __init__(self, workloads, capacities=None, device: int = 0, timing: bool = False,

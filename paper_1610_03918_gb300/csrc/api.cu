@@ -542,7 +542,8 @@ struct pic_batch {
     cudaGraphExec_t gexec[2] = {nullptr, nullptr};
   };
   std::vector<Group> groups;
-  cudaEvent_t ev[2] = {nullptr, nullptr};   // the groups' start on the batch's stream, their end
+  Group whole;                              // all members, on the batch's stream
+  cudaEvent_t ev[2] = {nullptr, nullptr};   // a step's start on the batch's stream, its end
   double t_ms = 0.0;
   int64_t t_steps = 0;
 };
@@ -551,6 +552,13 @@ struct pic_batch {
 // graph per ensemble step every member waited for the slowest one's solve, some
 // 50 us a step with little else running (eight members of the width sweep).
 constexpr int kMaxGroups = 8;
+// Calls of fewer steps, and timed ones, which wait after every step, launch one graph of
+// all members: starting and joining the groups' streams costs a call 15 to 40 us (8
+// members of 4 particles a cell 193 us a step in calls of one against 163, but 149 in
+// calls of 16; timed ones of 16 members 347 against 317).  Its branches run from the
+// smallest member to the largest (50 members 852 us, in the caller's order 938).  With
+// many members the groups are worth it from 2 steps and at last from 1 (50 members 835).
+static int group_steps(size_t members) { return members < 2 * kMaxGroups ? 4 : members < 3 * kMaxGroups ? 2 : 1; }
 
 namespace picgb {
 namespace {
@@ -644,6 +652,8 @@ pic_status pic_batch_init(const pic_config *cfgs, int32_t n, void *stream, pic_b
   });
   const int ng = std::min<int>(n, kMaxGroups);
   b->groups.resize(ng);
+  b->whole.m.assign(order.rbegin(), order.rend());
+  b->whole.stream = b->stream;
   for (int k = 0; k < n; ++k) {
     const int r = k % (2 * ng);
     b->groups[r < ng ? r : 2 * ng - 1 - r].m.push_back(order[k]);
@@ -677,6 +687,7 @@ pic_status pic_batch_step(pic_batch *b, int32_t nsteps) {
     b->steps_since_sort = 0;
     for (pic_ctx *c : b->m) c->steps_since_sort = 0;
   }
+  const bool joined = b->timing || nsteps < group_steps(b->m.size());
   pic_status st = PIC_OK;
   for (int32_t k = 0; k < nsteps && st == PIC_OK; ++k) {
     int sorting = b->steps_since_sort >= b->sort_every ? 1 : 0;
@@ -684,16 +695,24 @@ pic_status pic_batch_step(pic_batch *b, int32_t nsteps) {
       if (c->needs_sort) sorting = 1;
       c->needs_sort = 0;
     }
-    for (auto &q : b->groups)
-      if (check(group_graph(q, sorting)) != PIC_OK) st = PIC_ECUDA;
-    if (st == PIC_OK && (k == 0 || b->timing)) st = groups_fork(b);
-    for (auto &q : b->groups)
-      if (st == PIC_OK && note(cudaGraphLaunch(q.gexec[sorting], q.stream), "ensemble graph launch") != cudaSuccess)
+    if (joined) {
+      if (check(group_graph(b->whole, sorting)) != PIC_OK) st = PIC_ECUDA;
+      if (st == PIC_OK && (note(cudaEventRecord(b->ev[0], b->stream), "ensemble start") != cudaSuccess ||
+                           note(cudaGraphLaunch(b->whole.gexec[sorting], b->stream), "ensemble graph launch") != cudaSuccess ||
+                           note(cudaEventRecord(b->ev[1], b->stream), "ensemble end") != cudaSuccess))
         st = PIC_ECUDA;
-    // (also after a failure: what was launched ends before later work of the batch's stream)
-    if (k + 1 == nsteps || b->timing || st != PIC_OK) {
-      const pic_status sj = groups_join(b);
-      if (st == PIC_OK) st = sj;
+    } else {
+      for (auto &q : b->groups)
+        if (check(group_graph(q, sorting)) != PIC_OK) st = PIC_ECUDA;
+      if (st == PIC_OK && k == 0) st = groups_fork(b);
+      for (auto &q : b->groups)
+        if (st == PIC_OK && note(cudaGraphLaunch(q.gexec[sorting], q.stream), "ensemble graph launch") != cudaSuccess)
+          st = PIC_ECUDA;
+      // (also after a failure: what was launched ends before later work of the batch's stream)
+      if (k + 1 == nsteps || st != PIC_OK) {
+        const pic_status sj = groups_join(b);
+        if (st == PIC_OK) st = sj;
+      }
     }
     if (st != PIC_OK) break;
     for (pic_ctx *c : b->m) {
@@ -734,6 +753,8 @@ pic_status pic_batch_free(pic_batch *b) {
   for (auto &q : b->groups)
     if (q.stream) cudaStreamSynchronize(q.stream);
   if (b->stream) cudaStreamSynchronize(b->stream);
+  b->whole.stream = nullptr;   // the batch's
+  b->groups.push_back(b->whole);
   for (auto &q : b->groups) {
     for (int k = 0; k < 2; ++k) {
       if (q.gexec[k]) cudaGraphExecDestroy(q.gexec[k]);
