@@ -39,11 +39,10 @@ BYTES_PER_PARTICLE_STEP = 40
 # capture (dram__bytes_read.sum + dram__bytes_write.sum over the launch),
 # valid for the kernel source whose hash is recorded with it.
 NCU_TRAFFIC = {
-    # k_particles<0, 0, true>, 512x1024 trench at 40 ppc (33.91M particles, 0.8 GB
-    # of state, larger than L2, chunks in parts as at 100 ppc), launches 3 and 4:
-    # 694.5 MB read + 626.3 / 622.9 MB written
-    "source_sha256": "4a4e9716966d035f1260111005724054abc81cd0390e64e01fe9a6d0b0f25fa6",
-    "bytes_per_particle": 38.9,
+    # k_particles<0, 0>, 512x1024 trench at 20 ppc (16.96M particles, 0.4 GB of state,
+    # larger than L2), launches 3 and 4: 353.3 MB read + 285.8 MB written
+    "source_sha256": "ac85b62f19ab2e7b446a96c37b7a3995d7a625dacd161eecd5488b7a2e08555e",
+    "bytes_per_particle": 37.7,
 }
 
 
@@ -976,7 +975,9 @@ def main():
                        "warmup_steps_run": warm, "poisson_rtol": w.poisson_rtol,
                        "warm_start": {0: "zero", 1: "previous", 2: "extrapolated",
                                       4: "lift"}[args.warm_start],
-                       "poisson_inner_solver": "direct" if sim.solver() == pg.POISSON_AUTO else "multigrid PCG",
+                       "poisson_inner_solver": ("direct" if sim.solver() == pg.POISSON_AUTO else
+                                                "multigrid PCG" if args.poisson_method == "multigrid" else
+                                                "dense transforms where the box allows them, else multigrid PCG"),
                        "l2": "inputs larger than L2 (particle state %.1f GB)" % (n0 * 24 / 1e9),
                        "timing": "value: the timed steps run without phase events; phases and the "
                                  "roofline's kernel time: CUDA events between the phases over a "

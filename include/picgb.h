@@ -124,8 +124,9 @@ typedef struct {
                                      slab with at most one slot below it (the trench and the
                                      plate geometries); else, for such a slab and slot on up to
                                      1024 columns of any count, periodic or between two walls, or
-                                     with x periodic, a solve by dense transforms along y; else
-                                     as 1;
+                                     with x periodic, a solve by dense transforms along y, but
+                                     for large boxes (rows x columns^2 from 1.1e9 on) that
+                                     multigrid coarsens well; else as 1;
                                      1: conjugate gradient preconditioned by a multigrid V-cycle */
   int64_t hit_capacity;           /* hit records kept (PIC_DIAG_HITS) */
   void *stream;                   /* cudaStream_t to run on; NULL: a library-owned stream */

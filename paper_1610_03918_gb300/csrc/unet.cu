@@ -1987,8 +1987,8 @@ int unet_height(const pic_unet *u) { return u->H; }
 int unet_width(const pic_unet *u) { return u->W; }
 int unet_batch(const pic_unet *u) { return u->B; }
 // kernels one forward launches: 14 convolutions (the first one from the FP32
-// input), 3 transposed convolutions, the head, and the pools that no convolution's
-// epilogue takes
+// input), 3 transposed convolutions (a launch each with this network's channels), the
+// head, and the pools that no convolution's epilogue takes
 int unet_forward_kernels(const pic_unet *u) {
   int pools = 0;
   for (int l = 0; l < 3; ++l)
