@@ -717,6 +717,8 @@ cudaError_t fast_poisson_setup(pic_ctx *c) {
                                        int(kSmemMax));
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_fp_interface, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSmemMax));
+  if (e == cudaSuccess)   // (a slot's basis of 110 columns and more)
+    e = cudaFuncSetAttribute(k_fp_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSmemMax));
   if (e != cudaSuccess) return e;
   p.enabled = 1;
   return cudaGetLastError();
@@ -725,7 +727,7 @@ cudaError_t fast_poisson_setup(pic_ctx *c) {
 void fast_poisson_launch(pic_ctx *c, const float *r, float2 *pot, PoissonState *ps) {
   const FPArgs a = fp_args(c, r, pot, ps);
   const int rows = (a.m + 1) / 2;
-  launch(k_fp_forward, rows, kFftThreads, fft_smem_bytes(a.ny, a.wc), c->stream, a);
+  launch(k_fp_forward, rows, kFftThreads, fft_smem_bytes(a.ny, 0), c->stream, a);
   launch(k_fp_tridiag, a.nk + (a.slot ? a.wc : 0), kPcrThreads,
          tridiag_smem_bytes(a.m, a.slot ? a.ms : 0, a.wc), c->stream, a);
   if (a.slot) launch(k_fp_interface, 1, kSlotThreads, slot_smem_bytes(a.wc), c->stream, a);

@@ -2162,12 +2162,18 @@ pic_status poisson_solve(pic_ctx *c, bool zero_guess) {
   launch(k_outer_init, 1, 1, 0, c->stream, c->d_ps);
   c->launches += 1;
   const int batch = 4;
+  int passes = 0;
   for (;;) {
     launch(resid_kernel<kFull>(c), nb, kThreads, 0, c->stream, a);
     c->launches += 1;
     cudaMemcpyAsync(c->h_ps, c->d_ps, sizeof(PoissonState), cudaMemcpyDeviceToHost, c->stream);
     if (cudaStreamSynchronize(c->stream) != cudaSuccess) return PIC_ECUDA;
     if (!c->h_ps->go) break;
+    // a pass whose launch failed is not counted on the device, which then asks for another
+    if (++passes > kMaxOuter) {
+      note(cudaGetLastError(), "Poisson solve");
+      return PIC_ECUDA;
+    }
     if (one_pass_solver(c)) {   // adds its correction to phi itself
       launch_one_pass(c);
       continue;
