@@ -695,7 +695,9 @@ __global__ void __launch_bounds__(256) k_colsum(const bf16 *g, int g_cs, int g_o
   float s[8];
 #pragma unroll
   for (int k = 0; k < 8; ++k) s[k] = 0.f;
-  for (long long p = blockIdx.x * (long long)ppb + threadIdx.x / G; p < npix; p += (long long)gridDim.x * ppb) {
+  // (threads beyond the CTA's whole pixels, with 192 channels 16 of them, take none)
+  const long long p0 = int(threadIdx.x) < ppb * G ? blockIdx.x * (long long)ppb + threadIdx.x / G : npix;
+  for (long long p = p0; p < npix; p += (long long)gridDim.x * ppb) {
     const uint4 v = *reinterpret_cast<const uint4 *>(g + p * g_cs + g_off + 8 * grp);
     const bf16 *vv = reinterpret_cast<const bf16 *>(&v);
 #pragma unroll
